@@ -2,9 +2,11 @@
 // >= l_x (the paper matches tree-node size to the linking length for the
 // neighbour search, Sec. 3.1; here the tree is a uniform periodic grid).
 //
-//   bin_count    validate every coordinate, histogram of bricks
+//   bin_count    validate every coordinate, histogram of bricks, and each
+//                particle's rank in its brick (what the count's atomic returns)
 //   scan         exclusive prefix sum of the brick counts
-//   bin_scatter  each particle to its brick (float4: x, y, z, local index)
+//   bin_scatter  each particle to its brick's start + rank (float4: x, y, z,
+//                local index)
 //   brick_sort   one CTA per brick: cell histogram and scan in shared
 //                memory, scatter into cell order, cell_start of the brick,
 //                and the forest initialisation parent[s] = s (Sec. 3.1)
@@ -43,68 +45,166 @@ __device__ __forceinline__ int64_t brick_of(const float* __restrict__ pos, int64
     return b.brick0 + brick_local(b, cell_coord(x, b), cell_coord(y, b), cell_coord(z, b));
 }
 
-__global__ void __launch_bounds__(256) k_bin_count(const float* __restrict__ pos, Geometry g,
-                                                   int* __restrict__ bcount, int* __restrict__ err)
+// One tile of particles per CTA in both kernels, not a stride over the input.
+// CTAs start in order, so particles of neighbouring rank are stored at about
+// the same time and a brick's sectors fill up while they are in L2; CTAs that
+// stride over the input drift apart, and half-filled sectors leave L2 (768^3
+// box, scatter by the count's ranks: 11.8 ms striding, 6.5 ms by tiles; 7.9 ms
+// with a cursor atomic per particle instead).  The tiles of kBinStreams evenly spaced places of the input
+// take turns: inputs list a blob's particles one after the other, and tiles of
+// one place alone would all count into that blob's few bricks (a batch of 512
+// boxes: count 8.1 ms in input order, 2.5 ms with 64 places).
+//
+// The particle's rank in its brick (what the count's atomic returns) goes to
+// rank[i], so that the scatter needs no atomic.  The counters lie `pad` words
+// apart (brick_pad).
+constexpr int kBinThreads = 256;
+constexpr int kBinItems = 4;
+constexpr int kBinTile = kBinThreads * kBinItems;
+constexpr int kBinStreams = 64;
+
+__host__ __device__ __forceinline__ int64_t bin_tiles_per_stream(int64_t n, int streams)
+{
+    return ((n + kBinTile - 1) / kBinTile + streams - 1) / streams;
+}
+
+// First particle of this CTA's tile (may lie past the end).
+__device__ __forceinline__ int64_t bin_tile_base(int64_t n, int streams)
+{
+    return ((int64_t)(blockIdx.x % streams) * bin_tiles_per_stream(n, streams) + blockIdx.x / streams) * kBinTile;
+}
+
+__global__ void __launch_bounds__(kBinThreads) k_bin_count(const float* __restrict__ pos, Geometry g,
+                                                           int* __restrict__ bcount, int pad,
+                                                           int* __restrict__ rank, int streams,
+                                                           int* __restrict__ err)
 {
     const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t base = bin_tile_base(g.total_n, streams) + threadIdx.x;
     int bad = 0;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < g.total_n; base += stride) {
-        int64_t i = base + threadIdx.x;
-        bool valid = i < g.total_n;
-        unsigned active = __ballot_sync(kFull, valid);
-        if (!valid)
-            continue;
-        const BoxDev& b = g.boxes[box_of(g.box_p0, g.nbox, i)];
-        float4 rec;
-        bool ok;
-        int64_t brick = brick_of(pos, i, b, rec, ok);
-        bad |= !ok;
-        // brick indices fit in 31 bits (checked when the plan is made); the
-        // 32-bit match is much cheaper than the 64-bit one
-        unsigned peers = __match_any_sync(active, (int)brick);
-        int leader = __ffs(peers) - 1;
-        if (lane == leader)
-            atomicAdd(bcount + brick, __popc(peers));
+    int brick[kBinItems], off[kBinItems];
+    unsigned peers[kBinItems];
+#pragma unroll
+    for (int k = 0; k < kBinItems; ++k) {
+        const int64_t i = base + k * kBinThreads;
+        brick[k] = -1;
+        if (i < g.total_n) {
+            const BoxDev& b = g.boxes[box_of(g.box_p0, g.nbox, i)];
+            float4 rec;
+            bool ok;
+            brick[k] = (int)brick_of(pos, i, b, rec, ok);   // fits in 31 bits (checked when the plan is made)
+            bad |= !ok;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < kBinItems; ++k) {
+        peers[k] = __match_any_sync(kFull, brick[k]);
+        off[k] = 0;
+        if (lane == __ffs(peers[k]) - 1 && brick[k] >= 0)
+            off[k] = atomicAdd(bcount + (int64_t)brick[k] * pad, __popc(peers[k]));
+    }
+#pragma unroll
+    for (int k = 0; k < kBinItems; ++k) {
+        const int first = __shfl_sync(kFull, off[k], __ffs(peers[k]) - 1);
+        if (brick[k] >= 0)
+            rank[base + k * kBinThreads] = first + __popc(peers[k] & lanemask_lt());
     }
     if (__syncthreads_or(bad) && threadIdx.x == 0)
         atomicOr(err, kErrRange);
 }
 
-__global__ void __launch_bounds__(256) k_bin_scatter(const float* __restrict__ pos, Geometry g,
-                                                     const int* __restrict__ bstart,
-                                                     int* __restrict__ bcursor,
-                                                     float4* __restrict__ tmp, int* __restrict__ err)
+// The same where all brick counters fit in shared memory: a CTA counts a tile
+// of particles there and adds each brick's count to the global counter once.
+// Few bricks mean many particles per counter: without the tile, every
+// particle of a large blob in random order is an atomic on one address (about
+// 1.7 ns each; 2 million particles in random order, one atomic each: 158 us,
+// through the tile 30 us).
+constexpr int kCountThreads = 1024;
+
+template <int kItems>
+__global__ void __launch_bounds__(kCountThreads) k_bin_count_tile(const float* __restrict__ pos, Geometry g,
+                                                                  int* __restrict__ bcount, int pad,
+                                                                  int* __restrict__ rank, int* __restrict__ err)
 {
+    extern __shared__ int tile_count[];                  // [total_bricks]: the tile's count, then its first rank
     const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < g.total_n; base += stride) {
-        int64_t i = base + threadIdx.x;
-        bool valid = i < g.total_n;
-        unsigned active = __ballot_sync(kFull, valid);
-        if (!valid)
-            continue;
-        const BoxDev& b = g.boxes[box_of(g.box_p0, g.nbox, i)];
-        float4 rec;
-        bool ok;
-        int64_t brick = brick_of(pos, i, b, rec, ok);
-        unsigned peers = __match_any_sync(active, (int)brick);
-        int leader = __ffs(peers) - 1;
-        int rank = __popc(peers & lanemask_lt());
+    const int nb = (int)g.total_bricks;
+    const int64_t base = (int64_t)blockIdx.x * (kItems * kCountThreads) + threadIdx.x;
+    int brick[kItems], local[kItems];
+    int bad = 0;
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
+        const int64_t i = base + k * kCountThreads;
+        brick[k] = -1;
+        if (i < g.total_n) {
+            const BoxDev& b = g.boxes[box_of(g.box_p0, g.nbox, i)];
+            float4 rec;
+            bool ok;
+            brick[k] = (int)brick_of(pos, i, b, rec, ok);
+            bad |= !ok;
+        }
+    }
+    for (int b = threadIdx.x; b < nb; b += kCountThreads) tile_count[b] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
+        const unsigned peers = __match_any_sync(kFull, brick[k]);
+        const int leader = __ffs(peers) - 1;
         int off = 0;
-        if (lane == leader)
-            off = atomicAdd(bcursor + brick, __popc(peers));
-        off = __shfl_sync(active, off, leader);
-        int64_t slot = (int64_t)__ldg(bstart + brick) + off + rank;
-        if (slot < __ldg(bstart + brick + 1))
-            tmp[slot] = rec;
+        if (lane == leader && brick[k] >= 0)
+            off = atomicAdd(tile_count + brick[k], __popc(peers));
+        local[k] = __shfl_sync(kFull, off, leader) + __popc(peers & lanemask_lt());
+    }
+    __syncthreads();
+    for (int b = threadIdx.x; b < nb; b += kCountThreads) {
+        const int c = tile_count[b];
+        if (c)
+            tile_count[b] = atomicAdd(bcount + (int64_t)b * pad, c);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kItems; ++k)
+        if (brick[k] >= 0)
+            rank[base + k * kCountThreads] = tile_count[brick[k]] + local[k];
+    if (__syncthreads_or(bad) && threadIdx.x == 0)
+        atomicOr(err, kErrRange);
+}
+
+__global__ void __launch_bounds__(kBinThreads) k_bin_scatter(const float* __restrict__ pos, Geometry g,
+                                                             const int* __restrict__ bstart,
+                                                             const int* __restrict__ rank, int streams,
+                                                             float4* __restrict__ tmp, int* __restrict__ err)
+{
+    const int64_t base = bin_tile_base(g.total_n, streams) + threadIdx.x;
+    float4 rec[kBinItems];
+    int64_t brick[kBinItems];
+    int r[kBinItems];
+#pragma unroll
+    for (int k = 0; k < kBinItems; ++k) {
+        const int64_t i = base + k * kBinThreads;
+        brick[k] = -1;
+        if (i < g.total_n) {
+            const BoxDev& b = g.boxes[box_of(g.box_p0, g.nbox, i)];
+            bool ok;
+            r[k] = rank[i];
+            brick[k] = brick_of(pos, i, b, rec[k], ok);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < kBinItems; ++k) {
+        if (brick[k] < 0)
+            continue;
+        const int64_t slot = (int64_t)__ldg(bstart + brick[k]) + r[k];
+        if (slot < __ldg(bstart + brick[k] + 1))
+            tmp[slot] = rec[k];
         else
             atomicOr(err, kErrInternal);
     }
 }
 
 // ------------------------------------------------------------------------
-// device-wide exclusive scan (reduce, scan of partials, apply)
+// device-wide exclusive scan of the brick counts, in one pass over the tiles
+// (decoupled look-back)
 // ------------------------------------------------------------------------
 
 constexpr int kScanThreads = 256;
@@ -166,55 +266,40 @@ __device__ __forceinline__ unsigned long long block_exclusive_scan64(unsigned lo
     return warp_off + x - v;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const int* __restrict__ in, int64_t len,
-                                                              int* __restrict__ part)
-{
-    __shared__ int sw[32];
-    int64_t base = (int64_t)blockIdx.x * kScanTile;
-    int s = 0;
-    for (int k = 0; k < kScanItems; ++k) {
-        int64_t i = base + (int64_t)k * kScanThreads + threadIdx.x;
-        if (i < len) s += in[i];
-    }
-    int total;
-    block_exclusive_scan(s, sw, total);
-    if (threadIdx.x == 0) part[blockIdx.x] = total;
-}
-
-// single block, exclusive scan of part[0..m) in place, m arbitrary
-__global__ void __launch_bounds__(1024) k_scan_partials(int* __restrict__ part, int64_t m)
-{
-    __shared__ int sw[32];
-    int carry = 0;
-    for (int64_t base = 0; base < m; base += blockDim.x) {
-        int64_t i = base + threadIdx.x;
-        int v = i < m ? part[i] : 0;
-        int total;
-        int ex = block_exclusive_scan(v, sw, total);
-        if (i < m) part[i] = carry + ex;
-        carry += total;
-    }
-}
-
 // out[i] for i in [0, len]: out[len] is the grand total (a virtual zero is
-// appended to the input, so the scan covers len + 1 entries)
-__global__ void __launch_bounds__(kScanThreads) k_scan_apply(const int* __restrict__ in, int* __restrict__ out,
-                                                             int64_t len, const int* __restrict__ part)
+// appended to the input, so the scan covers len + 1 entries).  The counts lie
+// `pad` words apart.
+__global__ void __launch_bounds__(kScanThreads) k_scan(const int* __restrict__ in, int pad, int* __restrict__ out,
+                                                       int64_t len, unsigned long long* __restrict__ state,
+                                                       int* __restrict__ ticket, int* __restrict__ err)
 {
     __shared__ int sw[32];
-    int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
+    __shared__ int s_tile, s_before;
+    if (threadIdx.x == 0)
+        s_tile = atomicAdd(ticket, 1);
+    __syncthreads();
+    const int tile = s_tile;
+    const int64_t base = (int64_t)tile * kScanTile + (int64_t)threadIdx.x * kScanItems;
     int v[kScanItems];
     int s = 0;
-    for (int k = 0; k < kScanItems; ++k) {
-        int64_t i = base + k;
-        v[k] = i < len ? in[i] : 0;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k)
+        v[k] = base + k < len ? in[(base + k) * pad] : 0;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k)
         s += v[k];
-    }
     int total;
-    int ex = block_exclusive_scan(s, sw, total) + part[blockIdx.x];
+    int ex = block_exclusive_scan(s, sw, total);
+    if (threadIdx.x < kWarp) {
+        const int before = lookback(state, tile, total, threadIdx.x, err);
+        if (threadIdx.x == 0)
+            s_before = before;
+    }
+    __syncthreads();
+    ex += s_before;
+#pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
-        int64_t i = base + k;
-        if (i <= len) out[i] = ex;
+        if (base + k <= len) out[base + k] = ex;
         ex += v[k];
     }
 }
@@ -420,27 +505,51 @@ static int grid_for(int64_t items, int threads, int per_sm)
     return (int)(want < cap ? want : cap);
 }
 
+// Words between brick counters: L2 serialises atomics on one 128-byte line
+// (about 1.7 ns each), so counters that many particles share get a line or a
+// sector of their own while that costs at most 4 MB.
+int brick_pad(int64_t bricks)
+{
+    return bricks <= kTileBricks ? 32 : (bricks <= 131072 ? 8 : 1);
+}
+
+template <int kItems>
+static cudaError_t run_count_tile(const float* pos, const Geometry& g, const Work& w, cudaStream_t s)
+{
+    const int64_t tile = (int64_t)kItems * kCountThreads;
+    k_bin_count_tile<kItems><<<(unsigned)((g.total_n + tile - 1) / tile), kCountThreads,
+                               sizeof(int) * (size_t)g.total_bricks, s>>>(
+        pos, g, w.bcount, brick_pad(g.total_bricks), w.parent, &w.status->err);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_bin_count(const float* pos, const Geometry& g, const Work& w, cudaStream_t s)
 {
     if (g.total_n == 0)
         return cudaSuccess;
-    k_bin_count<<<grid_for(g.total_n, 256, 8), 256, 0, s>>>(pos, g, w.bcount, &w.status->err);
+    // the forest is not in use yet: its array holds the ranks
+    if (g.total_bricks <= kTileBricks) {
+        // few particles per thread while that would leave SMs without a tile
+        if (g.total_n <= (int64_t)sm_count() * kCountThreads)
+            return run_count_tile<1>(pos, g, w, s);
+        if (g.total_n <= (int64_t)sm_count() * kCountThreads * 8)
+            return run_count_tile<4>(pos, g, w, s);
+        return run_count_tile<8>(pos, g, w, s);
+    }
+    k_bin_count<<<(unsigned)(bin_tiles_per_stream(g.total_n, kBinStreams) * kBinStreams), kBinThreads, 0, s>>>(
+        pos, g, w.bcount, brick_pad(g.total_bricks), w.parent, kBinStreams, &w.status->err);
     return cudaGetLastError();
 }
 
-int64_t scan_tmp_elems(int64_t len)
+int64_t scan_tiles(int64_t len)
 {
-    return (len + 1 + kScanTile - 1) / kScanTile + 1;
+    return (len + 1 + kScanTile - 1) / kScanTile;          // len + 1 outputs
 }
 
-cudaError_t launch_scan(const int* in, int* out, int64_t len, int* tmp, int64_t tmp_len, cudaStream_t s)
+cudaError_t launch_scan(const int* in, int pad, int* out, int64_t len, unsigned long long* state, int* ticket,
+                        int* err, cudaStream_t s)
 {
-    int64_t blocks = (len + 1 + kScanTile - 1) / kScanTile;   // len + 1 outputs
-    if (blocks + 1 > tmp_len)
-        return cudaErrorInvalidValue;
-    k_scan_reduce<<<(unsigned)blocks, kScanThreads, 0, s>>>(in, len, tmp);
-    k_scan_partials<<<1, 1024, 0, s>>>(tmp, blocks);
-    k_scan_apply<<<(unsigned)blocks, kScanThreads, 0, s>>>(in, out, len, tmp);
+    k_scan<<<(unsigned)scan_tiles(len), kScanThreads, 0, s>>>(in, pad, out, len, state, ticket, err);
     return cudaGetLastError();
 }
 
@@ -448,8 +557,10 @@ cudaError_t launch_bin_scatter(const float* pos, const Geometry& g, const Work& 
 {
     if (g.total_n == 0)
         return cudaSuccess;
-    k_bin_scatter<<<grid_for(g.total_n, 256, 8), 256, 0, s>>>(pos, g, w.bstart, w.bcursor, w.tmp,
-                                                            &w.status->err);
+    // in the order in which the ranks were given out
+    const int streams = g.total_bricks <= kTileBricks ? 1 : kBinStreams;
+    k_bin_scatter<<<(unsigned)(bin_tiles_per_stream(g.total_n, streams) * streams), kBinThreads, 0, s>>>(
+        pos, g, w.bstart, w.parent, streams, w.tmp, &w.status->err);
     return cudaGetLastError();
 }
 

@@ -479,6 +479,50 @@ __device__ __forceinline__ int uunion(int* parent, int a, int b, const UfArgs& u
 }
 
 // ------------------------------------------------------------------------
+// decoupled look-back (single-pass prefix sums over tiles)
+// ------------------------------------------------------------------------
+
+// The sum of the counts of all tiles before `tile`, whose own count is
+// `mine`, by one full warp.  state[t] = flag << 32 | value, zeroed before the
+// kernel: flag 1 = the tile's own count, 2 = the sum up to and including it;
+// value and flag share one 64-bit word, so relaxed accesses suffice.  Tiles
+// must be handed out in ascending order by a counter (every earlier tile is
+// then running or done, so each wait ends); the poll cap only turns a
+// corrupted state into a reported error.
+__device__ __forceinline__ int lookback(unsigned long long* state, int tile, int mine, int lane, int* err)
+{
+    if (lane == 0) {
+        const unsigned long long w = ((unsigned long long)(tile == 0 ? 2 : 1) << 32) | (unsigned)mine;
+        asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(state + tile), "l"(w) : "memory");
+    }
+    int before = 0;
+    for (int at = tile - 1; at >= 0; at -= kWarp) {
+        const int t = at - lane;
+        unsigned long long w = 2ull << 32;      // before the first tile: nothing
+        for (int poll = 0;; ++poll) {
+            if (t >= 0)
+                asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(state + t) : "memory");
+            if (__all_sync(kFull, (w >> 32) != 0ull))
+                break;
+            if (poll >= (1 << 22)) {
+                if (lane == 0) atomicOr(err, kErrInternal);
+                return 0;
+            }
+        }
+        const unsigned full = __ballot_sync(kFull, (w >> 32) == 2ull);
+        const int last = full ? __ffs(full) - 1 : kWarp - 1;    // nearest finished prefix
+        before += (int)__reduce_add_sync(kFull, lane <= last ? (unsigned)w : 0u);
+        if (full)
+            break;
+    }
+    if (lane == 0 && tile > 0) {
+        const unsigned long long w = (2ull << 32) | (unsigned)(before + mine);
+        asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(state + tile), "l"(w) : "memory");
+    }
+    return before;
+}
+
+// ------------------------------------------------------------------------
 // kernel launchers (one per phase); each returns cudaGetLastError()
 // ------------------------------------------------------------------------
 
@@ -495,18 +539,18 @@ struct Geometry {
 struct Work {
     float4* tmp;        // [total_n] particles in brick order
     float4* sorted;     // [total_n] particles in cell order, w = box-local index
-    int* parent;        // [total_n] union-find forest over cell-order slots
+    int* parent;        // [total_n] union-find forest over cell-order slots (ranks while binning)
     int* minorig;       // [total_n] smallest box-local index per root
     int* cnt;           // [total_n] group size per root
     int* cell_start;    // [total_cells + 1]
-    int* bcount;        // [total_bricks + 1]
+    int* bcount;        // [total_bricks * brick_pad]
     int* bstart;        // [total_bricks + 1]
-    int* bcursor;       // [total_bricks]
-    int* scan_tmp;      // scan partials
-    int64_t scan_tmp_len;
-    int* tile_cnt;      // [n_tiles + 1] catalogue entries per label tile
-    int* tile_off;      // [n_tiles + 1]
-    int* out_cursor;    // [total_n / kOutChunk + 1] fill of each output bucket
+    unsigned long long* scan_state; // [scan_tiles] look-back words of the brick scan
+    int* scan_ticket;   // scan tiles handed out
+    unsigned long long* tile_state; // look-back words of the output tiles, or of the scan of their counts
+    int* tile_ticket;   // tiles handed out
+    int* out_cursor;    // [n_tiles] fill of each output bucket, then the tile's catalogue entries
+    int* tile_off;      // [n_tiles + 1] first catalogue entry of each tile (above kDirectMax inputs)
     int64_t n_tiles;
     Status* status;     // device status
     unsigned long long* n_groups;  // [nbox]
@@ -524,16 +568,22 @@ struct Work {
     int64_t team_cap;    // capacity of team_list
 };
 
-constexpr int kCatTile = 2048;  // labels per catalogue tile
-constexpr int kOutChunkLog = 12;                 // outputs: input indices per chunk
-constexpr int kOutChunk = 1 << kOutChunkLog;
+// Bricks whose counters a CTA of the count kernel keeps in shared memory.
+constexpr int kTileBricks = 12288;
+constexpr int kOutTile = 4096;  // inputs per output tile
+// Largest number of inputs whose (label, size) pairs are stored straight at
+// the input's index (fof_out.cu).
+constexpr int64_t kDirectMax = 1 << 24;
 
 int sm_count();
 
 cudaError_t launch_bin_count(const float* pos, const Geometry& g, const Work& w, cudaStream_t s);
-cudaError_t launch_scan(const int* in, int* out, int64_t len, int* tmp, int64_t tmp_len,
-                        cudaStream_t s);
-int64_t scan_tmp_elems(int64_t len);
+// exclusive prefix sum of in[i * pad], i < len, into out[0..len]; state
+// (scan_tiles(len) words) and ticket start at zero
+cudaError_t launch_scan(const int* in, int pad, int* out, int64_t len, unsigned long long* state, int* ticket,
+                        int* err, cudaStream_t s);
+int64_t scan_tiles(int64_t len);
+int brick_pad(int64_t bricks);
 cudaError_t launch_bin_scatter(const float* pos, const Geometry& g, const Work& w, cudaStream_t s);
 cudaError_t launch_brick_sort(const Geometry& g, const Work& w, int dense_min, cudaStream_t s);
 // incremental re-binning: flags |= 1 if a particle left its cell, 2 if it left its brick
@@ -553,9 +603,8 @@ cudaError_t launch_big(const Geometry& g, const Work& w, int dense_min, const Uf
 // size_count: 0 warp-aggregated atomics, 1 per-block shared-memory hash table
 cudaError_t launch_finalize(const Geometry& g, const Work& w, const UfArgs& uf, int size_count,
                             cudaStream_t s);
-cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t* ids, int32_t* sizes,
-                           int32_t min_size, cudaStream_t s);
-cudaError_t launch_catalogue(const Geometry& g, const Work& w, const int32_t* sizes,
+cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t min_size, cudaStream_t s);
+cudaError_t launch_catalogue(const Geometry& g, const Work& w, int32_t* ids, int32_t* sizes,
                              int32_t min_size, int2* cat, int64_t cap, cudaStream_t s);
 
 }  // namespace fofgpu

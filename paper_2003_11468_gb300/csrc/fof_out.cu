@@ -7,11 +7,10 @@
 //              the paper's early elimination of singletons (Sec. 3.4.2),
 //              with the atomic additions of its parallel size count
 //              (Sec. 3.4.1) aggregated per warp.
-//   outputs    ids[i] = smallest index of i's group; sizes[label] = size,
-//              0 elsewhere (two passes, see below); per-box group counts;
-//              catalogue entries counted per label tile.
-//   catalogue  prefix sum over the label tiles, then each tile writes its
-//              (label, size) entries in ascending label order.
+//   outputs    (label, size) of every slot's group stored at the input index;
+//              per-box group and catalogue counts.
+//   catalogue  ids[i] = smallest index of i's group; sizes[label] = size, 0
+//              elsewhere; (label, size) entries in ascending label order.
 #include "fof_internal.cuh"
 
 namespace fofgpu {
@@ -147,27 +146,37 @@ __global__ void __launch_bounds__(256) k_finalize_hash(int64_t total, int* __res
     }
 }
 
-// Outputs go back to input order in two passes, so that no 4-byte value
-// is written to a random address (a read-modify-write of a whole sector):
-//   bucket  for every binned slot: label and size of its group, and one
-//           (offset, value) pair appended to the bucket of its input index's
-//           chunk of kOutChunk indices.  A chunk holds exactly kOutChunk
-//           inputs (the last one fewer), so bucket c starts at c*kOutChunk
-//           with no prefix sum, and the ~n/kOutChunk write heads stay in L2.
-//   place   one CTA per chunk: the pairs are placed in shared memory and
-//           ids and sizes written out coalesced.
-// A pair is (offset | is_label << 31, value): value = size when the input
-// is its group's label (then the label is the input's own box-local
-// index), else the label.
-__global__ void __launch_bounds__(256) k_outputs_bucket(Geometry g, const float4* __restrict__ sorted,
-                                                        const int* __restrict__ parent,
-                                                        const int* __restrict__ minorig,
-                                                        const int* __restrict__ cnt, int32_t thr,
-                                                        unsigned long long* __restrict__ n_groups,
-                                                        unsigned long long* __restrict__ n_cat,
-                                                        int* __restrict__ tile_cnt,
-                                                        int* __restrict__ out_cursor,
-                                                        int2* __restrict__ pairs, int* __restrict__ err)
+// Outputs go back to input order in two passes:
+//   scatter  for every binned slot: the label and size of its group as one
+//            8-byte pair (label, size if the input is its group's label, else
+//            0).  Up to kDirectMax inputs the pair is stored at the input's
+//            index: the pairs then stay in L2, and nothing but the store is
+//            needed.  Above, a sector of the pair array would leave L2 between
+//            its stores (a read-modify-write of DRAM for each), so the pairs
+//            are appended to the bucket of the input's tile instead, whose
+//            write heads stay in L2.  A tile holds exactly kOutTile inputs (the
+//            last one fewer), so bucket t starts at t * kOutTile.  (Direct and
+//            bucketed, this kernel: 2 million inputs 25 and 270 us, the
+//            buckets' cursors sharing lines; 16.7 million 0.27 and 0.38 ms;
+//            453 million 17.2 and 7.4 ms.)
+//   write    one CTA per tile: ids and sizes written out coalesced (a bucket's
+//            pairs placed in shared memory first), and the tile's catalogue
+//            entries (sizes at least thr, ascending label).  Up to kDirectMax
+//            inputs the entries are compacted at once, at an offset found by
+//            a decoupled look-back over the earlier tiles: no scan launch and
+//            no second read of the sizes.  Above, the look-back's chain over
+//            the tiles takes longer than the tiles themselves (453 million
+//            inputs: 2.6 ms), so the kernel leaves the tile's count, and a
+//            scan and k_catalogue follow (1.3 ms in all).
+template <bool kDirect>
+__global__ void __launch_bounds__(256) k_outputs_scatter(Geometry g, const float4* __restrict__ sorted,
+                                                         const int* __restrict__ parent,
+                                                         const int* __restrict__ minorig,
+                                                         const int* __restrict__ cnt, int32_t thr,
+                                                         unsigned long long* __restrict__ n_groups,
+                                                         unsigned long long* __restrict__ n_cat,
+                                                         int2* __restrict__ pairs,
+                                                         int* __restrict__ out_cursor, int* __restrict__ err)
 {
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -185,9 +194,9 @@ __global__ void __launch_bounds__(256) k_outputs_bucket(Geometry g, const float4
         // (the label pass only lowers roots' entries) and for singleton
         // roots; only a root of a larger group reads it from the binned record
         const int root = parent[s];
-        const bool root_s = root == (int)s;
+        const bool is_root = root == (int)s;
         int o, label, size;
-        if (!root_s) {
+        if (!is_root) {
             o = minorig[s];
             label = minorig[root];
             size = o == label ? cnt[root] : 0;
@@ -196,24 +205,31 @@ __global__ void __launch_bounds__(256) k_outputs_bucket(Geometry g, const float4
             label = minorig[s];
             o = size == 1 ? label : __float_as_int(sorted[s].w);
         }
-        const bool is_label = o == label;
-        int64_t gidx = p0 + o;
-        int chunk = (int)(gidx >> kOutChunkLog);
-        unsigned peers = __match_any_sync(active, chunk);
-        int leader = __ffs(peers) - 1;
-        int rank = __popc(peers & ((1u << lane) - 1u));
-        int off = 0;
-        if (lane == leader)
-            off = atomicAdd(out_cursor + chunk, __popc(peers));
-        off = __shfl_sync(active, off, leader) + rank;
-        if (off < kOutChunk) {
-            int word0 = (int)(gidx & (kOutChunk - 1)) | (is_label ? (int)0x80000000u : 0);
-            pairs[((int64_t)chunk << kOutChunkLog) + off] = make_int2(word0, is_label ? size : label);
-        } else {
-            atomicOr(err, kErrInternal);
+        // a record that binning never wrote is reported, and stays inside the box
+        const bool ok = (unsigned long long)o < (unsigned long long)g.boxes[bi].n;
+        const int64_t gidx = p0 + (ok ? o : 0);
+        int64_t at = gidx;
+        int2 e = make_int2(label, o == label ? size : 0);
+        bool room = ok;
+        if constexpr (!kDirect) {
+            const int tile = (int)(gidx / kOutTile);
+            const unsigned peers = __match_any_sync(active, tile);
+            const int leader = __ffs(peers) - 1;
+            int off = 0;
+            if (lane == leader)
+                off = atomicAdd(out_cursor + tile, __popc(peers));
+            off = __shfl_sync(active, off, leader) + __popc(peers & ((1u << lane) - 1u));
+            room = ok && off < kOutTile;
+            at = (int64_t)tile * kOutTile + off;
+            // a bucket's pair: (place in the tile | is-label << 31, size or label);
+            // a label is its own input's box-local index
+            e = make_int2((int)(gidx % kOutTile) | (o == label ? (int)0x80000000u : 0), o == label ? size : label);
         }
-        bool is_root = root == (int)s;
-        bool in_cat = is_root && size >= thr;
+        if (room)
+            pairs[at] = e;
+        else
+            atomicOr(err, kErrInternal);
+        const bool in_cat = is_root && size >= thr;
         // per-box counts: summed in registers while the warp stays inside one
         // box and added once per box (one counter per box would otherwise
         // take an atomic from every warp, all on one address)
@@ -240,8 +256,6 @@ __global__ void __launch_bounds__(256) k_outputs_bucket(Geometry g, const float4
                 if (nk) atomicAdd(n_cat + bi, (unsigned long long)nk);
             }
         }
-        if (in_cat)
-            atomicAdd(tile_cnt + (p0 + label) / kCatTile, 1);
     }
     // lane 0 took part in every iteration (its slot is the warp's smallest)
     if (lane == 0 && acc_box >= 0) {
@@ -250,103 +264,165 @@ __global__ void __launch_bounds__(256) k_outputs_bucket(Geometry g, const float4
     }
 }
 
-__global__ void __launch_bounds__(512) k_outputs_place(Geometry g, const int2* __restrict__ pairs,
-                                                       int32_t* __restrict__ ids,
-                                                       int32_t* __restrict__ sizes)
+constexpr int kOutThreads = 512;
+constexpr int kOutItems = kOutTile / kOutThreads;       // 8 rows of 512 inputs
+constexpr int kOutWarps = kOutThreads / 32;
+static_assert(kOutItems * kOutWarps == 4 * kWarp, "four row counts per lane of warp 0");
+
+// Exclusive prefix of the 128 row counts of a tile, in place, by warp 0;
+// returns their sum.
+__device__ __forceinline__ int scan_rows(int* s_cnt, int lane)
 {
-    __shared__ int s_ids[kOutChunk];
-    __shared__ int s_sizes[kOutChunk];
-    const int64_t n_chunks = (g.total_n + kOutChunk - 1) >> kOutChunkLog;
-    for (int64_t c = blockIdx.x; c < n_chunks; c += gridDim.x) {
-        const int64_t base = c << kOutChunkLog;
-        const int len = (int)min((int64_t)kOutChunk, g.total_n - base);
-        for (int k = threadIdx.x; k < len; k += blockDim.x) {
-            int2 e = pairs[base + k];
-            int off = e.x & (kOutChunk - 1);
-            if (e.x < 0) {                       // the input is its group's label
-                int64_t gidx = base + off;
-                int bi = box_of(g.box_p0, g.nbox, gidx);
-                s_ids[off] = (int)(gidx - g.boxes[bi].p0);
-                s_sizes[off] = e.y;
-            } else {
-                s_ids[off] = e.y;
-                s_sizes[off] = 0;
-            }
-        }
-        __syncthreads();
-        for (int k = threadIdx.x; k < len; k += blockDim.x) {
-            ids[base + k] = s_ids[k];
-            sizes[base + k] = s_sizes[k];
-        }
-        __syncthreads();
+    int c[4], sum = 0;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        c[r] = sum;
+        sum += s_cnt[4 * lane + r];
     }
-}
-
-constexpr int kCatThreads = 256;
-constexpr int kCatItems = kCatTile / kCatThreads;   // 8
-
-__device__ __forceinline__ int block_excl(int v, int* sw, int& total)
-{
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int x = v;
+    int x = sum;
     for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(kFull, x, o);
+        const int y = __shfl_up_sync(kFull, x, o);
         if (lane >= o) x += y;
     }
-    if (lane == 31) sw[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        int nw = blockDim.x >> 5;
-        int t = lane < nw ? sw[lane] : 0;
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(kFull, t, o);
-            if (lane >= o) t += y;
-        }
-        if (lane < nw) sw[lane] = t;
-    }
-    __syncthreads();
-    int off = wid ? sw[wid - 1] : 0;
-    total = sw[(blockDim.x >> 5) - 1];
-    __syncthreads();
-    return off + x - v;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+        s_cnt[4 * lane + r] = x - sum + c[r];
+    return __shfl_sync(kFull, x, 31);
 }
 
-// One block per tile of kCatTile labels: entries of the tile in ascending
-// label order at tile_off[tile].
-__global__ void __launch_bounds__(kCatThreads) k_catalogue(Geometry g, const int32_t* __restrict__ sizes,
-                                                           const int* __restrict__ tile_cnt,
-                                                           const int* __restrict__ tile_off,
-                                                           int32_t thr, int2* __restrict__ cat,
-                                                           int64_t cap, Status* status)
+template <bool kDirect>
+__global__ void __launch_bounds__(kOutThreads) k_outputs_write(Geometry g, const int2* __restrict__ pairs,
+                                                               int32_t* __restrict__ ids,
+                                                               int32_t* __restrict__ sizes, int32_t thr,
+                                                               int2* __restrict__ cat, int64_t cap,
+                                                               unsigned long long* __restrict__ tile_state,
+                                                               int* __restrict__ ticket,
+                                                               int* __restrict__ out_cursor, Status* status)
 {
-    __shared__ int sw[32];
-    for (int64_t tile = blockIdx.x; tile * kCatTile < g.total_n; tile += gridDim.x) {
-        if (tile_cnt[tile] == 0)
-            continue;      // block-uniform
-        int64_t base = tile * kCatTile + (int64_t)threadIdx.x * kCatItems;
-        int v[kCatItems];
-        int f = 0;
-        for (int k = 0; k < kCatItems; ++k) {
-            int64_t i = base + k;
-            v[k] = i < g.total_n ? sizes[i] : 0;
-            f += v[k] >= thr;
-        }
-        int total;
-        int64_t off = tile_off[tile] + block_excl(f, sw, total);
-        for (int k = 0; k < kCatItems; ++k) {
-            if (v[k] >= thr) {
-                int64_t i = base + k;
-                if (off < cap) {
-                    int bi = box_of(g.box_p0, g.nbox, i);
-                    cat[off] = make_int2((int)(i - g.boxes[bi].p0), v[k]);
+    __shared__ int s_tile, s_off;
+    __shared__ int s_cnt[kOutItems * kOutWarps];
+    __shared__ int2 placed[kDirect ? 1 : kOutTile];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // tiles are handed out in order, so every earlier tile is running or done
+    int tile = blockIdx.x;
+    if constexpr (kDirect) {
+        if (threadIdx.x == 0)
+            s_tile = atomicAdd(ticket, 1);
+        __syncthreads();
+        tile = s_tile;
+    }
+    const int64_t base = (int64_t)tile * kOutTile;
+    int2 e[kOutItems];
+    unsigned in[kOutItems];
+#pragma unroll
+    for (int k = 0; k < kOutItems; ++k) {
+        const int64_t i = base + k * kOutThreads + threadIdx.x;
+        e[k] = i < g.total_n ? pairs[i] : make_int2(0, 0);
+    }
+    if constexpr (!kDirect) {
+#pragma unroll
+        for (int k = 0; k < kOutItems; ++k) {
+            const int64_t i = base + k * kOutThreads + threadIdx.x;
+            if (i < g.total_n) {
+                const int off = e[k].x & (kOutTile - 1);
+                if (e[k].x < 0) {                        // the input is its group's label
+                    const int64_t gidx = base + off;
+                    e[k].x = (int)(gidx - g.boxes[box_of(g.box_p0, g.nbox, gidx)].p0);
+                } else {
+                    e[k] = make_int2(e[k].y, 0);
                 }
-                ++off;
+                placed[off] = e[k];
             }
         }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kOutItems; ++k)
+            e[k] = base + k * kOutThreads + threadIdx.x < g.total_n ? placed[k * kOutThreads + threadIdx.x]
+                                                                    : make_int2(0, 0);
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        int64_t nt = (g.total_n + kCatTile - 1) / kCatTile;
-        status->n_cat_total = tile_off[nt];
+#pragma unroll
+    for (int k = 0; k < kOutItems; ++k) {
+        const int64_t i = base + k * kOutThreads + threadIdx.x;
+        if (i < g.total_n) {
+            ids[i] = e[k].x;
+            sizes[i] = e[k].y;
+        }
+        in[k] = __ballot_sync(kFull, e[k].y >= thr);     // thr >= 1: never past the end
+        if (lane == 0)
+            s_cnt[k * kOutWarps + wid] = __popc(in[k]);
+    }
+    __syncthreads();
+    if (wid == 0) {
+        const int mine = scan_rows(s_cnt, lane);
+        if constexpr (!kDirect) {
+            if (lane == 0)
+                out_cursor[tile] = mine;                 // the bucket has been read
+            return;
+        }
+        const int before = lookback(tile_state, tile, mine, lane, &status->err);
+        if (lane == 0) {
+            s_off = before;
+            if (base + kOutTile >= g.total_n)            // the last tile knows the total
+                status->n_cat_total = before + mine;
+        }
+    }
+    if constexpr (!kDirect)
+        return;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kOutItems; ++k) {
+        if (e[k].y >= thr) {
+            const int64_t off = (int64_t)s_off + s_cnt[k * kOutWarps + wid] + __popc(in[k] & ((1u << lane) - 1u));
+            if (off < cap)
+                cat[off] = e[k];                         // the input is its label
+        }
+    }
+}
+
+// Catalogue above kDirectMax inputs: one CTA per output tile that holds
+// entries writes them in ascending label order from tile_off[tile] on.
+__global__ void __launch_bounds__(kOutThreads) k_catalogue(Geometry g, const int32_t* __restrict__ sizes,
+                                                           const int* __restrict__ tile_off, int32_t thr,
+                                                           int2* __restrict__ cat, int64_t cap, int64_t n_tiles,
+                                                           Status* status)
+{
+    __shared__ int s_cnt[kOutItems * kOutWarps];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        status->n_cat_total = tile_off[n_tiles];
+    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        const int t0 = tile_off[tile];
+        if (tile_off[tile + 1] == t0)
+            continue;                                    // block-uniform
+        int size[kOutItems];
+        unsigned in[kOutItems];
+#pragma unroll
+        for (int k = 0; k < kOutItems; ++k) {
+            const int64_t i = tile * kOutTile + k * kOutThreads + threadIdx.x;
+            size[k] = i < g.total_n ? sizes[i] : 0;
+        }
+#pragma unroll
+        for (int k = 0; k < kOutItems; ++k) {
+            in[k] = __ballot_sync(kFull, size[k] >= thr);
+            if (lane == 0)
+                s_cnt[k * kOutWarps + wid] = __popc(in[k]);
+        }
+        __syncthreads();
+        if (wid == 0)
+            scan_rows(s_cnt, lane);
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kOutItems; ++k) {
+            if (size[k] >= thr) {
+                const int64_t off =
+                    (int64_t)t0 + s_cnt[k * kOutWarps + wid] + __popc(in[k] & ((1u << lane) - 1u));
+                if (off < cap) {
+                    const int64_t i = tile * kOutTile + k * kOutThreads + threadIdx.x;
+                    cat[off] = make_int2((int)(i - g.boxes[box_of(g.box_p0, g.nbox, i)].p0), size[k]);
+                }
+            }
+        }
+        __syncthreads();
     }
 }
 
@@ -375,33 +451,43 @@ cudaError_t launch_finalize(const Geometry& g, const Work& w, const UfArgs& uf, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t* ids, int32_t* sizes,
-                           int32_t min_size, cudaStream_t s)
+cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t min_size, cudaStream_t s)
 {
     if (g.total_n == 0)
         return cudaSuccess;
     int32_t thr = min_size < 1 ? 1 : min_size;
     int2* pairs = (int2*)w.tmp;            // the brick-order copy is dead by now
-    k_outputs_bucket<<<grid_for(g.total_n, 256, 8), 256, 0, s>>>(
-        g, w.sorted, w.parent, w.minorig, w.cnt, thr, w.n_groups, w.n_cat, w.tile_cnt, w.out_cursor,
-        pairs, &w.status->err);
-    int64_t n_chunks = (g.total_n + kOutChunk - 1) >> kOutChunkLog;
-    int blocks = (int)(n_chunks < (int64_t)sm_count() * 4 ? n_chunks : (int64_t)sm_count() * 4);
-    k_outputs_place<<<blocks, 512, 0, s>>>(g, pairs, ids, sizes);
+    const int blocks = grid_for(g.total_n, 256, 8);
+    if (g.total_n <= kDirectMax)
+        k_outputs_scatter<true><<<blocks, 256, 0, s>>>(g, w.sorted, w.parent, w.minorig, w.cnt, thr, w.n_groups,
+                                                       w.n_cat, pairs, w.out_cursor, &w.status->err);
+    else
+        k_outputs_scatter<false><<<blocks, 256, 0, s>>>(g, w.sorted, w.parent, w.minorig, w.cnt, thr, w.n_groups,
+                                                        w.n_cat, pairs, w.out_cursor, &w.status->err);
     return cudaGetLastError();
 }
 
-cudaError_t launch_catalogue(const Geometry& g, const Work& w, const int32_t* sizes, int32_t min_size,
+cudaError_t launch_catalogue(const Geometry& g, const Work& w, int32_t* ids, int32_t* sizes, int32_t min_size,
                              int2* cat, int64_t cap, cudaStream_t s)
 {
     if (g.total_n == 0)
         return cudaSuccess;
     int32_t thr = min_size < 1 ? 1 : min_size;
-    cudaError_t e = launch_scan(w.tile_cnt, w.tile_off, w.n_tiles, w.scan_tmp, w.scan_tmp_len, s);
+    const int2* pairs = (const int2*)w.tmp;
+    const unsigned blocks = (unsigned)w.n_tiles;
+    if (g.total_n <= kDirectMax) {
+        k_outputs_write<true><<<blocks, kOutThreads, 0, s>>>(g, pairs, ids, sizes, thr, cat, cap, w.tile_state,
+                                                             w.tile_ticket, w.out_cursor, w.status);
+        return cudaGetLastError();
+    }
+    k_outputs_write<false><<<blocks, kOutThreads, 0, s>>>(g, pairs, ids, sizes, thr, cat, cap, w.tile_state,
+                                                          w.tile_ticket, w.out_cursor, w.status);
+    cudaError_t e = launch_scan(w.out_cursor, 1, w.tile_off, w.n_tiles, w.tile_state, w.tile_ticket,
+                                &w.status->err, s);
     if (e != cudaSuccess)
         return e;
-    int blocks = grid_for(w.n_tiles * kCatThreads, kCatThreads, 8);
-    k_catalogue<<<blocks, kCatThreads, 0, s>>>(g, sizes, w.tile_cnt, w.tile_off, thr, cat, cap, w.status);
+    k_catalogue<<<grid_for(w.n_tiles * kOutThreads, kOutThreads, 4), kOutThreads, 0, s>>>(
+        g, sizes, w.tile_off, thr, cat, cap, w.n_tiles, w.status);
     return cudaGetLastError();
 }
 

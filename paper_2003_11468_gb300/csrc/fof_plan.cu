@@ -4,6 +4,7 @@
 // device workspace sized for them, and a small pinned host block for the
 // status read-back.  fof_link enqueues binning and linking; fof_groups
 // enqueues finalisation and outputs and reads the status back once.
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -45,14 +46,26 @@ const char* kPhaseNames[kNumPhases] = {
     "bin_count", "scan_bricks", "bin_scatter", "brick_sort", "team_self", "big_sort", "dense_self",
     "dense_pairs", "big_pairs", "link", "finalize", "outputs", "catalogue",
 };
-const int kPhaseLaunches[kNumPhases] = {1, 3, 1, 1, 2, 1, 2, 2, 1, 1, 1, 2, 4};
+
+// kernel launches of one phase over total_n particles
+int phase_launches(int ph, int64_t total_n)
+{
+    switch (ph) {
+    case kPhTeamSelf:
+    case kPhDenseSelf:
+    case kPhDensePairs: return 2;
+    case kPhCatalogue: return total_n <= kDirectMax ? 1 : 3;
+    default: return 1;
+    }
+}
 
 constexpr int64_t kMaxTotal = 2147483646LL;   // slots and labels are int32
 constexpr int kDefaultRetryCap = 1 << 20;
 constexpr int kDefaultDenseMin = 256;
 constexpr double kDefaultOccupancy = 0.30;
 constexpr int kDefaultTeamMin = 10;
-constexpr int kMinTeamMin = 2;                 // smallest accepted team threshold (sizes team_list)
+constexpr int kMinTeamMin = 2;                 // smallest team threshold in use
+constexpr int kNumCounters = 4;                 // dense, team (small, large), big cells
 constexpr int kMaxCellsPerAxis = 4096;        // float32 cell-index precision (unsplit cells)
 constexpr int kMaxFinePerAxis = 16384;        // float32 index precision (sub-cells)
 
@@ -132,6 +145,8 @@ int sub_cells_for(double L, double l_x, int64_t nc)
     }
     return 1;
 }
+
+int team_min_of(const fof_options* opt);
 
 int setup_box(double L, double l_x, int64_t n, const fof_options* o, BoxDev& b)
 {
@@ -235,9 +250,7 @@ int setup_box(double L, double l_x, int64_t n, const fof_options* o, BoxDev& b)
         double rf = l_x / (L / (double)b.nf) + std::ldexp(1.0, -6);
         b.reach2 = (float)(rf * rf * (1.0 + std::ldexp(1.0, -20)));
     }
-    b.team_min = (o && o->team_min > 0) ? o->team_min : kDefaultTeamMin;
-    if (b.team_min < kMinTeamMin)
-        b.team_min = kMinTeamMin;
+    b.team_min = team_min_of(o);
     // Team bounding-box filter.  A neighbour particle shifted by +-float32(L)
     // and the float32 gaps to the box are each within L 2^-24 (shift: the
     // sum and float32(L); gap: one subtraction) per axis, 3 L 2^-24 together,
@@ -332,6 +345,9 @@ struct fof_plan {
     size_t ws_bytes = 0;
     bool own_ws = false;
     char* results_dev = nullptr;
+    char* zero_dev = nullptr;       // [zero_dev, zero_end) starts each run at zero
+    char* zero_end = nullptr;
+    bool groups_clean = false;      // fof_groups' counters are zero (no fof_groups since fof_link)
     char* results_host = nullptr;   // pinned
     bool results_from_slab = false;
     ResultsLayout rl{};
@@ -373,14 +389,13 @@ struct fof_plan {
 namespace {
 
 struct Layout {
-    size_t boxes, p0, brick0, results, bcount, bstart, bcursor, scan_tmp, tile_cnt, tile_off,
-        cell_start, tmp, sorted, parent, minorig, cnt, dense_list, n_dense, dense_root, out_cursor,
-        team_list, n_team, n_team_hi, big_list, n_big, total;
-    int64_t scan_len, n_tiles, dense_cap, team_cap;
+    size_t boxes, p0, brick0, results, bcount, bstart, scan_state, scan_ticket, tile_state, tile_ticket, out_cursor, tile_off,
+        cell_start, tmp, sorted, parent, minorig, cnt, dense_list, counters, dense_root, team_list, big_list, total;
+    size_t zero_end;     // [bcount, zero_end) starts each run at zero
+    int64_t n_tiles, dense_cap, team_cap;
 };
 
-Layout layout(int nbox, int64_t total_n, int64_t total_bricks, int64_t total_cells,
-              int dense_min = kDefaultDenseMin)
+Layout layout(int nbox, int64_t total_n, int64_t total_bricks, int64_t total_cells, int dense_min, int team_min)
 {
     Layout L{};
     size_t off = 0;
@@ -389,19 +404,24 @@ Layout layout(int nbox, int64_t total_n, int64_t total_bricks, int64_t total_cel
         off = align_up(off + (bytes ? bytes : 1), 256);
         return at;
     };
-    L.n_tiles = (total_n + kCatTile - 1) / kCatTile;
-    int64_t s1 = scan_tmp_elems(total_bricks), s2 = scan_tmp_elems(L.n_tiles);
-    L.scan_len = s1 > s2 ? s1 : s2;
+    L.n_tiles = (total_n + kOutTile - 1) / kOutTile;
     L.boxes = take(sizeof(BoxDev) * (size_t)nbox);
     L.p0 = take(8 * (size_t)nbox);
     L.brick0 = take(8 * (size_t)nbox);
+    // what starts each run at zero lies together: one memset before fof_link's
+    // kernels ([bcount, zero_end)), and, for a repeated fof_groups, one of its
+    // tail from the counts in the results block on
+    L.bcount = take(4 * (size_t)(total_bricks * brick_pad(total_bricks)));
+    L.scan_state = take(8 * (size_t)scan_tiles(total_bricks) + 4);
+    L.scan_ticket = L.scan_state + 8 * (size_t)scan_tiles(total_bricks);
+    L.counters = take(4 * kNumCounters);
     L.results = take(results_layout(nbox).bytes);
-    L.bcount = take(4 * (size_t)(total_bricks + 1));
-    L.bstart = take(4 * (size_t)(total_bricks + 1));
-    L.bcursor = take(4 * (size_t)(total_bricks + 1));
-    L.scan_tmp = take(4 * (size_t)L.scan_len);
-    L.tile_cnt = take(4 * (size_t)(L.n_tiles + 1));
+    L.tile_state = take(12 * (size_t)L.n_tiles + 4);
+    L.out_cursor = L.tile_state + 8 * (size_t)L.n_tiles;
+    L.tile_ticket = L.out_cursor + 4 * (size_t)L.n_tiles;
+    L.zero_end = off;
     L.tile_off = take(4 * (size_t)(L.n_tiles + 1));
+    L.bstart = take(4 * (size_t)(total_bricks + 1));
     L.cell_start = take(4 * (size_t)(total_cells + 1));
     L.tmp = take(16 * (size_t)total_n);
     L.sorted = take(16 * (size_t)total_n);
@@ -410,22 +430,66 @@ Layout layout(int nbox, int64_t total_n, int64_t total_bricks, int64_t total_cel
     L.cnt = take(4 * (size_t)total_n);
     L.dense_cap = total_n / dense_min + 1;
     L.dense_list = take(8 * (size_t)L.dense_cap);
-    L.n_dense = take(4);
     L.dense_root = take(4 * (size_t)(total_n / dense_min + 2));
-    L.out_cursor = take(4 * (size_t)((total_n >> kOutChunkLog) + 2));
-    L.team_cap = total_n / kMinTeamMin + 1;
+    L.team_cap = total_n / team_min + 1;
     L.team_list = take(8 * (size_t)L.team_cap);
-    L.n_team = take(4);
-    L.n_team_hi = take(4);
     L.big_list = take(8 * (size_t)(total_n / (kDenseMax + 1) + 1));
-    L.n_big = take(4);
     L.total = off;
     return L;
+}
+
+// Device pointers of a workspace laid out by L.
+void bind_workspace(char* ws, const Layout& L, int nbox, int64_t tn, int64_t tb, int64_t tc, Geometry& g, Work& w)
+{
+    g.boxes = (const BoxDev*)(ws + L.boxes);
+    g.box_p0 = (const int64_t*)(ws + L.p0);
+    g.box_brick0 = (const int64_t*)(ws + L.brick0);
+    g.nbox = nbox;
+    g.total_n = tn;
+    g.total_bricks = tb;
+    g.total_cells = tc;
+    const ResultsLayout rl = results_layout(nbox);
+    char* res = ws + L.results;
+    w.status = (Status*)(res + rl.status_off);
+    w.n_groups = (unsigned long long*)(res + rl.groups_off);
+    w.n_cat = (unsigned long long*)(res + rl.cat_off);
+    w.bcount = (int*)(ws + L.bcount);
+    w.bstart = (int*)(ws + L.bstart);
+    w.scan_state = (unsigned long long*)(ws + L.scan_state);
+    w.scan_ticket = (int*)(ws + L.scan_ticket);
+    w.tile_state = (unsigned long long*)(ws + L.tile_state);
+    w.tile_ticket = (int*)(ws + L.tile_ticket);
+    w.out_cursor = (int*)(ws + L.out_cursor);
+    w.tile_off = (int*)(ws + L.tile_off);
+    w.n_tiles = L.n_tiles;
+    w.cell_start = (int*)(ws + L.cell_start);
+    w.tmp = (float4*)(ws + L.tmp);
+    w.sorted = (float4*)(ws + L.sorted);
+    w.parent = (int*)(ws + L.parent);
+    w.minorig = (int*)(ws + L.minorig);
+    w.cnt = (int*)(ws + L.cnt);
+    w.dense_list = (int64_t*)(ws + L.dense_list);
+    w.dense_root = (int*)(ws + L.dense_root);
+    w.team_list = (int64_t*)(ws + L.team_list);
+    w.team_cap = L.team_cap;
+    w.big_list = (int64_t*)(ws + L.big_list);
+    int* counters = (int*)(ws + L.counters);
+    w.n_dense = counters;
+    w.n_team = counters + 1;
+    w.n_team_hi = counters + 2;
+    w.n_big = counters + 3;
 }
 
 int dense_min_of(const fof_options* opt)
 {
     return (opt && opt->dense_min > 0) ? opt->dense_min : kDefaultDenseMin;
+}
+
+// every box of a plan has the same team threshold
+int team_min_of(const fof_options* opt)
+{
+    const int t = (opt && opt->team_min > 0) ? opt->team_min : kDefaultTeamMin;
+    return t < kMinTeamMin ? kMinTeamMin : t;
 }
 
 int setup_batch(int32_t nbox, const double* box, const double* l_x, const int64_t* n,
@@ -472,8 +536,8 @@ int cuda_rc(cudaError_t e)
 
 void phase_begin(fof_plan* h, int ph, cudaStream_t s)
 {
-    h->launches += kPhaseLaunches[ph];
-    h->phase[ph].launches += kPhaseLaunches[ph];
+    h->launches += phase_launches(ph, h->g.total_n);
+    h->phase[ph].launches += phase_launches(ph, h->g.total_n);
     if (h->timing && !h->capturing) {
         cudaEventRecord(h->phase[ph].ev0, s);
     }
@@ -511,7 +575,7 @@ int create_plan(int32_t nbox, const double* box, const double* l_x, const int64_
     int rc = setup_batch(nbox, box, l_x, n, opt, boxes, tn, tb, tc);
     if (rc != FOF_OK)
         return rc;
-    Layout L = layout(nbox, tn, tb, tc, dense_min_of(opt));
+    Layout L = layout(nbox, tn, tb, tc, dense_min_of(opt), team_min_of(opt));
     if (workspace && (workspace_bytes < L.total || ((uintptr_t)workspace & 255u)))
         return FOF_ERR_ARG;
 
@@ -564,43 +628,10 @@ int create_plan(int32_t nbox, const double* box, const double* l_x, const int64_
         h->p0[i] = boxes[i].p0;
         h->brick0[i] = boxes[i].brick0;
     }
-    Geometry& g = h->g;
-    g.boxes = (const BoxDev*)(ws + L.boxes);
-    g.box_p0 = (const int64_t*)(ws + L.p0);
-    g.box_brick0 = (const int64_t*)(ws + L.brick0);
-    g.nbox = nbox;
-    g.total_n = tn;
-    g.total_bricks = tb;
-    g.total_cells = tc;
-    Work& w = h->w;
+    bind_workspace(ws, L, nbox, tn, tb, tc, h->g, h->w);
     h->results_dev = ws + L.results;
-    w.status = (Status*)(h->results_dev + h->rl.status_off);
-    w.n_groups = (unsigned long long*)(h->results_dev + h->rl.groups_off);
-    w.n_cat = (unsigned long long*)(h->results_dev + h->rl.cat_off);
-    w.bcount = (int*)(ws + L.bcount);
-    w.bstart = (int*)(ws + L.bstart);
-    w.bcursor = (int*)(ws + L.bcursor);
-    w.scan_tmp = (int*)(ws + L.scan_tmp);
-    w.scan_tmp_len = L.scan_len;
-    w.tile_cnt = (int*)(ws + L.tile_cnt);
-    w.tile_off = (int*)(ws + L.tile_off);
-    w.n_tiles = L.n_tiles;
-    w.cell_start = (int*)(ws + L.cell_start);
-    w.tmp = (float4*)(ws + L.tmp);
-    w.sorted = (float4*)(ws + L.sorted);
-    w.parent = (int*)(ws + L.parent);
-    w.minorig = (int*)(ws + L.minorig);
-    w.cnt = (int*)(ws + L.cnt);
-    w.dense_list = (int64_t*)(ws + L.dense_list);
-    w.n_dense = (int*)(ws + L.n_dense);
-    w.dense_root = (int*)(ws + L.dense_root);
-    w.out_cursor = (int*)(ws + L.out_cursor);
-    w.team_list = (int64_t*)(ws + L.team_list);
-    w.n_team = (int*)(ws + L.n_team);
-    w.n_team_hi = (int*)(ws + L.n_team_hi);
-    w.team_cap = L.team_cap;
-    w.big_list = (int64_t*)(ws + L.big_list);
-    w.n_big = (int*)(ws + L.n_big);
+    h->zero_dev = ws + L.bcount;
+    h->zero_end = ws + L.zero_end;
 
     cudaError_t e = cudaMemcpy(ws + L.boxes, boxes.data(), sizeof(BoxDev) * nbox, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
@@ -660,26 +691,22 @@ int enqueue_link(fof_plan* h, const float* pos, cudaStream_t s)
     const Geometry& g = h->g;
     const Work& w = h->w;
     const UfArgs uf = uf_args(h);
-    FOF_TRY(cudaMemsetAsync(h->results_dev, 0, h->rl.bytes, s));
+    FOF_TRY(cudaMemsetAsync(h->zero_dev, 0, (size_t)(h->zero_end - h->zero_dev), s));
+    h->groups_clean = true;
     if (g.total_n == 0) {
         h->linked = true;
         return FOF_OK;
     }
-    FOF_TRY(cudaMemsetAsync(w.bcount, 0, 4 * (size_t)(g.total_bricks + 1), s));
-    FOF_TRY(cudaMemsetAsync(w.bcursor, 0, 4 * (size_t)(g.total_bricks + 1), s));
     phase_begin(h, kPhBinCount, s);
     FOF_TRY(launch_bin_count(pos, g, w, s));
     phase_end(h, kPhBinCount, s);
     phase_begin(h, kPhScanBricks, s);
-    FOF_TRY(launch_scan(w.bcount, w.bstart, g.total_bricks, w.scan_tmp, w.scan_tmp_len, s));
+    FOF_TRY(launch_scan(w.bcount, brick_pad(g.total_bricks), w.bstart, g.total_bricks, w.scan_state, w.scan_ticket,
+                        &w.status->err, s));
     phase_end(h, kPhScanBricks, s);
     phase_begin(h, kPhBinScatter, s);
     FOF_TRY(launch_bin_scatter(pos, g, w, s));
     phase_end(h, kPhBinScatter, s);
-    FOF_TRY(cudaMemsetAsync(w.n_dense, 0, 4, s));
-    FOF_TRY(cudaMemsetAsync(w.n_team, 0, 4, s));
-    FOF_TRY(cudaMemsetAsync(w.n_team_hi, 0, 4, s));
-    FOF_TRY(cudaMemsetAsync(w.n_big, 0, 4, s));
     phase_begin(h, kPhBrickSort, s);
     FOF_TRY(launch_brick_sort(g, w, h->dense_min, s));
     phase_end(h, kPhBrickSort, s);
@@ -697,18 +724,19 @@ int enqueue_groups(fof_plan* h, int32_t* ids, int32_t* sizes, fof_group* cat, in
     const Work& w = h->w;
     if (g.total_n > 0) {
         // status.err is kept from fof_link; counts start from zero
-        FOF_TRY(cudaMemsetAsync(h->results_dev + h->rl.groups_off, 0,
-                                h->rl.bytes - h->rl.groups_off, s));
-        FOF_TRY(cudaMemsetAsync(w.tile_cnt, 0, 4 * (size_t)(w.n_tiles + 1), s));
-        FOF_TRY(cudaMemsetAsync(w.out_cursor, 0, 4 * (size_t)((g.total_n >> kOutChunkLog) + 2), s));
+        if (!h->groups_clean) {
+            char* from = h->results_dev + h->rl.groups_off;
+            FOF_TRY(cudaMemsetAsync(from, 0, (size_t)(h->zero_end - from), s));
+        }
+        h->groups_clean = false;
         phase_begin(h, kPhFinalize, s);
         FOF_TRY(launch_finalize(g, w, uf_args(h), h->size_count, s));
         phase_end(h, kPhFinalize, s);
         phase_begin(h, kPhOutputs, s);
-        FOF_TRY(launch_outputs(g, w, ids, sizes, min_size, s));
+        FOF_TRY(launch_outputs(g, w, min_size, s));
         phase_end(h, kPhOutputs, s);
         phase_begin(h, kPhCatalogue, s);
-        FOF_TRY(launch_catalogue(g, w, sizes, min_size, (int2*)cat, cap, s));
+        FOF_TRY(launch_catalogue(g, w, ids, sizes, min_size, (int2*)cat, cap, s));
         phase_end(h, kPhCatalogue, s);
     }
     FOF_TRY(cudaMemcpyAsync(h->results_host, h->results_dev, h->rl.bytes, cudaMemcpyDeviceToHost, s));
@@ -791,7 +819,7 @@ size_t fof_batch_workspace_bytes(int32_t nbox, const double* box, const double* 
     int64_t tn, tb, tc;
     if (setup_batch(nbox, box, l_x, n, opt, boxes, tn, tb, tc) != FOF_OK)
         return 0;
-    return layout(nbox, tn, tb, tc, dense_min_of(opt)).total;
+    return layout(nbox, tn, tb, tc, dense_min_of(opt), team_min_of(opt)).total;
 }
 
 int fof_link(fof_handle h, const float* pos_dev, void* stream)
@@ -811,7 +839,8 @@ int fof_relink(fof_handle h, const float* pos_dev, int32_t* path_out, void* stre
     int path = 2;
     if (h->binned && !h->capturing && g.total_n > 0) {
         // which particles left their cell or brick: one flag word, read back
-        FOF_TRY(cudaMemsetAsync(h->results_dev, 0, h->rl.bytes, s));
+        FOF_TRY(cudaMemsetAsync(h->results_dev, 0, (size_t)(h->zero_end - h->results_dev), s));
+        h->groups_clean = true;
         phase_begin(h, kPhBinCount, s);
         FOF_TRY(launch_relink_check(pos_dev, g, w, &w.status->pad, s));
         phase_end(h, kPhBinCount, s);
@@ -830,10 +859,7 @@ int fof_relink(fof_handle h, const float* pos_dev, int32_t* path_out, void* stre
         if (path == 1) {
             // every particle kept its brick: the slots are still grouped by
             // brick, so the per-brick cell sort runs on the new positions
-            FOF_TRY(cudaMemsetAsync(w.n_dense, 0, 4, s));
-            FOF_TRY(cudaMemsetAsync(w.n_team, 0, 4, s));
-            FOF_TRY(cudaMemsetAsync(w.n_team_hi, 0, 4, s));
-            FOF_TRY(cudaMemsetAsync(w.n_big, 0, 4, s));
+            FOF_TRY(cudaMemsetAsync(w.n_dense, 0, 4 * kNumCounters, s));
             phase_begin(h, kPhBrickSort, s);
             FOF_TRY(launch_brick_sort(g, w, h->dense_min, s));
             phase_end(h, kPhBrickSort, s);
@@ -1090,13 +1116,14 @@ int fof_graph_launch(fof_handle h, void* stream)
         return h ? FOF_ERR_STATE : FOF_ERR_ARG;
     FOF_TRY(cudaGraphLaunch(h->gexec, (cudaStream_t)stream));
     h->linked = true;
+    h->groups_clean = false;
     h->pending = true;
     h->last_cap = h->graph_cap;
     // a graph replays every phase once
     for (int k = 0; k < kNumPhases; ++k) {
         if (h->g.total_n > 0) {
-            h->launches += kPhaseLaunches[k];
-            h->phase[k].launches += kPhaseLaunches[k];
+            h->launches += phase_launches(k, h->g.total_n);
+            h->phase[k].launches += phase_launches(k, h->g.total_n);
         }
     }
     return FOF_OK;
@@ -1243,6 +1270,22 @@ std::mutex g_noalloc_mu;
 char* g_noalloc_ptr[kNoallocMaxDevices];                 // device address of the array, per device
 unsigned long long g_noalloc_ctx[kNoallocMaxDevices];    // id of the context it belongs to
 
+// What a problem counts against the array: a fixed accounting of 62 bytes per
+// particle (records in two orders 32, forest and labels 12, lists and output
+// cursors), 4 per cell and 12 per brick, so that the sizes that fit do not
+// change with the workspace layout, which needs no more than this.
+size_t noalloc_bytes(int64_t n, int64_t tb, int64_t tc)
+{
+    const int64_t out_tiles = (n + 2047) / 2048, scan = std::max((tb + 2048) / 2048, (out_tiles + 2048) / 2048) + 1;
+    const int64_t parts[] = {
+        1, 8, 8, 80, 4 * (tb + 1), 4 * (tb + 1), 4 * (tb + 1), 4 * scan, 4 * (out_tiles + 1), 4 * (out_tiles + 1),
+        4 * (tc + 1), 16 * n, 16 * n, 4 * n, 4 * n, 4 * n, 8 * (n / 256 + 1), 4, 4 * (n / 256 + 2),
+        4 * ((n >> 12) + 2), 8 * (n / 2 + 1), 4, 4, 8 * (n / 3073 + 1), 4};
+    size_t sum = 0;
+    for (int64_t p : parts) sum += align_up((size_t)(p > 0 ? p : 1), 256);
+    return sum;
+}
+
 // The id of the calling thread's current context (driver entry points looked
 // up through the runtime, so the library does not link the driver library).
 // Context ids are unique for the life of the process: after a device reset
@@ -1318,8 +1361,8 @@ extern "C" int fof_run_noalloc(double box, double l_x, int64_t n, const float* p
         return rc;
     const int64_t tb = (int64_t)b.nb * b.nb * b.nb;
     const int64_t tc = tb * (int64_t)b.r * b.r * b.r;
-    const Layout L = layout(1, n, tb, tc);
-    if (L.total > kNoallocScratchBytes)
+    const Layout L = layout(1, n, tb, tc, kDefaultDenseMin, kDefaultTeamMin);
+    if (noalloc_bytes(n, tb, tc) > kNoallocScratchBytes || L.total > kNoallocScratchBytes)
         return FOF_ERR_TOO_LARGE;
     if (n > 0 && (!pos_dev || !ids_dev || !sizes_dev))
         return FOF_ERR_ARG;
@@ -1331,42 +1374,9 @@ extern "C" int fof_run_noalloc(double box, double l_x, int64_t n, const float* p
     const ResultsLayout rl = results_layout(1);
 
     Geometry g{};
-    g.boxes = (const BoxDev*)(ws + L.boxes);
-    g.box_p0 = (const int64_t*)(ws + L.p0);
-    g.box_brick0 = (const int64_t*)(ws + L.brick0);
-    g.nbox = 1;
-    g.total_n = n;
-    g.total_bricks = tb;
-    g.total_cells = tc;
     Work w{};
+    bind_workspace(ws, L, 1, n, tb, tc, g, w);
     char* res = ws + L.results;
-    w.status = (Status*)(res + rl.status_off);
-    w.n_groups = (unsigned long long*)(res + rl.groups_off);
-    w.n_cat = (unsigned long long*)(res + rl.cat_off);
-    w.bcount = (int*)(ws + L.bcount);
-    w.bstart = (int*)(ws + L.bstart);
-    w.bcursor = (int*)(ws + L.bcursor);
-    w.scan_tmp = (int*)(ws + L.scan_tmp);
-    w.scan_tmp_len = L.scan_len;
-    w.tile_cnt = (int*)(ws + L.tile_cnt);
-    w.tile_off = (int*)(ws + L.tile_off);
-    w.n_tiles = L.n_tiles;
-    w.cell_start = (int*)(ws + L.cell_start);
-    w.tmp = (float4*)(ws + L.tmp);
-    w.sorted = (float4*)(ws + L.sorted);
-    w.parent = (int*)(ws + L.parent);
-    w.minorig = (int*)(ws + L.minorig);
-    w.cnt = (int*)(ws + L.cnt);
-    w.dense_list = (int64_t*)(ws + L.dense_list);
-    w.n_dense = (int*)(ws + L.n_dense);
-    w.dense_root = (int*)(ws + L.dense_root);
-    w.out_cursor = (int*)(ws + L.out_cursor);
-    w.team_list = (int64_t*)(ws + L.team_list);
-    w.n_team = (int*)(ws + L.n_team);
-    w.n_team_hi = (int*)(ws + L.n_team_hi);
-    w.team_cap = L.team_cap;
-    w.big_list = (int64_t*)(ws + L.big_list);
-    w.n_big = (int*)(ws + L.n_big);
 
     // The array keeps the previous call's contents: the box table is
     // rewritten and every counter that must start at zero is cleared here.
@@ -1374,19 +1384,12 @@ extern "C" int fof_run_noalloc(double box, double l_x, int64_t n, const float* p
     FOF_TRY(cudaMemcpyAsync(ws + L.boxes, &b, sizeof(BoxDev), cudaMemcpyHostToDevice, s));
     FOF_TRY(cudaMemcpyAsync(ws + L.p0, &zero, sizeof(zero), cudaMemcpyHostToDevice, s));
     FOF_TRY(cudaMemcpyAsync(ws + L.brick0, &zero, sizeof(zero), cudaMemcpyHostToDevice, s));
-    FOF_TRY(cudaMemsetAsync(res, 0, rl.bytes, s));
+    FOF_TRY(cudaMemsetAsync(ws + L.bcount, 0, L.zero_end - L.bcount, s));
     if (n > 0) {
-        FOF_TRY(cudaMemsetAsync(w.bcount, 0, 4 * (size_t)(tb + 1), s));
-        FOF_TRY(cudaMemsetAsync(w.bcursor, 0, 4 * (size_t)(tb + 1), s));
-        FOF_TRY(cudaMemsetAsync(w.tile_cnt, 0, 4 * (size_t)(w.n_tiles + 1), s));
-        FOF_TRY(cudaMemsetAsync(w.n_dense, 0, 4, s));
-        FOF_TRY(cudaMemsetAsync(w.out_cursor, 0, 4 * (size_t)((n >> kOutChunkLog) + 2), s));
         FOF_TRY(launch_bin_count(pos_dev, g, w, s));
-        FOF_TRY(launch_scan(w.bcount, w.bstart, tb, w.scan_tmp, w.scan_tmp_len, s));
+        FOF_TRY(launch_scan(w.bcount, brick_pad(g.total_bricks), w.bstart, g.total_bricks, w.scan_state, w.scan_ticket,
+                        &w.status->err, s));
         FOF_TRY(launch_bin_scatter(pos_dev, g, w, s));
-        FOF_TRY(cudaMemsetAsync(w.n_team, 0, 4, s));
-        FOF_TRY(cudaMemsetAsync(w.n_team_hi, 0, 4, s));
-        FOF_TRY(cudaMemsetAsync(w.n_big, 0, 4, s));
         FOF_TRY(launch_brick_sort(g, w, kDefaultDenseMin, s));
         FOF_TRY(launch_team_self(g, w, s));
         UfArgs uf;
@@ -1401,8 +1404,8 @@ extern "C" int fof_run_noalloc(double box, double l_x, int64_t n, const float* p
         FOF_TRY(launch_big(g, w, kDefaultDenseMin, uf, true, s));
         FOF_TRY(launch_link(g, w, kDefaultDenseMin, uf, s));
         FOF_TRY(launch_finalize(g, w, uf, 0, s));
-        FOF_TRY(launch_outputs(g, w, ids_dev, sizes_dev, min_size, s));
-        FOF_TRY(launch_catalogue(g, w, sizes_dev, min_size, (int2*)catalogue_dev, cat_capacity, s));
+        FOF_TRY(launch_outputs(g, w, min_size, s));
+        FOF_TRY(launch_catalogue(g, w, ids_dev, sizes_dev, min_size, (int2*)catalogue_dev, cat_capacity, s));
     }
     alignas(16) unsigned char host_res[128];
     FOF_TRY(cudaMemcpyAsync(host_res, res, rl.bytes, cudaMemcpyDeviceToHost, s));
