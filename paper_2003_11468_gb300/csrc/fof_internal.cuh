@@ -100,6 +100,34 @@ struct Status {
 };
 
 // ------------------------------------------------------------------------
+// warp helpers
+// ------------------------------------------------------------------------
+
+// Inclusive warp prefix sum.
+__device__ __forceinline__ int warp_incl(int v, int lane)
+{
+    for (int o = 1; o < 32; o <<= 1) {
+        int y = __shfl_up_sync(kFull, v, o);
+        if (lane >= o) v += y;
+    }
+    return v;
+}
+
+// Last lane l with start(l) <= t, where `start` is a non-decreasing per-lane
+// value with start(0) == 0 <= t (a binary search over the lanes; lanes
+// with an empty range share their successor's start and are never chosen).
+__device__ __forceinline__ int owner_lane(int start, int t)
+{
+    int lo = 0;
+#pragma unroll
+    for (int step = 16; step; step >>= 1) {      // lo + step <= 31 throughout
+        const int probe = __shfl_sync(kFull, start, lo + step);
+        if (probe <= t) lo += step;
+    }
+    return lo;
+}
+
+// ------------------------------------------------------------------------
 // box lookup: box index of a concatenated particle / brick index
 // ------------------------------------------------------------------------
 
@@ -592,7 +620,7 @@ cudaError_t launch_relink_check(const float* pos, const Geometry& g, const Work&
 cudaError_t launch_forest_init(const Geometry& g, const Work& w, cudaStream_t s);
 cudaError_t launch_dense(const Geometry& g, const Work& w, int dense_min, const UfArgs& uf, bool pairs,
                          cudaStream_t s);
-size_t dense_smem();
+bool dense_one_launch(int64_t total_n);
 cudaError_t launch_link(const Geometry& g, const Work& w, int dense_min, const UfArgs& uf,
                         cudaStream_t s);
 cudaError_t launch_team_self(const Geometry& g, const Work& w, cudaStream_t s);

@@ -137,30 +137,6 @@ __device__ __forceinline__ unsigned lanemask_lt()
     return m;
 }
 
-// Inclusive warp prefix sum.
-__device__ __forceinline__ int warp_incl(int v, int lane)
-{
-    for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(kFull, v, o);
-        if (lane >= o) v += y;
-    }
-    return v;
-}
-
-// Last lane l with start(l) <= t, where `start` is a non-decreasing per-lane
-// value with start(0) == 0 <= t (a binary search over the lanes; lanes
-// with an empty range share their successor's start and are never chosen).
-__device__ __forceinline__ int owner_lane(int start, int t)
-{
-    int lo = 0;
-#pragma unroll
-    for (int step = 16; step; step >>= 1) {      // lo + step <= 31 throughout
-        const int probe = __shfl_sync(kFull, start, lo + step);
-        if (probe <= t) lo += step;
-    }
-    return lo;
-}
-
 // The index of the r-th (0-based) set bit of m (r < popc(m)).
 __device__ __forceinline__ int nth_bit(unsigned m, int r)
 {

@@ -51,9 +51,9 @@ const char* kPhaseNames[kNumPhases] = {
 int phase_launches(int ph, int64_t total_n)
 {
     switch (ph) {
-    case kPhTeamSelf:
+    case kPhTeamSelf: return 2;
     case kPhDenseSelf:
-    case kPhDensePairs: return 2;
+    case kPhDensePairs: return dense_one_launch(total_n) ? 1 : 2;
     case kPhCatalogue: return total_n <= kDirectMax ? 1 : 3;
     default: return 1;
     }
