@@ -66,6 +66,9 @@ struct BoxDev {
     float reach2;     // (l_x / hf)^2 (1 + 2^-6): a sub-cell whose box is farther
                       // than this (in fine units, squared) holds no partner
     int32_t team_min; // occupancy from which k_link links a cell as a warp team
+    float inv_zb;     // float32(32 nc / L): z bins of a cell's z order (k_team_self)
+    float zb_width;   // a particle's z exceeds that of one in the same or an earlier
+                      // bin of its cell by more than -zb_width
     float bb_reach2;  // (l_x + 8 L 2^-24)^2 (1 + 2^-20): squared float32 gap from a
                       // bounding box beyond which no partner lies
 };
@@ -79,16 +82,15 @@ constexpr int kDenseMax = 3072;   // particles of a dense cell (shared memory)
 // Largest team cell whose own pairs one warp links in shared memory
 // (k_team_self); larger unsplit cells link their own pairs in k_link.
 constexpr int kTeamSelfMax = 256;
-// Team cells up to kTeamSplit particles are listed from the front of the
-// team list, larger ones from its back, so each of k_team_self's two
-// instantiations walks only its own cells.
+// Team cells up to kTeamSplit particles (one warp each in k_team_self) are
+// listed from the front of the team list, larger ones (one CTA each) from its
+// back.
 constexpr int kTeamSplit = 128;
 // Team cells from this size on are stored in z order by k_team_self, and the
 // kernels that stream them from the cell below read only the z-prefix that
-// can pair; sorting the many smaller cells costs more than it saves (measured
-// on the 1024^3 box at 0.30 particles per cell: from 25 on, together with a
-// team threshold of 10, the step is 1.5 ms shorter than from 17 with 8).
-constexpr int kSortMin = 25;
+// can pair (768^3 box, step: 83.0 ms from 17 on, 83.3 from 25, 83.6 from 10,
+// where sorting the many small cells costs more than it saves).
+constexpr int kSortMin = 17;
 constexpr int kMaxQ = 12;
 constexpr int kMaxQ3 = kMaxQ * kMaxQ * kMaxQ;
 

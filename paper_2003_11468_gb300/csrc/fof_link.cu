@@ -402,17 +402,16 @@ __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4*
                                             tc.cz + dz >= b.nc ? b.Lf : 0.f, 0.f);
             }
             // Neighbours k < 9 lie one cell up in z.  A team cell there (sorted
-            // by z in k_team_self) is cut to the prefix that the box filter can
-            // pass: past it, the z gap to the team alone squares above
-            // bb_reach2 (the filter's sum only adds non-negative terms, and
-            // the gap only grows along the z order).
-            // The prefix end is the first slot past the cut (a monotone
-            // predicate along the z order), bracketed by two rounds of a
-            // 4-ary search: the three lanes 3k, 3k+1, 3k+2 probe neighbour
-            // k's range at its quarters in one round.  The cut keeps [0, hi):
-            // every slot from hi on is past the cut, so it is conservative
-            // (the box filter drops the few kept slots between the first
-            // slot past the cut and hi).
+            // by z bin in k_team_self) is cut to the prefix that the box filter
+            // can pass: past it, the z gap to the team alone squares above
+            // bb_reach2 (the filter's sum only adds non-negative terms).  A
+            // slot after a probed one lies in its bin or a later one, so its
+            // z is at least the probed z less the width of a bin (zb_width).
+            // The cut is bracketed by two rounds of a 4-ary search: the three
+            // lanes 3k, 3k+1, 3k+2 probe neighbour k's range at its quarters
+            // in one round, and the cut keeps [0, hi): hi is the cell's end or
+            // a probed slot past the cut, so every slot from hi on is past it
+            // too (the box filter drops the few kept slots below hi).
             {
                 const int gk = lane / 3, sub = lane - 3 * gk;
                 const int src = gk < 9 ? gk : 0;
@@ -426,7 +425,7 @@ __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4*
                     bool beyond = false;
                     if (lo < hi) {
                         const int pr = sub == 0 ? p0 : (sub == 1 ? p1 : p2);
-                        const float d = __fsub_rn(__fadd_rn(sorted[jg + pr].z, sz), tbx.hz);
+                        const float d = __fsub_rn(__fadd_rn(__fsub_rn(sorted[jg + pr].z, b.zb_width), sz), tbx.hz);
                         beyond = d > 0.f && __fmul_rn(d, d) > b.bb_reach2;
                     }
                     const unsigned g3 = (__ballot_sync(kFull, beyond) >> (3 * src)) & 7u;
@@ -522,80 +521,79 @@ __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4*
 }
 
 // Self task of a team cell (team_min..kTeamSelfMax particles, not split
-// into sub-cells), one warp per cell.  The cell's particles are staged in
-// shared memory; the adjacency of the cell is built as bit rows, one
-// 32 x 32 block at a time: lane i tests (i, j) for the 32 j of a block,
-// collecting row i's word, and a ballot over the lanes gives row j's word of
-// the mirrored block, so each unordered pair is tested once outside the
-// diagonal blocks.  The components are then traced by breadth-first search
-// over bit sets (frontier rows OR-reduced across the warp), in ascending
-// order of their smallest member s, and every member's parent is set to s.
-// Isolated particles keep parent = self.  The kernel runs before any kernel
-// that links across cells, so no other thread touches these parents.
-// The kernel is instantiated for cells of up to 128 particles (half the
-// shared memory and registers, twice the resident warps) and for 129..256.
+// into sub-cells): cells of up to kTeamSplit particles by one warp each, larger
+// ones by a CTA of four warps.  The cell's particles are staged in shared
+// memory in z order; its adjacency is built as bit rows, one 32 x 32 block at
+// a time: lane i collects row i's word of the block, and the mirrored block's
+// words follow by a bit transpose across the lanes, so each unordered pair is
+// tested once outside the diagonal blocks.  The components are then traced by
+// breadth-first search over bit sets, each lane holding its rows in registers
+// (a step is a few ANDs and one ballot per 32 vertices), in ascending order of
+// their smallest member s, and every member's parent is set to s.  Isolated
+// particles keep parent = self.  The kernel runs before any kernel that links
+// across cells, so no other thread touches these parents.
+//
+// Bound by issue where cells are many, by one cell's chain where they are few
+// (one warp took 93,000 cycles for a cell of 256 when it sorted with a bitonic
+// network, mirrored blocks by a ballot per candidate and searched rows in
+// shared memory).  Before and after, us: 4,096 particles 78 and 14, 2 million
+// 153 and 57, 16.8 million (256^3) 642 and 348, 453 million (768^3) 13740 and
+// 9050.
 constexpr int kTeamWarps = 4;
+constexpr int kTeamBlocks = 8;               // CTAs per SM (64 registers, 27 KB)
+constexpr int kZBins = 32;                   // z bins of the order of a team cell
 
-// Cells of up to 128 particles copy the next cell's positions ahead into
-// shared memory (cp.async, buffer Q) instead of registers.
-template <int kMax>
-constexpr bool team_ahead_smem()
-{
-    return kMax <= 128;
-}
-
-template <int kMax>
-struct TeamSmem {
-    static constexpr int kWords = kMax / 32;
-    static constexpr int kStride = kWords + 1;         // odd stride: conflict-free rows
-    float4 P[kMax];
-    float4 Q[team_ahead_smem<kMax>() ? kMax : 1];     // the next cell, copied ahead
-    unsigned adj[kMax * kStride];
+struct TeamWarpSmem {                        // one warp's cell
+    static constexpr int kWords = kTeamSplit / 32;
+    static constexpr int kStride = kWords + 1;          // odd stride: conflict-free rows
+    float4 P[kTeamSplit];
+    float4 Q[kTeamSplit];                    // the next cell, copied ahead
+    unsigned adj[kTeamSplit * kStride];
+    int bin[kZBins];
 };
 
-// resident blocks per SM the instantiation is compiled for (registers)
-template <int kMax>
-constexpr int team_blocks()
-{
-    return kMax <= 128 ? 8 : 4;
-}
+struct TeamCtaSmem {                         // one CTA's cell
+    static constexpr int kWords = kTeamSelfMax / 32;
+    static constexpr int kStride = kWords + 1;
+    float4 P[kTeamSelfMax];
+    unsigned adj[kTeamSelfMax * kStride];
+    int bin[kZBins];
+    unsigned todo[kWords];
+    unsigned front[2][kWords];
+    float zlo[kWords], zhi[kWords];
+};
 
-template <int kMax>
-size_t team_smem_bytes()
-{
-    return sizeof(TeamSmem<kMax>) * kTeamWarps;
-}
+union TeamSmem {
+    TeamWarpSmem warp[kTeamWarps];
+    TeamCtaSmem cta;
+};
 
 // Positions that link to nothing: rows and columns beyond the cell's
 // particles.  Any difference with a real position or the other sentinel
 // squares to +inf in float32, so the pre-test rejects it.
 constexpr float kFar = 1e30f;
 
-// Tests of lane i's particle against particles jb*32 + t, t < jn8 (a
-// multiple of 8), returning row i's word of block jb.  For an off-diagonal
-// block (kOff) the ballot of each test is row j's word of block ib; lane j
-// keeps it and stores it once at the end.  The float32 pre-test decides a group of 4 pairs in an
-// unrolled loop (groups of 8 hold twice the candidate registers and made
-// the 128-particle instantiation spill); pairs in the uncertainty band take
-// the exact test after the group, in a loop entered only when some lane has
-// one, so the unrolled body stays small.  Inside one cell no pair needs the periodic wrap when
-// the box has at least 3 cells per axis (the cell side is then below L/2,
-// so the wrapped float32 separation equals the plain difference); kWrap
-// takes the full predicate for boxes with fewer cells.
-template <int kMax, bool kOff, bool kWrap>
-__device__ __forceinline__ unsigned block_tests(const float4& pi, TeamSmem<kMax>& S, int jb, int ib, int jn8,
-                                                int lane, const BoxDev& b)
+__device__ __forceinline__ float4 far_point(float v)
 {
-    constexpr int kAdjStride = TeamSmem<kMax>::kStride;
-    const float4* pj = &S.P[jb * 32];
-    unsigned row = 0;
-    unsigned col = 0;                          // off-diagonal: row (jb*32 + lane)'s word ib
+    return make_float4(v, v, v, 0.f);
+}
+
+// Row word of particle pi against pj[0..jn8), jn8 a multiple of 8.  The float32
+// pre-test decides; pairs in the uncertainty band are noted and take the exact
+// test after the block, in a loop entered only when some lane has one.  Inside
+// one cell no pair needs the periodic wrap when the box has at least 3 cells
+// per axis (the cell side is then below L/2, so the wrapped float32 separation
+// equals the plain difference); kWrap takes the full predicate for boxes with
+// fewer cells.
+template <bool kWrap>
+__device__ __forceinline__ unsigned block_word(const float4& pi, const float4* pj, int jn8, const BoxDev& b)
+{
     const float t_lo = b.t_lo, t_hi = b.t_hi;
-    for (int t0 = 0; t0 < jn8; t0 += 4) {
-        // 4 pre-tests: certainly linked (below t_lo) or undecided (the band)
-        unsigned byte = 0, hib = 0;
+    unsigned row = 0, band = 0;
+    for (int t0 = 0; t0 < jn8; t0 += 8) {
+        unsigned r8 = 0, b8 = 0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < 8; ++u) {
             const float4 q = pj[t0 + u];
             float s2;
             if (kWrap) {
@@ -606,280 +604,396 @@ __device__ __forceinline__ unsigned block_tests(const float4& pi, TeamSmem<kMax>
                 const float dz = __fsub_rn(pi.z, q.z);
                 s2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
             }
-            const bool lk = s2 < t_lo;
-            byte |= (unsigned)lk << u;
-            hib |= (unsigned)(s2 <= t_hi) << u;
-            if (kOff) {
-                const unsigned c = __ballot_sync(kFull, lk);
-                col = lane == t0 + u ? c : col;
-            }
+            const bool hi = s2 <= t_hi;
+            if (hi)
+                r8 |= 1u << u;
+            if (hi && s2 >= t_lo)
+                b8 |= 1u << u;
         }
-        // the exact test for the undecided pairs (rare)
-        const unsigned band = hib & ~byte;
-        if (__any_sync(kFull, band != 0u)) {
-            for (int u = 0; u < 4; ++u) {
-                const bool ex = ((band >> u) & 1u) && linked_exact_inl(pi, pj[t0 + u], b.L, b.l2);
-                byte |= (unsigned)ex << u;
-                if (kOff) {
-                    const unsigned c = __ballot_sync(kFull, ex);
-                    col |= lane == t0 + u ? c : 0u;
-                }
-            }
-        }
-        row |= byte << t0;
+        row |= r8 << t0;
+        band |= b8 << t0;
     }
-    // the mirrored words, one store per lane (rows past the block's
-    // particles are never read)
-    if (kOff)
-        S.adj[(jb * 32 + lane) * kAdjStride + ib] = col;
+    if (__any_sync(kFull, band != 0u))
+        while (band) {
+            const int t = __ffs(band) - 1;
+            band &= band - 1u;
+            if (!linked_exact_inl(pi, pj[t], b.L, b.l2))
+                row &= ~(1u << t);
+        }
     return row;
 }
 
-// Positions of a listed cell (size << 32 | first slot) into registers:
-// lane k holds particles k, k + 32, ...
-template <int kMin, int kMax>
-__device__ __forceinline__ void team_fetch(float4 (&R)[kMax / 32], int64_t e, const float4* sorted, int lane)
+// 32 x 32 bit matrix, row r in lane r: returns column `lane` as a row.
+__device__ __forceinline__ unsigned transpose32(unsigned x, int lane)
 {
-    const int c0 = (int)(uint32_t)e, m = (int)(e >> 32);
-    if (m <= kMin || m > kMax)                 // another instantiation's cell
-        return;
+    unsigned m = 0x0000ffffu;
 #pragma unroll
-    for (int r = 0; r < kMax / 32; ++r)
-        if (lane + 32 * r < m)
-            R[r] = sorted[c0 + lane + 32 * r];
+    for (int k = 16; k; k >>= 1) {
+        const unsigned y = __shfl_xor_sync(kFull, x, k);
+        x = (lane & k) ? (x & ~m) | ((y >> k) & m) : (x & m) | ((y & m) << k);
+        m ^= m << (k >> 1);
+    }
+    return x;
 }
 
-// The same into shared memory (S.Q) with cp.async, one commit group.
-template <int kMin, int kMax>
-__device__ __forceinline__ void team_fetch_smem(TeamSmem<kMax>& S, int64_t e, const float4* sorted, int lane)
+// z bin of a particle in its cell (cz): a monotone function of z
+__device__ __forceinline__ int z_bin(float z, int cz, const BoxDev& b)
+{
+    const int k = (int)__fmul_rn(z, b.inv_zb) - kZBins * cz;
+    return min(max(k, 0), kZBins - 1);
+}
+
+// Adjacency block (ib, jb), jb >= ib, of the staged cell: its words and those
+// of the mirrored block.  `apart`: no pair of the block can be linked.
+template <int kStride>
+__device__ __forceinline__ void adjacency_block(const float4* P, unsigned* adj, int m, int ib, int jb, bool apart,
+                                                int lane, const BoxDev& b)
+{
+    const int i = ib * 32 + lane;
+    unsigned row = 0u;
+    if (!apart) {
+        const float4 pi = i < m ? P[i] : far_point(-kFar);
+        const int jn8 = (min(32, m - jb * 32) + 7) & ~7;
+        row = b.nc >= 3 ? block_word<false>(pi, P + jb * 32, jn8, b) : block_word<true>(pi, P + jb * 32, jn8, b);
+    }
+    if (jb == ib)
+        row &= ~(1u << lane);                  // the particle itself
+    adj[i * kStride + jb] = row;
+    if (jb != ib)
+        adj[(jb * 32 + lane) * kStride + ib] = apart ? 0u : transpose32(row, lane);
+}
+
+// Components of the adjacency rows of a cell of kNw * 32 rows by one warp:
+// lane l holds rows l, l + 32, ...; the vertex sets are the same in every lane.
+template <int kNw>
+__device__ __forceinline__ void trace_components(const unsigned (&rows)[kNw][kNw], int* parent, int c0, int lane)
+{
+    unsigned todo[kNw];
+#pragma unroll
+    for (int r = 0; r < kNw; ++r) {
+        unsigned any = 0u;
+#pragma unroll
+        for (int k = 0; k < kNw; ++k)
+            any |= rows[r][k];
+        todo[r] = __ballot_sync(kFull, any != 0u);
+    }
+    for (;;) {
+        unsigned comp[kNw], front[kNw];
+        int s = -1;
+#pragma unroll
+        for (int r = 0; r < kNw; ++r) {
+            const bool here = s < 0 && todo[r] != 0u;
+            front[r] = here ? todo[r] & (0u - todo[r]) : 0u;
+            if (here)
+                s = r * 32 + __ffs(todo[r]) - 1;
+            comp[r] = front[r];
+        }
+        if (s < 0)
+            break;
+        for (int step = 0; step < kNw * 32; ++step) {      // every step adds a vertex
+            unsigned nxt[kNw], any = 0u;
+#pragma unroll
+            for (int r = 0; r < kNw; ++r) {
+                unsigned hit = 0u;
+#pragma unroll
+                for (int k = 0; k < kNw; ++k)
+                    hit |= rows[r][k] & front[k];
+                nxt[r] = __ballot_sync(kFull, hit != 0u) & ~comp[r];
+                any |= nxt[r];
+            }
+#pragma unroll
+            for (int r = 0; r < kNw; ++r) {
+                comp[r] |= nxt[r];
+                front[r] = nxt[r];
+            }
+            if (!any)
+                break;
+        }
+#pragma unroll
+        for (int r = 0; r < kNw; ++r) {
+            todo[r] &= ~comp[r];
+            if ((comp[r] >> lane) & 1u)
+                parent[c0 + r * 32 + lane] = c0 + s;
+        }
+    }
+}
+
+template <int kNw>
+__device__ __forceinline__ void trace_staged(const TeamWarpSmem& S, int* parent, int c0, int lane)
+{
+    unsigned rows[kNw][kNw];
+#pragma unroll
+    for (int r = 0; r < kNw; ++r)
+#pragma unroll
+        for (int k = 0; k < kNw; ++k)
+            rows[r][k] = S.adj[(r * 32 + lane) * TeamWarpSmem::kStride + k];
+    trace_components<kNw>(rows, parent, c0, lane);
+}
+
+// Positions of a listed cell (size << 32 | first slot) into S.Q with cp.async,
+// one commit group; lane k copies particles k, k + 32, ...
+__device__ __forceinline__ void team_fetch(TeamWarpSmem& S, int64_t e, const float4* sorted, int lane)
 {
     const int c0 = (int)(uint32_t)e, m = (int)(e >> 32);
-    if (m > kMin && m <= kMax) {
 #pragma unroll
-        for (int r = 0; r < kMax / 32; ++r)
-            if (lane + 32 * r < m)
-                cp_async16(&S.Q[lane + 32 * r], sorted + c0 + lane + 32 * r);
-    }
+    for (int r = 0; r < kTeamSplit / 32; ++r)
+        if (lane + 32 * r < m)
+            cp_async16(&S.Q[lane + 32 * r], sorted + c0 + lane + 32 * r);
     cp_async_commit();
 }
 
-// Sorts the staged cell (nw * 32 entries of S.P, sentinels after the cell's
-// particles) by z in place: a bitonic network over the next power of two,
-// padded with more sentinels.  Every z is finite and non-negative, the
-// sentinels' z (kFar) exceeds every position, so the cell's particles come
-// first in exact float order.
-template <int kMax>
-__device__ __forceinline__ void sort_cell_z(TeamSmem<kMax>& S, int nw, int lane)
+// One cell of 33..kTeamSelfMax particles by the whole CTA.
+__device__ __forceinline__ void team_cell_cta(TeamCtaSmem& S, int c0, int m, float4* sorted, int* parent,
+                                              int* minorig, const BoxDev& b)
 {
-    const int n = nw * 32;
-    int n2 = 32;
-    while (n2 < n) n2 <<= 1;                   // <= kMax
-    for (int k = n + lane; k < n2; k += 32)
-        S.P[k] = make_float4(kFar, kFar, kFar, 0.f);
-    __syncwarp();
-    for (int size = 2; size <= n2; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            // pair p: its lower index i is p with a zero inserted at the
-            // stride bit, so every lane has a pair and accesses stay dense
-            for (int pr = lane; pr < (n2 >> 1); pr += 32) {
-                const int i = ((pr & ~(stride - 1)) << 1) | (pr & (stride - 1));
-                const int l = i | stride;
-                const float4 a = S.P[i], c = S.P[l];
-                if ((a.z > c.z) == ((i & size) == 0)) {
-                    S.P[i] = c;
-                    S.P[l] = a;
-                }
-            }
-            __syncwarp();
+    constexpr int kThreads = kTeamWarps * 32, kPer = kTeamSelfMax / kThreads;
+    constexpr int kNw = TeamCtaSmem::kWords, kStride = TeamCtaSmem::kStride;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int nw = (m + 31) >> 5;
+    float4 v[kPer];
+    int bin[kPer], rank[kPer];
+    if (threadIdx.x < kZBins)
+        S.bin[threadIdx.x] = 0;
+#pragma unroll
+    for (int r = 0; r < kPer; ++r) {
+        const int k = r * kThreads + threadIdx.x;
+        if (k < m)
+            v[r] = sorted[c0 + k];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kPer; ++r) {
+        const int k = r * kThreads + threadIdx.x;
+        if (k < m) {
+            bin[r] = z_bin(v[r].z, cell_coord(v[r].z, b), b);
+            rank[r] = atomicAdd(S.bin + bin[r], 1);
         }
     }
+    __syncthreads();
+    if (wid == 0) {
+        const int c = S.bin[lane];
+        S.bin[lane] = warp_incl(c, lane) - c;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kPer; ++r) {
+        const int k = r * kThreads + threadIdx.x;
+        if (k < m) {
+            const int at = S.bin[bin[r]] + rank[r];
+            S.P[at] = v[r];
+            sorted[c0 + at] = v[r];
+            minorig[c0 + at] = __float_as_int(v[r].w);
+        } else if (k < nw * 32) {
+            S.P[k] = far_point(kFar);
+        }
+    }
+    __syncthreads();
+    // the z range of each 32 particles: blocks too far apart hold no link
+    for (int r = wid; r < nw; r += kTeamWarps) {
+        const unsigned z = __float_as_uint(S.P[r * 32 + lane].z + 0.f);    // finite and >= 0: ordered bits
+        const bool in = r * 32 + lane < m;
+        const unsigned lo = __reduce_min_sync(kFull, in ? z : 0x7f800000u), hi = __reduce_max_sync(kFull, in ? z : 0u);
+        if (lane == 0) {
+            S.zlo[r] = __uint_as_float(lo);
+            S.zhi[r] = __uint_as_float(hi);
+        }
+    }
+    __syncthreads();
+    for (int p = wid; p < nw * (nw + 1) / 2; p += kTeamWarps) {
+        int ib = 0, jb = p;
+        while (jb >= nw - ib) {
+            jb -= nw - ib;
+            ++ib;
+        }
+        jb += ib;
+        const float gap = __fsub_rn(S.zlo[jb], S.zhi[ib]);
+        adjacency_block<kStride>(S.P, S.adj, m, ib, jb, b.nc >= 3 && gap > 0.f && __fmul_rn(gap, gap) > b.t_hi, lane,
+                                 b);
+    }
+    __syncthreads();
+    // warp w searches row blocks w and w + kTeamWarps; the frontier's words are
+    // exchanged through shared memory, two buffers in turn
+    unsigned rows[2][kNw];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int r = wid + h * kTeamWarps;
+        unsigned any = 0u;
+#pragma unroll
+        for (int k = 0; k < kNw; ++k) {
+            rows[h][k] = r < nw && k < nw ? S.adj[(r * 32 + lane) * kStride + k] : 0u;
+            any |= rows[h][k];
+        }
+        const unsigned t = __ballot_sync(kFull, any != 0u);
+        if (lane == 0)
+            S.todo[r] = t;
+    }
+    __syncthreads();
+    unsigned todo[kNw];
+#pragma unroll
+    for (int k = 0; k < kNw; ++k)
+        todo[k] = S.todo[k];
+    int buf = 0;
+    for (;;) {
+        unsigned front[kNw];
+        int s = -1;
+#pragma unroll
+        for (int k = 0; k < kNw; ++k) {
+            const bool here = s < 0 && todo[k] != 0u;
+            front[k] = here ? todo[k] & (0u - todo[k]) : 0u;
+            if (here)
+                s = k * 32 + __ffs(todo[k]) - 1;
+        }
+        if (s < 0)
+            break;
+        unsigned own[2];                       // this warp's words of the component
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            own[h] = (s >> 5) == wid + h * kTeamWarps ? 1u << (s & 31) : 0u;
+        for (int step = 0; step < kTeamSelfMax; ++step) {  // every step adds a vertex
+#pragma unroll
+            for (int k = 0; k < kNw; ++k)
+                todo[k] &= ~front[k];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                unsigned hit = 0u;
+#pragma unroll
+                for (int k = 0; k < kNw; ++k)
+                    hit |= rows[h][k] & front[k];
+                const unsigned nxt = __ballot_sync(kFull, hit != 0u) & ~own[h];
+                own[h] |= nxt;
+                if (lane == 0)
+                    S.front[buf][wid + h * kTeamWarps] = nxt;
+            }
+            __syncthreads();
+            unsigned any = 0u;
+#pragma unroll
+            for (int k = 0; k < kNw; ++k) {
+                front[k] = S.front[buf][k];
+                any |= front[k];
+            }
+            buf ^= 1;
+            if (!any)
+                break;
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if ((own[h] >> lane) & 1u)
+                parent[c0 + (wid + h * kTeamWarps) * 32 + lane] = c0 + s;
+    }
+    __syncthreads();                           // smem reused by the next cell
 }
 
-template <int kMin, int kMax>
-__global__ void __launch_bounds__(kTeamWarps * 32, team_blocks<kMax>())
-    k_team_self(Geometry g, const int64_t* __restrict__ list, const int* __restrict__ n_list, int64_t back,
-                float4* sorted, int* __restrict__ parent, int* __restrict__ minorig, int* err)
+__global__ void __launch_bounds__(kTeamWarps * 32, kTeamBlocks)
+    k_team_self(Geometry g, const int64_t* __restrict__ list, int64_t cap, const int* __restrict__ n_lo,
+                const int* __restrict__ n_hi, float4* sorted, int* __restrict__ parent, int* __restrict__ minorig)
 {
-    // entries from the front of the list (back == 0) or from its back end
-    auto entry = [&](int i) { return back ? list[back - 1 - i] : list[i]; };
-    constexpr int kTeamMax = kMax;
-    constexpr int kTeamWords = kMax / 32;
-    constexpr int kAdjStride = TeamSmem<kMax>::kStride;
     extern __shared__ float4 team_raw[];
+    TeamSmem& smem = *reinterpret_cast<TeamSmem*>(team_raw);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    TeamSmem<kMax>& S = reinterpret_cast<TeamSmem<kMax>*>(team_raw)[wid];
-    const int n = *n_list;
+    // cells above kTeamSplit lie at the back of the list
+    for (int it = blockIdx.x, n = *n_hi; it < n; it += gridDim.x) {
+        const int64_t e = list[cap - 1 - it];
+        const int c0 = (int)(uint32_t)e;
+        team_cell_cta(smem.cta, c0, (int)(e >> 32), sorted, parent, minorig, g.boxes[box_of(g.box_p0, g.nbox, c0)]);
+    }
+    // the others, one per warp, the last CTAs first (they have the fewest
+    // large cells).  Software pipeline: the next cell's positions are copied
+    // ahead while this cell is linked, and the entry after it is read.
+    TeamWarpSmem& S = smem.warp[wid];
+    const int n = *n_lo;
     const int stride = gridDim.x * kTeamWarps;
-    // software pipeline: the next cell's positions are loaded while this
-    // cell is linked (into shared memory with cp.async for cells up to 128,
-    // into registers for larger ones), and the entry after it is read
-    int it = blockIdx.x * kTeamWarps + wid;
-    int64_t e = it < n ? entry(it) : 0;
-    constexpr bool kAhead = team_ahead_smem<kMax>();
-    float4 R[kAhead ? 1 : kTeamWords];
-    if constexpr (kAhead)
-        team_fetch_smem<kMin, kMax>(S, e, sorted, lane);
-    else
-        team_fetch<kMin, kMax>(R, e, sorted, lane);
-    int64_t e_next = it + stride < n ? entry(it + stride) : 0;
+    int it = (gridDim.x - 1 - blockIdx.x) * kTeamWarps + wid;
+    int64_t e = it < n ? list[it] : 0;
+    team_fetch(S, e, sorted, lane);
+    int64_t e_next = it + stride < n ? list[it + stride] : 0;
     for (; it < n; it += stride) {
         const int c0 = (int)(uint32_t)e, m = (int)(e >> 32);
         const int nw = (m + 31) >> 5;
-        const bool in_range = m > kMin && m <= kMax;
-        if constexpr (kAhead)
-            cp_async_wait_all();               // each lane reads back only its own copies
-        if (in_range) {
+        const BoxDev& b = g.boxes[box_of(g.box_p0, g.nbox, c0)];
+        cp_async_wait_all();                   // each lane reads back only its own copies
+        // the cell in z order (bins of 1/32 of the cell), also in global
+        // memory: the streams of the neighbours below then read only a
+        // z-prefix of it (k_link), and blocks of 32 here are z-slabs whose
+        // gaps prune block pairs.  No kernel has read these slots' order yet
+        // (cross-cell links come later).  Cells below kSortMin are not sorted
+        // (k_link searches no smaller).
+        if (m >= kSortMin) {
+            S.bin[lane] = 0;
+            __syncwarp();
+            int place[kTeamSplit / 32];        // bin << 8 | rank
 #pragma unroll
-            for (int r = 0; r < kTeamWords; ++r) {   // the ragged tail links nothing
+            for (int r = 0; r < kTeamSplit / 32; ++r) {
                 const int k = lane + 32 * r;
-                if (k < nw * 32) {
-                    float4 v = make_float4(kFar, kFar, kFar, 0.f);
-                    if (k < m) {
-                        if constexpr (kAhead)
-                            v = S.Q[k];
-                        else
-                            v = R[r];
-                    }
-                    S.P[k] = v;
+                if (k < m) {
+                    const float z = S.Q[k].z;
+                    const int bin = z_bin(z, cell_coord(z, b), b);
+                    place[r] = (bin << 8) | atomicAdd(S.bin + bin, 1);
                 }
             }
+            __syncwarp();
+            const int c = S.bin[lane];
+            __syncwarp();
+            S.bin[lane] = warp_incl(c, lane) - c;
+            __syncwarp();
+#pragma unroll
+            for (int r = 0; r < kTeamSplit / 32; ++r) {
+                const int k = lane + 32 * r;
+                if (k < m) {
+                    const int at = S.bin[place[r] >> 8] + (place[r] & 255);
+                    const float4 v = S.Q[k];
+                    S.P[at] = v;
+                    sorted[c0 + at] = v;
+                    minorig[c0 + at] = __float_as_int(v.w);
+                }
+            }
+        } else if (lane < m) {                 // kSortMin <= 32: one particle per lane
+            S.P[lane] = S.Q[lane];
         }
+        if (nw * 32 - 32 + lane >= m)          // the ragged tail links nothing
+            S.P[nw * 32 - 32 + lane] = far_point(kFar);
         __syncwarp();
         e = e_next;
-        if (it + stride < n) {
-            if constexpr (kAhead)
-                team_fetch_smem<kMin, kMax>(S, e, sorted, lane);
-            else
-                team_fetch<kMin, kMax>(R, e, sorted, lane);
-        }
-        e_next = it + 2 * stride < n ? entry(it + 2 * stride) : 0;
-        if (!in_range)                         // another instantiation's cell
-            continue;
-        const BoxDev& b = g.boxes[box_of(g.box_p0, g.nbox, c0)];
+        if (it + stride < n)
+            team_fetch(S, e, sorted, lane);
+        e_next = it + 2 * stride < n ? list[it + 2 * stride] : 0;
 
-        // the cell in z order, also in global memory: the streams of the
-        // neighbours below then read only a z-prefix of it (k_link), and
-        // blocks of 32 here are z-slabs whose gaps prune block pairs.  No
-        // kernel has read these slots' order yet (cross-cell links come later).
-        // Cells below kSortMin are not sorted (k_link searches no smaller).
-        if (m >= kSortMin) {
-            sort_cell_z<kMax>(S, nw, lane);
-            for (int k = lane; k < m; k += 32) {
-                const float4 q = S.P[k];
-                sorted[c0 + k] = q;
-                minorig[c0 + k] = __float_as_int(q.w);
-            }
-        }
-
-        // adjacency rows (row1: the only word when nw == 1)
-        unsigned row1 = 0u;
-        for (int ib = 0; ib < nw; ++ib) {
-            const int i = ib * 32 + lane;
-            const float4 pi = i < m ? S.P[i] : make_float4(-kFar, -kFar, -kFar, 0.f);
-            for (int jb = ib; jb < nw; ++jb) {
-                const int jn8 = (min(32, m - jb * 32) + 7) & ~7;
-                unsigned row;
-                // z-slabs of a sorted cell too far apart: every pair's float32
-                // separation squared exceeds t_hi (rounding is monotone), so no link
-                const float gap = jb > ib && m >= kSortMin ? __fsub_rn(S.P[jb * 32].z, S.P[ib * 32 + 31].z) : 0.f;
-                if (b.nc >= 3 && gap > 0.f && __fmul_rn(gap, gap) > b.t_hi) {
-                    row = 0u;
-                    if (lane < min(32, m - jb * 32))
-                        S.adj[(jb * 32 + lane) * kAdjStride + ib] = 0u;
-                } else if (b.nc >= 3) {
-                    row = jb == ib ? block_tests<kMax, false, false>(pi, S, jb, ib, jn8, lane, b)
-                                   : block_tests<kMax, true, false>(pi, S, jb, ib, jn8, lane, b);
-                } else {
-                    row = jb == ib ? block_tests<kMax, false, true>(pi, S, jb, ib, jn8, lane, b)
-                                   : block_tests<kMax, true, true>(pi, S, jb, ib, jn8, lane, b);
-                }
-                if (jb == ib)
-                    row &= ~(1u << lane);      // the particle itself
-                if (nw == 1)
-                    row1 = i < m ? row : 0u;
-                else if (i < m)
-                    S.adj[i * kAdjStride + jb] = row;
-            }
-        }
         if (nw == 1) {
-            // up to 32 particles: lane i keeps row i in a register, and a BFS
-            // step is one OR-reduction of the frontier's rows
-            unsigned todo = __ballot_sync(kFull, row1 != 0u);
-            while (todo) {
-                const int s = __ffs(todo) - 1;
-                unsigned comp = 1u << s, front = comp;
-                for (int step = 0; step < 32; ++step) {   // every step adds a vertex
-                    const unsigned nxt =
-                        __reduce_or_sync(kFull, ((front >> lane) & 1u) ? row1 : 0u) & ~comp;
-                    if (!nxt)
-                        break;
-                    comp |= nxt;
-                    front = nxt;
-                }
-                todo &= ~comp;
-                if (((comp >> lane) & 1u) && lane != s)
-                    parent[c0 + lane] = c0 + s;
-            }
+            const float4 pi = lane < m ? S.P[lane] : far_point(-kFar);
+            const int jn8 = (m + 7) & ~7;
+            unsigned rows[1][1];
+            rows[0][0] = (b.nc >= 3 ? block_word<false>(pi, S.P, jn8, b) : block_word<true>(pi, S.P, jn8, b)) &
+                         ~(1u << lane);
+            trace_components<1>(rows, parent, c0, lane);
             __syncwarp();                      // smem reused by the next cell
             continue;
         }
+        // 32 to a block, in z order: blocks too far apart hold no link (every
+        // pair's float32 separation squared exceeds t_hi; rounding is monotone)
+        float zlo = 0.f, zhi = 0.f;            // lane r: the z range of block r
+        for (int r = 0; r < nw; ++r) {
+            const unsigned z = __float_as_uint(S.P[r * 32 + lane].z + 0.f);    // finite and >= 0: ordered bits
+            const bool in = r * 32 + lane < m;
+            const unsigned lo = __reduce_min_sync(kFull, in ? z : 0x7f800000u),
+                           hi = __reduce_max_sync(kFull, in ? z : 0u);
+            zlo = lane == r ? __uint_as_float(lo) : zlo;
+            zhi = lane == r ? __uint_as_float(hi) : zhi;
+        }
+        for (int ib = 0; ib < nw; ++ib)
+            for (int jb = ib; jb < nw; ++jb) {
+                const float gap = __fsub_rn(__shfl_sync(kFull, zlo, jb), __shfl_sync(kFull, zhi, ib));
+                adjacency_block<TeamWarpSmem::kStride>(
+                    S.P, S.adj, m, ib, jb, b.nc >= 3 && gap > 0.f && __fmul_rn(gap, gap) > b.t_hi, lane, b);
+            }
         __syncwarp();
-
-        // lane w < nw holds word w of each vertex set
-        unsigned todo = 0;
-        for (int ib = 0; ib < nw; ++ib) {
-            const int v = ib * 32 + lane;
-            unsigned any = 0;
-            if (v < m)
-                for (int k = 0; k < nw; ++k)
-                    any |= S.adj[v * kAdjStride + k];
-            const unsigned w = __ballot_sync(kFull, any != 0);
-            todo = lane == ib ? w : todo;
-        }
-        for (;;) {
-            const unsigned nz = __ballot_sync(kFull, todo != 0);
-            if (!nz)
-                break;
-            const int w0 = __ffs(nz) - 1;
-            const int s = w0 * 32 + __ffs(__shfl_sync(kFull, todo, w0)) - 1;
-            unsigned comp = lane == w0 ? 1u << (s & 31) : 0u;
-            unsigned front = comp;
-            for (int step = 0; step < kTeamMax; ++step) {   // every step adds a vertex
-                unsigned acc[kTeamWords];
-#pragma unroll
-                for (int k = 0; k < kTeamWords; ++k)
-                    acc[k] = 0;
-                for (int w = 0; w < nw; ++w) {
-                    const unsigned fw = __shfl_sync(kFull, front, w);
-                    if ((fw >> lane) & 1u) {
-                        const unsigned* r = &S.adj[(w * 32 + lane) * kAdjStride];
-#pragma unroll
-                        for (int k = 0; k < kTeamWords; ++k)
-                            if (k < nw) acc[k] |= r[k];
-                    }
-                }
-                unsigned nxt = 0;
-#pragma unroll
-                for (int k = 0; k < kTeamWords; ++k)
-                    if (k < nw) {
-                        const unsigned r = __reduce_or_sync(kFull, acc[k]);
-                        nxt = lane == k ? r : nxt;
-                    }
-                nxt &= ~comp;
-                comp |= nxt;
-                front = nxt;
-                if (!__ballot_sync(kFull, nxt != 0))
-                    break;
-            }
-            todo &= ~comp;
-            for (int w = 0; w < nw; ++w) {
-                const unsigned cw = __shfl_sync(kFull, comp, w);
-                if ((cw >> lane) & 1u)
-                    parent[c0 + w * 32 + lane] = c0 + s;
-            }
-        }
+        if (nw == 2)
+            trace_staged<2>(S, parent, c0, lane);
+        else if (nw == 3)
+            trace_staged<3>(S, parent, c0, lane);
+        else
+            trace_staged<4>(S, parent, c0, lane);
         __syncwarp();                          // smem reused by the next cell
     }
+    cp_async_wait_all();
 }
 
 }  // namespace
@@ -888,28 +1002,12 @@ cudaError_t launch_team_self(const Geometry& g, const Work& w, cudaStream_t s)
 {
     if (g.total_n == 0)
         return cudaSuccess;
-    // the shared-memory opt-in is per device; setting it again is harmless
-    static bool configured[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64 || !configured[dev]) {
-        e = cudaFuncSetAttribute(k_team_self<0, kTeamSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)team_smem_bytes<kTeamSplit>());
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(k_team_self<kTeamSplit, kTeamSelfMax>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)team_smem_bytes<kTeamSelfMax>());
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) configured[dev] = true;
-    }
-    k_team_self<0, kTeamSplit><<<sm_count() * team_blocks<kTeamSplit>(), kTeamWarps * 32,
-                                 team_smem_bytes<kTeamSplit>(), s>>>(
-        g, w.team_list, w.n_team, 0, w.sorted, w.parent, w.minorig, &w.status->err);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_team_self<kTeamSplit, kTeamSelfMax><<<sm_count() * team_blocks<kTeamSelfMax>(), kTeamWarps * 32,
-                                            team_smem_bytes<kTeamSelfMax>(), s>>>(
-        g, w.team_list, w.n_team_hi, w.team_cap, w.sorted, w.parent, w.minorig, &w.status->err);
+    // no more CTAs than warps with a cell
+    int64_t blocks = w.team_cap / kTeamWarps + 1;
+    const int64_t most = (int64_t)sm_count() * kTeamBlocks;
+    if (blocks > most) blocks = most;
+    k_team_self<<<(unsigned)blocks, kTeamWarps * 32, sizeof(TeamSmem), s>>>(g, w.team_list, w.team_cap, w.n_team,
+                                                                           w.n_team_hi, w.sorted, w.parent, w.minorig);
     return cudaGetLastError();
 }
 

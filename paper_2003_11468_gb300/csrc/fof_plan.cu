@@ -51,7 +51,6 @@ const char* kPhaseNames[kNumPhases] = {
 int phase_launches(int ph, int64_t total_n)
 {
     switch (ph) {
-    case kPhTeamSelf: return 2;
     case kPhDenseSelf:
     case kPhDensePairs: return dense_one_launch(total_n) ? 1 : 2;
     case kPhCatalogue: return total_n <= kDirectMax ? 1 : 3;
@@ -261,6 +260,13 @@ int setup_box(double L, double l_x, int64_t n, const fof_options* o, BoxDev& b)
         double rb = l_x * (1.0 + std::ldexp(1.0, -50)) + 8.0 * L * std::ldexp(1.0, -24);
         b.bb_reach2 = float_up(rb * rb * (1.0 + std::ldexp(1.0, -20)));
     }
+    // z bins, 32 per cell.  The bin number (int)fl32(z * inv_zb) - 32 cz is
+    // within nc 32 2^-23 <= 2^-6 bins of exact, and so is the cell's edge, where
+    // numbers are clamped; so members of one bin, or of a bin and a later one,
+    // satisfy z' > z - (1 + 2^-4) L / (32 nc).  The width is taken 1/8 larger,
+    // which also covers the rounding of the subtraction (below L 2^-24).
+    b.inv_zb = (float)(32.0 * (double)b.nc / L);
+    b.zb_width = float_up(1.125 * L / (32.0 * (double)b.nc));
     b.xmax = (float)L;
     while ((double)b.xmax >= L) b.xmax = std::nextafter(b.xmax, 0.0f);
 
