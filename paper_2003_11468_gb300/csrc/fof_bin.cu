@@ -15,6 +15,8 @@
 // writes stay in L2: the brick count is small enough that every brick's
 // write head is L2-resident, which turns the random-order scatter into
 // full-sector DRAM writes.
+#include <cooperative_groups.h>
+
 #include "fof_internal.cuh"
 
 namespace fofgpu {
@@ -237,41 +239,15 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* smem_warp, int& 
     return warp_off + x - v;
 }
 
-// The same for 64-bit words (fields that never carry into each other).
-__device__ __forceinline__ unsigned long long block_exclusive_scan64(unsigned long long v,
-                                                                     unsigned long long* smem_warp,
-                                                                     unsigned long long& total)
-{
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    unsigned long long x = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long y = __shfl_up_sync(kFull, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) smem_warp[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        const int nw = blockDim.x >> 5;
-        unsigned long long t = lane < nw ? smem_warp[lane] : 0ull;
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(kFull, t, o);
-            if (lane >= o) t += y;
-        }
-        if (lane < nw) smem_warp[lane] = t;
-    }
-    __syncthreads();
-    const unsigned long long warp_off = wid ? smem_warp[wid - 1] : 0ull;
-    total = smem_warp[(blockDim.x >> 5) - 1];
-    __syncthreads();
-    return warp_off + x - v;
-}
-
 // out[i] for i in [0, len]: out[len] is the grand total (a virtual zero is
 // appended to the input, so the scan covers len + 1 entries).  The counts lie
 // `pad` words apart.
+// `heavy` (or null): entries above heavy_from are listed there.
 __global__ void __launch_bounds__(kScanThreads) k_scan(const int* __restrict__ in, int pad, int* __restrict__ out,
                                                        int64_t len, unsigned long long* __restrict__ state,
-                                                       int* __restrict__ ticket, int* __restrict__ err)
+                                                       int* __restrict__ ticket, int heavy_from,
+                                                       int* __restrict__ heavy, int* __restrict__ n_heavy,
+                                                       int* __restrict__ err)
 {
     __shared__ int sw[32];
     __shared__ int s_tile, s_before;
@@ -286,8 +262,11 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const int* __restrict__ i
     for (int k = 0; k < kScanItems; ++k)
         v[k] = base + k < len ? in[(base + k) * pad] : 0;
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k)
+    for (int k = 0; k < kScanItems; ++k) {
         s += v[k];
+        if (heavy && v[k] > heavy_from)
+            heavy[atomicAdd(n_heavy, 1)] = (int)(base + k);
+    }
     int total;
     int ex = block_exclusive_scan(s, sw, total);
     if (threadIdx.x < kWarp) {
@@ -308,131 +287,470 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const int* __restrict__ i
 // per-brick cell sort
 // ------------------------------------------------------------------------
 
-constexpr int kSortThreads = 1024;
 constexpr int kMaxR3 = 4096;   // r <= 16
 
-__global__ void __launch_bounds__(kSortThreads) k_brick_sort(Geometry g, const float4* __restrict__ tmp,
-                                                             const int* __restrict__ bstart,
-                                                             float4* __restrict__ sorted,
-                                                             int* __restrict__ parent,
-                                                             int* __restrict__ minorig,
-                                                             int* __restrict__ cnt,
-                                                             int* __restrict__ cell_start,
-                                                             int* __restrict__ err,
-                                                             int64_t* __restrict__ dense_list,
-                                                             int* __restrict__ n_dense,
-                                                             int dense_min,
-                                                             int64_t* __restrict__ team_list,
-                                                             int* __restrict__ n_team,
-                                                             int* __restrict__ n_team_hi,
-                                                             int64_t team_cap,
-                                                             int64_t* __restrict__ big_list,
-                                                             int* __restrict__ n_big)
+struct CellLists {
+    int64_t* list[4];          // dense cells, team cells (small), big cells, team cells (from the back end)
+    int* n[4];
+    int64_t team_cap;
+};
+
+// which list a cell of h particles belongs to: 0 dense, 1 small team, 2 big,
+// 3 large team, -1 none
+__device__ __forceinline__ int cell_list(int h, const BoxDev& b, int dense_min)
 {
-    __shared__ int hist[kMaxR3];
-    __shared__ int sw[32];
-    __shared__ unsigned long long sw64[32];
-    __shared__ int list_base[4];
-    for (int64_t gb = blockIdx.x; gb < g.total_bricks; gb += gridDim.x) {
-        const int bi = box_of(g.box_brick0, g.nbox, gb);
-        const BoxDev& b = g.boxes[bi];
-        const int r3 = b.r * b.r * b.r;
-        const int m = b.r - 1;
-        const int s0 = bstart[gb], s1 = bstart[gb + 1];
-        for (int c = threadIdx.x; c < r3; c += blockDim.x) hist[c] = 0;
-        __syncthreads();
-        for (int k = s0 + threadIdx.x; k < s1; k += blockDim.x) {
-            float4 p = tmp[k];
-            int lc = local_code(cell_coord(p.x, b) & m, cell_coord(p.y, b) & m, cell_coord(p.z, b) & m);
-            atomicAdd(hist + lc, 1);
-        }
-        __syncthreads();
-        // exclusive scan of hist[0..r3): each thread owns a contiguous run
-        const int per = (r3 + blockDim.x - 1) / blockDim.x;
-        const int c0 = threadIdx.x * per;
-        int run = 0;
-        for (int c = c0; c < c0 + per && c < r3; ++c) run += hist[c];
-        int total;
-        int ex = block_exclusive_scan(run, sw, total);
-        const int ex0 = ex;
-        const int64_t cbase = b.cell0 + (gb - b.brick0) * (int64_t)r3;
-        int nd = 0, nt = 0, nth = 0, nbg = 0;   // this thread's dense, team (small, large) and big cells
-        for (int c = c0; c < c0 + per && c < r3; ++c) {
-            const int h = hist[c];
-            ex += h;
-            if (is_big(h, b))
-                ++nbg;
-            else if (is_sub(h, b, dense_min))
-                ++nd;
-            else if (h >= b.team_min && h <= kTeamSplit)
-                ++nt;
-            else if (h >= b.team_min && h <= kTeamSelfMax)
-                ++nth;
-        }
-        // list slots: one reservation per brick (a shared counter per cell
-        // would serialise millions of atomics on one address).  The four
-        // counts (each at most kMaxR3 per brick) share one scan as 16-bit
-        // fields of a 64-bit word.
-        unsigned long long tot4;
-        const unsigned long long o4 = block_exclusive_scan64(
-            (unsigned long long)nd | ((unsigned long long)nt << 16) | ((unsigned long long)nth << 32) |
-                ((unsigned long long)nbg << 48),
-            sw64, tot4);
-        const int nd_tot = (int)(tot4 & 0xffffu), nt_tot = (int)((tot4 >> 16) & 0xffffu);
-        const int nth_tot = (int)((tot4 >> 32) & 0xffffu), nb_tot = (int)(tot4 >> 48);
-        int od = (int)(o4 & 0xffffu), ot = (int)((o4 >> 16) & 0xffffu);
-        int oth = (int)((o4 >> 32) & 0xffffu), obg = (int)(o4 >> 48);
-        if (threadIdx.x == 0) {
-            list_base[0] = nd_tot ? atomicAdd(n_dense, nd_tot) : 0;
-            list_base[1] = nt_tot ? atomicAdd(n_team, nt_tot) : 0;
-            list_base[2] = nb_tot ? atomicAdd(n_big, nb_tot) : 0;
-            list_base[3] = nth_tot ? atomicAdd(n_team_hi, nth_tot) : 0;
-        }
-        __syncthreads();
-        od += list_base[0];
-        ot += list_base[1];
-        obg += list_base[2];
-        oth += list_base[3];
-        ex = ex0;
-        for (int c = c0; c < c0 + per && c < r3; ++c) {
-            const int h = hist[c];
-            const int start = s0 + ex;
-            hist[c] = ex;                       // becomes the cursor
-            ex += h;
-            if (is_big(h, b))
-                big_list[obg++] = cbase + c;
-            else if (is_sub(h, b, dense_min))
-                dense_list[od++] = cbase + c;
-            else if (h >= b.team_min && h <= kTeamSplit)
-                team_list[ot++] = ((int64_t)h << 32) | (uint32_t)start;
-            else if (h >= b.team_min && h <= kTeamSelfMax)
-                team_list[team_cap - 1 - oth++] = ((int64_t)h << 32) | (uint32_t)start;
-        }
-        __syncthreads();
-        for (int k = s0 + threadIdx.x; k < s1; k += blockDim.x) {
-            float4 p = tmp[k];
-            int lc = local_code(cell_coord(p.x, b) & m, cell_coord(p.y, b) & m, cell_coord(p.z, b) & m);
-            int slot = s0 + atomicAdd(hist + lc, 1);
-            if (slot >= s1) {
-                atomicOr(err, kErrInternal);
-                continue;
+    if (is_big(h, b))
+        return 2;
+    if (is_sub(h, b, dense_min))
+        return 0;
+    if (h < b.team_min || h > kTeamSelfMax)
+        return -1;
+    return h <= kTeamSplit ? 1 : 3;
+}
+
+__device__ __forceinline__ int* list_counter(const CellLists& L, int l)
+{
+    return l == 0 ? L.n[0] : (l == 1 ? L.n[1] : (l == 2 ? L.n[2] : L.n[3]));
+}
+
+// A brick's listed cells are counted as four 16-bit fields of one word (at most
+// kMaxR3 cells per brick).
+__device__ __forceinline__ unsigned long long list_one(int l)
+{
+    return l < 0 ? 0ull : 1ull << (16 * l);
+}
+
+// The cell `key` of h particles from slot `start` on, as entry `at` (past the
+// brick's base) of its list.
+__device__ __forceinline__ void list_cell(const CellLists& L, const int* list_base, int l, int at, int h, int64_t key,
+                                          int start)
+{
+    const int64_t pos = list_base[l] + at;
+    if (l == 0)
+        L.list[0][pos] = key;
+    else if (l == 2)
+        L.list[2][pos] = key;
+    else
+        L.list[1][l == 1 ? pos : L.team_cap - 1 - pos] = ((int64_t)h << 32) | (uint32_t)start;
+}
+
+// What the cell code of a particle inside its brick needs of its box (in
+// registers: the box table would be read again after every store).
+struct CodeGeo {
+    float inv_hf;
+    int nf, q, rmask;
+    uint32_t magic_q;
+};
+
+__device__ __forceinline__ CodeGeo code_geo(const BoxDev& b)
+{
+    return CodeGeo{b.inv_hf, b.nf, b.q, b.r - 1, b.magic_q};
+}
+
+__device__ __forceinline__ int code_axis(float x, const CodeGeo& c)
+{
+    int g = (int)__fmul_rn(x, c.inv_hf);       // cell_coord
+    g = min(max(g, 0), c.nf - 1);
+    return (c.q == 1 ? g : (int)__umulhi((unsigned)g, c.magic_q)) & c.rmask;
+}
+
+__device__ __forceinline__ int code_of(const float4& p, const CodeGeo& c)
+{
+    return (int)local_code(code_axis(p.x, c), code_axis(p.y, c), code_axis(p.z, c));
+}
+
+// One CTA per brick of up to heavy_from particles.  A mean brick has 1,200
+// particles in 4,096 cells, most of them empty, and what bounds it is the
+// chain: load, histogram, scan, cursors, scatter.  So
+//   * the next brick's records are copied ahead into shared memory (cp.async;
+//     each thread reads back only its own copies) while this one is sorted;
+//   * counts and cursors are 16-bit halves of shared-memory words, eight cells
+//     to a load, so two histograms fit and take turns (the one not in use is
+//     cleared meanwhile) and a brick takes three barriers;
+//   * the lists are looked at only in bricks that hold a cell for one, and
+//     their reservations return while the scatter runs.
+// Warp w owns the cells of per_warp consecutive groups of eight, lane by lane,
+// so the histogram is read and written conflict-free; a lane's groups share one
+// warp scan as 16-bit fields.  Registers are what limits the copies and loads
+// in flight: a spill here costs 10 to 50%, because the scattered stores leave
+// little of L1.  Both sort kernels, before (1,024 threads, 32-bit counts, twelve
+// barriers) and after, us: 64 boxes of 36,000 particles 205 and 116, 16.8
+// million (256^3) 575 and 422, 512 boxes of 650,000 12850 and 8700, 453 million
+// (768^3) 12200 and 10900.
+constexpr int kSortThreads = 256;
+constexpr int kSortWarps = kSortThreads / 32;
+constexpr int kSortBlocks = 4;
+constexpr int kSortKeep = 3;                           // records of a brick copied ahead per thread
+constexpr int kFlight = 2;                             // loads in flight per thread beyond them
+constexpr int kSortGroups = kMaxR3 / (8 * kSortThreads);   // groups of eight cells per lane
+static_assert(kSortGroups <= 4 && kBrickMax < 65536, "16-bit counts, four fields");
+
+struct SortSmem {
+    float4 rec[2][kSortKeep * kSortThreads];
+    unsigned hist[2][kMaxR3 / 2];
+    int part[kSortWarps];
+    unsigned long long list_pack;
+    int list_base[4];
+};
+
+// +1 on cell c's 16-bit half; returns its value before
+__device__ __forceinline__ int bump(unsigned* hist, int c)
+{
+    const int sh = (c & 1) * 16;
+    return (int)((atomicAdd(hist + (c >> 1), 1u << sh) >> sh) & 0xffffu);
+}
+
+__device__ __forceinline__ int half_of(const unsigned* hist, int c)
+{
+    return (int)((hist[c >> 1] >> ((c & 1) * 16)) & 0xffffu);
+}
+
+__global__ void __launch_bounds__(kSortThreads, kSortBlocks)
+    k_brick_sort(Geometry g, const float4* __restrict__ tmp, const int* __restrict__ bstart,
+                 float4* __restrict__ sorted, int* __restrict__ parent, int* __restrict__ minorig,
+                 int* __restrict__ cnt, int* __restrict__ cell_start, int dense_min, CellLists lists,
+                 int heavy_from, int* __restrict__ err)
+{
+    extern __shared__ float4 sort_raw[];
+    SortSmem& S = *reinterpret_cast<SortSmem*>(sort_raw);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    for (int c = tid; c < kMaxR3; c += kSortThreads) S.hist[0][c] = 0u;     // both
+    if (tid == 0)
+        S.list_pack = 0ull;
+    __syncthreads();
+    const int64_t nb = g.total_bricks, stride = gridDim.x;
+    auto fetch = [&](int s0, int s1, int buf) {                // one commit group
+        if (s1 - s0 <= heavy_from) {
+#pragma unroll
+            for (int i = 0; i < kSortKeep; ++i) {
+                const int k = i * kSortThreads + tid;
+                if (s0 + k < s1)
+                    cp_async16(&S.rec[buf][k], tmp + s0 + k);
             }
-            sorted[slot] = p;
-            minorig[slot] = __float_as_int(p.w);
         }
-        for (int k = s0 + threadIdx.x; k < s1; k += blockDim.x) {
+        cp_async_commit();
+    };
+    int64_t gb = blockIdx.x;
+    int s0 = 0, s1 = 0, n0 = 0, n1 = 0;                        // this brick's and the next one's slots
+    if (gb < nb) {
+        s0 = bstart[gb];
+        s1 = bstart[gb + 1];
+    }
+    if (gb + stride < nb) {
+        n0 = bstart[gb + stride];
+        n1 = bstart[gb + stride + 1];
+    }
+    fetch(s0, s1, 0);
+    int bi = 0, buf = 0, hb = 0;               // record buffer and histogram of this brick
+    for (; gb < nb; gb += stride, buf ^= 1) {
+        cp_async_wait_all();
+        fetch(n0, n1, buf ^ 1);                // each thread read its own copies there one brick ago
+        const int a0 = s0, a1 = s1;
+        s0 = n0;
+        s1 = n1;
+        if (gb + 2 * stride < nb) {
+            n0 = bstart[gb + 2 * stride];
+            n1 = bstart[gb + 2 * stride + 1];
+        } else {
+            n0 = n1 = 0;
+        }
+        const float4* rec = S.rec[buf];
+        unsigned* hist = S.hist[hb];
+        if (a1 - a0 > heavy_from)
+            continue;                          // k_brick_sort_heavy's (block-uniform)
+        while (bi + 1 < g.nbox && g.box_brick0[bi + 1] <= gb) ++bi;
+        const BoxDev& b = g.boxes[bi];
+        const CodeGeo cg = code_geo(b);
+        const int n = a1 - a0, r3 = (cg.rmask + 1) * (cg.rmask + 1) * (cg.rmask + 1);
+        int code[kSortKeep];
+#pragma unroll
+        for (int i = 0; i < kSortKeep; ++i) {
+            const int k = i * kSortThreads + tid;
+            if (k < n) {
+                code[i] = code_of(rec[k], cg);
+                bump(hist, code[i]);
+            }
+        }
+        for (int kb = kSortKeep * kSortThreads + tid; kb < n; kb += kFlight * kSortThreads) {
+            float4 v[kFlight];
+#pragma unroll
+            for (int i = 0; i < kFlight; ++i)
+                if (kb + i * kSortThreads < n)
+                    v[i] = tmp[a0 + kb + i * kSortThreads];
+#pragma unroll
+            for (int i = 0; i < kFlight; ++i)
+                if (kb + i * kSortThreads < n)
+                    bump(hist, code_of(v[i], cg));
+        }
+        __syncthreads();
+        // the other histogram was last used by the previous brick, which every
+        // thread has finished: cleared for the next one
+        for (int q = tid; q < kMaxR3 / 8; q += kSortThreads)
+            reinterpret_cast<uint4*>(S.hist[hb ^ 1])[q] = make_uint4(0u, 0u, 0u, 0u);
+        hb ^= 1;
+        const int octs = (r3 + 7) / 8, per_warp = (octs + kSortWarps - 1) / kSortWarps;
+        const int q0 = wid * per_warp, q1 = min(q0 + per_warp, octs);
+        const int listed_from = min(min(b.team_min, dense_min), kDenseMax + 1);
+        unsigned long long sums = 0ull;        // 16-bit field i: particles of this lane's group i
+        unsigned most = 0u;                    // largest count, in either half
+#pragma unroll
+        for (int i = 0; i < kSortGroups; ++i) {
+            const int q = q0 + i * 32 + lane;
+            const uint4 h = q < q1 ? reinterpret_cast<const uint4*>(hist)[q] : make_uint4(0u, 0u, 0u, 0u);
+            const unsigned t = h.x + h.y + h.z + h.w;                  // halves add up without a carry
+            sums |= (unsigned long long)((t & 0xffffu) + (t >> 16)) << (16 * i);
+            most = __vmaxu2(most, __vmaxu2(__vmaxu2(h.x, h.y), __vmaxu2(h.z, h.w)));
+        }
+        unsigned long long inc = sums;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += y;
+        }
+        const unsigned long long all = __shfl_sync(kFull, inc, 31);
+        if (lane == 0)
+            S.part[wid] = (int)((all & 0xffffu) + ((all >> 16) & 0xffffu) + ((all >> 32) & 0xffffu) + (all >> 48));
+        const bool listed = __syncthreads_or((int)max(most & 0xffffu, most >> 16) >= listed_from);
+        const int64_t cbase = b.cell0 + (gb - b.brick0) * (int64_t)r3;
+        unsigned full = 0u;                    // this lane's groups with a listed cell
+        unsigned long long list_at = 0ull;     // this thread's entries of each list start there
+        {
+            // particles in the groups before
+            int base = (int)__reduce_add_sync(kFull, lane < wid ? (unsigned)S.part[lane] : 0u);
+            unsigned long long mine = 0ull;    // listed cells of this thread
+            unsigned long long before = inc - sums;
+#pragma unroll 1
+            for (int i = 0; i < kSortGroups; ++i) {
+                const int q = q0 + i * 32 + lane;
+                if (q < q1) {
+                    uint4* cells = reinterpret_cast<uint4*>(hist) + q;
+                    const uint4 h = *cells;
+                    int x = base + (int)(before & 0xffffu);
+                    // a half-word pair of counts becomes the pair of its cursors
+                    auto cursors = [&](unsigned w) {
+                        const int lo = x, hi = x + (int)(w & 0xffffu);
+                        x = hi + (int)(w >> 16);
+                        return make_int2(lo, hi);
+                    };
+                    const int2 p0 = cursors(h.x), p1 = cursors(h.y), p2 = cursors(h.z), p3 = cursors(h.w);
+                    *cells = make_uint4((unsigned)(p0.x | (p0.y << 16)), (unsigned)(p1.x | (p1.y << 16)),
+                                        (unsigned)(p2.x | (p2.y << 16)), (unsigned)(p3.x | (p3.y << 16)));
+                    int* out = cell_start + cbase + 8 * q;
+                    if (8 * q + 8 <= r3 && (cbase & 3) == 0) {
+                        reinterpret_cast<int4*>(out)[0] = make_int4(a0 + p0.x, a0 + p0.y, a0 + p1.x, a0 + p1.y);
+                        reinterpret_cast<int4*>(out)[1] = make_int4(a0 + p2.x, a0 + p2.y, a0 + p3.x, a0 + p3.y);
+                    } else {                   // bricks of fewer than 8 cells, or after one
+                        for (int u = 0; u < 8 && 8 * q + u < r3; ++u) out[u] = a0 + half_of(hist, 8 * q + u);
+                    }
+                    const unsigned top = __vmaxu2(__vmaxu2(h.x, h.y), __vmaxu2(h.z, h.w));
+                    if ((int)max(top & 0xffffu, top >> 16) >= listed_from) {
+                        full |= 1u << i;
+                        auto listed_pair = [&](unsigned w) {
+                            mine += list_one(cell_list((int)(w & 0xffffu), b, dense_min)) +
+                                    list_one(cell_list((int)(w >> 16), b, dense_min));
+                        };
+                        listed_pair(h.x);
+                        listed_pair(h.y);
+                        listed_pair(h.z);
+                        listed_pair(h.w);
+                    }
+                }
+                base += (int)((all >> (16 * i)) & 0xffffu);
+                before >>= 16;
+            }
+            // the end of the last cell (the next brick writes the same value)
+            if (tid == 0)
+                cell_start[cbase + r3] = a1;
+            if (mine)
+                list_at = atomicAdd(&S.list_pack, mine);
+        }
+        __syncthreads();
+        // one reservation per list and brick (a shared counter per cell would
+        // serialise millions of atomics on one address); it returns meanwhile
+        int reserved = 0;
+        if (listed && tid < 4) {
+            const int cells = (int)((S.list_pack >> (16 * tid)) & 0xffffu);
+            if (cells)
+                reserved = atomicAdd(list_counter(lists, tid), cells);
+        }
+#pragma unroll
+        for (int i = 0; i < kSortKeep; ++i) {
+            const int k = i * kSortThreads + tid;
+            if (k < n) {
+                const float4 v = rec[k];
+                const int slot = a0 + bump(hist, code[i]);
+                sorted[slot] = v;
+                minorig[slot] = __float_as_int(v.w);
+            }
+        }
+        for (int kb = kSortKeep * kSortThreads + tid; kb < n; kb += kFlight * kSortThreads) {
+            float4 v[kFlight];
+#pragma unroll
+            for (int i = 0; i < kFlight; ++i)
+                if (kb + i * kSortThreads < n)
+                    v[i] = tmp[a0 + kb + i * kSortThreads];
+#pragma unroll
+            for (int i = 0; i < kFlight; ++i)
+                if (kb + i * kSortThreads < n) {
+                    const int slot = a0 + bump(hist, code_of(v[i], cg));
+                    if (slot < a1) {
+                        sorted[slot] = v[i];
+                        minorig[slot] = __float_as_int(v[i].w);
+                    } else {
+                        atomicOr(err, kErrInternal);
+                    }
+                }
+        }
+        for (int k = a0 + tid; k < a1; k += kSortThreads) {
             parent[k] = k;
             cnt[k] = 1;
         }
-        // the cursors now hold each cell's end: the cell starts, written
-        // coalesced (cell c + 1 starts where c ends; the next brick writes
-        // the same value at its first cell)
+        if (listed) {
+            if (tid < 4)
+                S.list_base[tid] = reserved;
+            __syncthreads();
+            if (tid == 0)
+                S.list_pack = 0ull;
+            // the cursors now hold each cell's end
+            for (; full; full &= full - 1u) {
+                const int c0 = 8 * (q0 + (__ffs(full) - 1) * 32 + lane);
+                int start = c0 ? half_of(hist, c0 - 1) : 0;
+                for (int c = c0; c < c0 + 8; ++c) {
+                    const int end = half_of(hist, c), size = end - start;
+                    const int l = c < r3 ? cell_list(size, b, dense_min) : -1;
+                    if (l >= 0) {
+                        list_cell(lists, S.list_base, l, (int)((list_at >> (16 * l)) & 0xffffu), size, cbase + c,
+                                  a0 + start);
+                        list_at += list_one(l);
+                    }
+                    start = end;
+                }
+            }
+        }
+    }
+    cp_async_wait_all();
+}
+
+// Bricks above kHeavyBrick particles: a cluster of CTAs per brick, each CTA
+// with its share of the particles and its own histogram; CTA r also owns an
+// equal share of the cells, whose counts it sums over the cluster through
+// distributed shared memory and turns into every CTA's cursors.  One CTA of
+// 1,024 threads took 570 us for the fullest brick of the 256^3 box (350,000
+// particles); the 150 bricks above kHeavyBrick together take 155 us here (260
+// with 1,024 threads per CTA, of which fewer clusters run at a time).
+constexpr int kCluster = 8;
+constexpr int kHeavyThreads = 512;
+constexpr int kHeavyBlocks = 2;
+constexpr int kHeavyFlight = 4;                 // loads in flight per thread
+static_assert(kMaxR3 / kCluster <= kHeavyThreads, "one cell per thread");
+
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kHeavyThreads, kHeavyBlocks)
+    k_brick_sort_heavy(Geometry g, const float4* __restrict__ tmp, const int* __restrict__ bstart,
+                       const int* __restrict__ heavy, const int* __restrict__ n_heavy, float4* __restrict__ sorted,
+                       int* __restrict__ parent, int* __restrict__ minorig, int* __restrict__ cnt,
+                       int* __restrict__ cell_start, int dense_min, CellLists lists, int* __restrict__ err)
+{
+    namespace cg = cooperative_groups;
+    __shared__ int hist[kMaxR3];
+    __shared__ int part[kWarp];
+    __shared__ unsigned long long list_pack;
+    __shared__ int list_base[4];
+    __shared__ int cells_total;                    // particles in this CTA's cells
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    const int n = *n_heavy;
+    for (int it = blockIdx.x / kCluster; it < n; it += gridDim.x / kCluster) {
+        const int64_t gb = heavy[it];
+        const int s0 = bstart[gb], s1 = bstart[gb + 1];
+        const BoxDev& b = g.boxes[box_of(g.box_brick0, g.nbox, gb)];
+        const CodeGeo geo = code_geo(b);
+        const int r3 = b.r * b.r * b.r;
+        for (int c = threadIdx.x; c < r3; c += kHeavyThreads) hist[c] = 0;
         __syncthreads();
-        for (int c = threadIdx.x; c < r3; c += blockDim.x)
-            cell_start[cbase + c + 1] = s0 + hist[c];
+        // this CTA's particles
+        const int share = (s1 - s0 + kCluster - 1) / kCluster;
+        const int k0 = s0 + rank * share, k1 = min(k0 + share, s1);
+        for (int kb = k0 + threadIdx.x; kb < k1; kb += kHeavyFlight * kHeavyThreads) {
+            float4 v[kHeavyFlight];
+#pragma unroll
+            for (int i = 0; i < kHeavyFlight; ++i)
+                if (kb + i * kHeavyThreads < k1)
+                    v[i] = tmp[kb + i * kHeavyThreads];
+#pragma unroll
+            for (int i = 0; i < kHeavyFlight; ++i)
+                if (kb + i * kHeavyThreads < k1)
+                    atomicAdd(hist + code_of(v[i], geo), 1);
+        }
+        cluster.sync();
+        // this CTA's cells, one per thread: the cluster's counts and each
+        // CTA's offset in the cell
+        const int own = (r3 + kCluster - 1) / kCluster;
+        const int c = rank * own + threadIdx.x;
+        const bool mine = (int)threadIdx.x < own && c < r3;
+        int before[kCluster], h = 0;
+#pragma unroll
+        for (int q = 0; q < kCluster; ++q) {
+            before[q] = h;
+            if (mine)
+                h += *cluster.map_shared_rank(hist + c, q);
+        }
         if (threadIdx.x == 0)
-            cell_start[cbase] = s0;
+            list_pack = 0ull;
+        int total;
+        const int ex = block_exclusive_scan(h, part, total);
+        const int l = mine ? cell_list(h, b, dense_min) : -1;
+        unsigned long long at = 0ull;
+        if (l >= 0)
+            at = atomicAdd(&list_pack, list_one(l));
+        if (threadIdx.x == 0)
+            cells_total = total;
+        cluster.sync();
+        int start = s0 + ex;
+        for (int q = 0; q < rank; ++q)
+            start += *cluster.map_shared_rank(&cells_total, q);
+        const int64_t cbase = b.cell0 + (gb - b.brick0) * (int64_t)r3;
+        if (mine) {
+#pragma unroll
+            for (int q = 0; q < kCluster; ++q)
+                *cluster.map_shared_rank(hist + c, q) = start + before[q];
+            cell_start[cbase + c + 1] = start + h;
+            if (c == 0)
+                cell_start[cbase] = s0;
+        }
+        int reserved = 0;
+        if (threadIdx.x < 4) {
+            const int cells = (int)((list_pack >> (16 * threadIdx.x)) & 0xffffu);
+            if (cells)
+                reserved = atomicAdd(list_counter(lists, threadIdx.x), cells);
+        }
+        cluster.sync();
+        for (int kb = k0 + threadIdx.x; kb < k1; kb += kHeavyFlight * kHeavyThreads) {
+            float4 v[kHeavyFlight];
+#pragma unroll
+            for (int i = 0; i < kHeavyFlight; ++i)
+                if (kb + i * kHeavyThreads < k1)
+                    v[i] = tmp[kb + i * kHeavyThreads];
+#pragma unroll
+            for (int i = 0; i < kHeavyFlight; ++i) {
+                const int k = kb + i * kHeavyThreads;
+                if (k < k1) {
+                    const int slot = atomicAdd(hist + code_of(v[i], geo), 1);
+                    if (slot < s1) {
+                        sorted[slot] = v[i];
+                        minorig[slot] = __float_as_int(v[i].w);
+                    } else {
+                        atomicOr(err, kErrInternal);
+                    }
+                    parent[k] = k;
+                    cnt[k] = 1;
+                }
+            }
+        }
+        // after the last cluster barrier no other CTA touches this one's memory
+        if (threadIdx.x < 4)
+            list_base[threadIdx.x] = reserved;
         __syncthreads();
+        if (l >= 0)
+            list_cell(lists, list_base, l, (int)((at >> (16 * l)) & 0xffffu), h, cbase + c, start);
     }
 }
 
@@ -547,9 +865,10 @@ int64_t scan_tiles(int64_t len)
 }
 
 cudaError_t launch_scan(const int* in, int pad, int* out, int64_t len, unsigned long long* state, int* ticket,
-                        int* err, cudaStream_t s)
+                        int heavy_from, int* heavy, int* n_heavy, int* err, cudaStream_t s)
 {
-    k_scan<<<(unsigned)scan_tiles(len), kScanThreads, 0, s>>>(in, pad, out, len, state, ticket, err);
+    k_scan<<<(unsigned)scan_tiles(len), kScanThreads, 0, s>>>(in, pad, out, len, state, ticket, heavy_from, heavy,
+                                                              n_heavy, err);
     return cudaGetLastError();
 }
 
@@ -568,15 +887,50 @@ cudaError_t launch_brick_sort(const Geometry& g, const Work& w, int dense_min, c
 {
     if (g.total_bricks == 0)
         return cudaSuccess;
+    const CellLists lists = {{w.dense_list, w.team_list, w.big_list, w.team_list},
+                             {w.n_dense, w.n_team, w.n_big, w.n_team_hi},
+                             w.team_cap};
+    if (heavy_bricks(g.total_n)) {
+        int64_t clusters = g.total_n / kHeavyBrick;
+        const int64_t most = (int64_t)sm_count() * kHeavyBlocks / kCluster;
+        if (clusters > most) clusters = most;
+        k_brick_sort_heavy<<<(unsigned)(clusters * kCluster), kHeavyThreads, 0, s>>>(
+            g, w.tmp, w.bstart, w.heavy_list, w.n_heavy, w.sorted, w.parent, w.minorig, w.cnt, w.cell_start,
+            dense_min, lists, &w.status->err);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    // the shared-memory opt-in is per device; setting it again is harmless
+    static bool configured[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64 || !configured[dev]) {
+        e = cudaFuncSetAttribute(k_brick_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem));
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < 64) configured[dev] = true;
+    }
     int64_t blocks = g.total_bricks;
-    int64_t cap = (int64_t)sm_count() * 4 * 16;
+    int64_t cap = (int64_t)sm_count() * kSortBlocks;
     if (blocks > cap) blocks = cap;
-    k_brick_sort<<<(unsigned)blocks, kSortThreads, 0, s>>>(g, w.tmp, w.bstart, w.sorted, w.parent,
-                                                         w.minorig, w.cnt, w.cell_start,
-                                                         &w.status->err, w.dense_list, w.n_dense,
-                                                         dense_min, w.team_list, w.n_team, w.n_team_hi,
-                                                         w.team_cap, w.big_list, w.n_big);
+    k_brick_sort<<<(unsigned)blocks, kSortThreads, sizeof(SortSmem), s>>>(g, w.tmp, w.bstart, w.sorted, w.parent, w.minorig, w.cnt,
+                                                         w.cell_start, dense_min, lists, heavy_from(g.total_n),
+                                                         &w.status->err);
     return cudaGetLastError();
+}
+
+// Bricks above this many particles go to k_brick_sort_heavy: the limit of the
+// 16-bit counts while a plan's particles all fit them (no brick can be above,
+// and the launch is saved), else the size from which one CTA's chain is the
+// longer one.
+int heavy_from(int64_t total_n)
+{
+    return total_n <= kBrickMax ? kBrickMax : kHeavyBrick;
+}
+
+bool heavy_bricks(int64_t total_n)
+{
+    return total_n > kBrickMax;
 }
 
 cudaError_t launch_relink_check(const float* pos, const Geometry& g, const Work& w, int* flags,

@@ -129,6 +129,24 @@ __device__ __forceinline__ int owner_lane(int start, int t)
     return lo;
 }
 
+// 16-byte asynchronous copy global -> shared (cp.async), its commit and
+// the wait for all of the thread's copies
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem)
+{
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
+}
+
+__device__ __forceinline__ void cp_async_commit()
+{
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+__device__ __forceinline__ void cp_async_wait_all()
+{
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 // ------------------------------------------------------------------------
 // box lookup: box index of a concatenated particle / brick index
 // ------------------------------------------------------------------------
@@ -577,6 +595,8 @@ struct Work {
     int* bstart;        // [total_bricks + 1]
     unsigned long long* scan_state; // [scan_tiles] look-back words of the brick scan
     int* scan_ticket;   // scan tiles handed out
+    int* n_heavy;       // bricks above heavy_from particles
+    int* heavy_list;    // [total_n / kHeavyBrick + 1] their indices
     unsigned long long* tile_state; // look-back words of the output tiles, or of the scan of their counts
     int* tile_ticket;   // tiles handed out
     int* out_cursor;    // [n_tiles] fill of each output bucket, then the tile's catalogue entries
@@ -598,6 +618,10 @@ struct Work {
     int64_t team_cap;    // capacity of team_list
 };
 
+// Bricks above this many particles are sorted by a cluster of CTAs (from 4,096
+// on the clusters' own steps take longer: 256^3 box 522 us instead of 410).
+constexpr int kHeavyBrick = 8192;
+constexpr int kBrickMax = 65535;   // particles of a brick that one CTA can sort
 // Bricks whose counters a CTA of the count kernel keeps in shared memory.
 constexpr int kTileBricks = 12288;
 constexpr int kOutTile = 4096;  // inputs per output tile
@@ -609,9 +633,12 @@ int sm_count();
 
 cudaError_t launch_bin_count(const float* pos, const Geometry& g, const Work& w, cudaStream_t s);
 // exclusive prefix sum of in[i * pad], i < len, into out[0..len]; state
-// (scan_tiles(len) words) and ticket start at zero
+// (scan_tiles(len) words) and ticket start at zero; entries above heavy_from
+// are listed in `heavy` unless it is null
 cudaError_t launch_scan(const int* in, int pad, int* out, int64_t len, unsigned long long* state, int* ticket,
-                        int* err, cudaStream_t s);
+                        int heavy_from, int* heavy, int* n_heavy, int* err, cudaStream_t s);
+int heavy_from(int64_t total_n);
+bool heavy_bricks(int64_t total_n);   // whether a brick can be above heavy_from
 int64_t scan_tiles(int64_t len);
 int brick_pad(int64_t bricks);
 cudaError_t launch_bin_scatter(const float* pos, const Geometry& g, const Work& w, cudaStream_t s);

@@ -99,24 +99,6 @@ __device__ __forceinline__ unsigned reach_mask(const float4& p, const BoxDev& b,
     return (hz ? m9 : 0u) | (hy ? xm << 9 : 0u) | (hx << 12);
 }
 
-// 16-byte asynchronous copy global -> shared (cp.async), its commit and
-// the wait for all of the thread's copies
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem)
-{
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
-}
-
-__device__ __forceinline__ void cp_async_commit()
-{
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-__device__ __forceinline__ void cp_async_wait_all()
-{
-    asm volatile("cp.async.wait_all;" ::: "memory");
-}
-
 __device__ __forceinline__ float4 shfl4(float4 v, int src)
 {
     v.x = __shfl_sync(kFull, v.x, src);

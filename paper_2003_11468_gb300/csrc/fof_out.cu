@@ -483,7 +483,7 @@ cudaError_t launch_catalogue(const Geometry& g, const Work& w, int32_t* ids, int
     k_outputs_write<false><<<blocks, kOutThreads, 0, s>>>(g, pairs, ids, sizes, thr, cat, cap, w.tile_state,
                                                           w.tile_ticket, w.out_cursor, w.status);
     cudaError_t e = launch_scan(w.out_cursor, 1, w.tile_off, w.n_tiles, w.tile_state, w.tile_ticket,
-                                &w.status->err, s);
+                                0, nullptr, nullptr, &w.status->err, s);
     if (e != cudaSuccess)
         return e;
     k_catalogue<<<grid_for(w.n_tiles * kOutThreads, kOutThreads, 4), kOutThreads, 0, s>>>(

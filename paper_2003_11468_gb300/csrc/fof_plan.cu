@@ -53,6 +53,7 @@ int phase_launches(int ph, int64_t total_n)
     switch (ph) {
     case kPhDenseSelf:
     case kPhDensePairs: return dense_one_launch(total_n) ? 1 : 2;
+    case kPhBrickSort: return heavy_bricks(total_n) ? 2 : 1;
     case kPhCatalogue: return total_n <= kDirectMax ? 1 : 3;
     default: return 1;
     }
@@ -65,6 +66,7 @@ constexpr double kDefaultOccupancy = 0.30;
 constexpr int kDefaultTeamMin = 10;
 constexpr int kMinTeamMin = 2;                 // smallest team threshold in use
 constexpr int kNumCounters = 4;                 // dense, team (small, large), big cells
+constexpr int kCounterPad = 32;                // words between them: a 128-byte line each
 constexpr int kMaxCellsPerAxis = 4096;        // float32 cell-index precision (unsplit cells)
 constexpr int kMaxFinePerAxis = 16384;        // float32 index precision (sub-cells)
 
@@ -395,7 +397,7 @@ struct fof_plan {
 namespace {
 
 struct Layout {
-    size_t boxes, p0, brick0, results, bcount, bstart, scan_state, scan_ticket, tile_state, tile_ticket, out_cursor, tile_off,
+    size_t boxes, p0, brick0, results, bcount, bstart, scan_state, scan_ticket, heavy_list, tile_state, tile_ticket, out_cursor, tile_off,
         cell_start, tmp, sorted, parent, minorig, cnt, dense_list, counters, dense_root, team_list, big_list, total;
     size_t zero_end;     // [bcount, zero_end) starts each run at zero
     int64_t n_tiles, dense_cap, team_cap;
@@ -418,9 +420,9 @@ Layout layout(int nbox, int64_t total_n, int64_t total_bricks, int64_t total_cel
     // kernels ([bcount, zero_end)), and, for a repeated fof_groups, one of its
     // tail from the counts in the results block on
     L.bcount = take(4 * (size_t)(total_bricks * brick_pad(total_bricks)));
-    L.scan_state = take(8 * (size_t)scan_tiles(total_bricks) + 4);
+    L.scan_state = take(8 * (size_t)scan_tiles(total_bricks) + 8);      // and the ticket and n_heavy
     L.scan_ticket = L.scan_state + 8 * (size_t)scan_tiles(total_bricks);
-    L.counters = take(4 * kNumCounters);
+    L.counters = take(4 * kNumCounters * kCounterPad);
     L.results = take(results_layout(nbox).bytes);
     L.tile_state = take(12 * (size_t)L.n_tiles + 4);
     L.out_cursor = L.tile_state + 8 * (size_t)L.n_tiles;
@@ -439,6 +441,7 @@ Layout layout(int nbox, int64_t total_n, int64_t total_bricks, int64_t total_cel
     L.dense_root = take(4 * (size_t)(total_n / dense_min + 2));
     L.team_cap = total_n / team_min + 1;
     L.team_list = take(8 * (size_t)L.team_cap);
+    L.heavy_list = take(4 * (size_t)(total_n / kHeavyBrick + 1));
     L.big_list = take(8 * (size_t)(total_n / (kDenseMax + 1) + 1));
     L.total = off;
     return L;
@@ -463,6 +466,8 @@ void bind_workspace(char* ws, const Layout& L, int nbox, int64_t tn, int64_t tb,
     w.bstart = (int*)(ws + L.bstart);
     w.scan_state = (unsigned long long*)(ws + L.scan_state);
     w.scan_ticket = (int*)(ws + L.scan_ticket);
+    w.n_heavy = w.scan_ticket + 1;
+    w.heavy_list = (int*)(ws + L.heavy_list);
     w.tile_state = (unsigned long long*)(ws + L.tile_state);
     w.tile_ticket = (int*)(ws + L.tile_ticket);
     w.out_cursor = (int*)(ws + L.out_cursor);
@@ -481,9 +486,9 @@ void bind_workspace(char* ws, const Layout& L, int nbox, int64_t tn, int64_t tb,
     w.big_list = (int64_t*)(ws + L.big_list);
     int* counters = (int*)(ws + L.counters);
     w.n_dense = counters;
-    w.n_team = counters + 1;
-    w.n_team_hi = counters + 2;
-    w.n_big = counters + 3;
+    w.n_team = counters + kCounterPad;
+    w.n_team_hi = counters + 2 * kCounterPad;
+    w.n_big = counters + 3 * kCounterPad;
 }
 
 int dense_min_of(const fof_options* opt)
@@ -708,7 +713,7 @@ int enqueue_link(fof_plan* h, const float* pos, cudaStream_t s)
     phase_end(h, kPhBinCount, s);
     phase_begin(h, kPhScanBricks, s);
     FOF_TRY(launch_scan(w.bcount, brick_pad(g.total_bricks), w.bstart, g.total_bricks, w.scan_state, w.scan_ticket,
-                        &w.status->err, s));
+                        heavy_from(g.total_n), w.heavy_list, w.n_heavy, &w.status->err, s));
     phase_end(h, kPhScanBricks, s);
     phase_begin(h, kPhBinScatter, s);
     FOF_TRY(launch_bin_scatter(pos, g, w, s));
@@ -865,7 +870,7 @@ int fof_relink(fof_handle h, const float* pos_dev, int32_t* path_out, void* stre
         if (path == 1) {
             // every particle kept its brick: the slots are still grouped by
             // brick, so the per-brick cell sort runs on the new positions
-            FOF_TRY(cudaMemsetAsync(w.n_dense, 0, 4 * kNumCounters, s));
+            FOF_TRY(cudaMemsetAsync(w.n_dense, 0, 4 * kNumCounters * kCounterPad, s));
             phase_begin(h, kPhBrickSort, s);
             FOF_TRY(launch_brick_sort(g, w, h->dense_min, s));
             phase_end(h, kPhBrickSort, s);
@@ -1394,7 +1399,7 @@ extern "C" int fof_run_noalloc(double box, double l_x, int64_t n, const float* p
     if (n > 0) {
         FOF_TRY(launch_bin_count(pos_dev, g, w, s));
         FOF_TRY(launch_scan(w.bcount, brick_pad(g.total_bricks), w.bstart, g.total_bricks, w.scan_state, w.scan_ticket,
-                        &w.status->err, s));
+                        heavy_from(g.total_n), w.heavy_list, w.n_heavy, &w.status->err, s));
         FOF_TRY(launch_bin_scatter(pos_dev, g, w, s));
         FOF_TRY(launch_brick_sort(g, w, kDefaultDenseMin, s));
         FOF_TRY(launch_team_self(g, w, s));
