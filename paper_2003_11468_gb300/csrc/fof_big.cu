@@ -99,6 +99,8 @@ template <bool kVar>
 __global__ void __launch_bounds__(kBigThreads) k_big_sort(Geometry g, Work w, UfArgs uf)
 {
     __shared__ BigSmem S;
+    pdl_wait();
+    pdl_trigger();
     const int n_big = *w.n_big;
     for (int it = blockIdx.x; it < n_big; it += gridDim.x) {
         const int64_t key = w.big_list[it];
@@ -184,6 +186,8 @@ template <bool kVar>
 __global__ void __launch_bounds__(kBigThreads) k_big_pairs(Geometry g, Work w, int dense_min, UfArgs uf)
 {
     __shared__ BigSmem S;
+    pdl_wait();
+    pdl_trigger();
     const int n_big = *w.n_big;
     for (int it = blockIdx.x; it < n_big; it += gridDim.x) {
         const int64_t key = w.big_list[it];
@@ -287,25 +291,22 @@ __global__ void __launch_bounds__(kBigThreads) k_big_pairs(Geometry g, Work w, i
 
 }  // namespace
 
+int big_launches(const Geometry& g)
+{
+    return g.max_split_n > kDenseMax ? 1 : 0;   // no cell can be larger than its box
+}
+
 cudaError_t launch_big(const Geometry& g, const Work& w, int dense_min, const UfArgs& uf, bool pairs,
                        cudaStream_t s)
 {
-    if (g.total_n == 0)
+    if (big_launches(g) == 0)
         return cudaSuccess;
     const int blocks = sm_count() * 2;
-    const bool var = uf.var != 0;
-    if (pairs) {
-        if (var)
-            k_big_pairs<true><<<blocks, kBigThreads, 0, s>>>(g, w, dense_min, uf);
-        else
-            k_big_pairs<false><<<blocks, kBigThreads, 0, s>>>(g, w, dense_min, uf);
-    } else {
-        if (var)
-            k_big_sort<true><<<blocks, kBigThreads, 0, s>>>(g, w, uf);
-        else
-            k_big_sort<false><<<blocks, kBigThreads, 0, s>>>(g, w, uf);
-    }
-    return cudaGetLastError();
+    if (pairs)
+        return uf.var ? launch_next(g.total_n, k_big_pairs<true>, blocks, kBigThreads, 0, s, g, w, dense_min, uf)
+                      : launch_next(g.total_n, k_big_pairs<false>, blocks, kBigThreads, 0, s, g, w, dense_min, uf);
+    return uf.var ? launch_next(g.total_n, k_big_sort<true>, blocks, kBigThreads, 0, s, g, w, uf)
+                  : launch_next(g.total_n, k_big_sort<false>, blocks, kBigThreads, 0, s, g, w, uf);
 }
 
 }  // namespace fofgpu

@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(const float* __restri
                                                            int* __restrict__ rank, int streams,
                                                            int* __restrict__ err)
 {
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const int64_t base = bin_tile_base(g.total_n, streams) + threadIdx.x;
     int bad = 0;
@@ -129,6 +130,7 @@ __global__ void __launch_bounds__(kCountThreads) k_bin_count_tile(const float* _
                                                                   int* __restrict__ rank, int* __restrict__ err)
 {
     extern __shared__ int tile_count[];                  // [total_bricks]: the tile's count, then its first rank
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const int nb = (int)g.total_bricks;
     const int64_t base = (int64_t)blockIdx.x * (kItems * kCountThreads) + threadIdx.x;
@@ -173,10 +175,11 @@ __global__ void __launch_bounds__(kCountThreads) k_bin_count_tile(const float* _
 }
 
 __global__ void __launch_bounds__(kBinThreads) k_bin_scatter(const float* __restrict__ pos, Geometry g,
-                                                             const int* __restrict__ bstart,
-                                                             const int* __restrict__ rank, int streams,
+                                                             const int* bstart, const int* rank, int streams,
                                                              float4* __restrict__ tmp, int* __restrict__ err)
 {
+    pdl_wait();
+    pdl_trigger();
     const int64_t base = bin_tile_base(g.total_n, streams) + threadIdx.x;
     float4 rec[kBinItems];
     int64_t brick[kBinItems];
@@ -196,8 +199,8 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_scatter(const float* __rest
     for (int k = 0; k < kBinItems; ++k) {
         if (brick[k] < 0)
             continue;
-        const int64_t slot = (int64_t)__ldg(bstart + brick[k]) + r[k];
-        if (slot < __ldg(bstart + brick[k] + 1))
+        const int64_t slot = (int64_t)bstart[brick[k]] + r[k];
+        if (slot < bstart[brick[k] + 1])
             tmp[slot] = rec[k];
         else
             atomicOr(err, kErrInternal);
@@ -243,7 +246,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* smem_warp, int& 
 // appended to the input, so the scan covers len + 1 entries).  The counts lie
 // `pad` words apart.
 // `heavy` (or null): entries above heavy_from are listed there.
-__global__ void __launch_bounds__(kScanThreads) k_scan(const int* __restrict__ in, int pad, int* __restrict__ out,
+__global__ void __launch_bounds__(kScanThreads) k_scan(const int* in, int pad, int* __restrict__ out,
                                                        int64_t len, unsigned long long* __restrict__ state,
                                                        int* __restrict__ ticket, int heavy_from,
                                                        int* __restrict__ heavy, int* __restrict__ n_heavy,
@@ -251,6 +254,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const int* __restrict__ i
 {
     __shared__ int sw[32];
     __shared__ int s_tile, s_before;
+    pdl_wait();
+    pdl_trigger();
     if (threadIdx.x == 0)
         s_tile = atomicAdd(ticket, 1);
     __syncthreads();
@@ -406,11 +411,16 @@ __device__ __forceinline__ int half_of(const unsigned* hist, int c)
 }
 
 __global__ void __launch_bounds__(kSortThreads, kSortBlocks)
-    k_brick_sort(Geometry g, const float4* __restrict__ tmp, const int* __restrict__ bstart,
+    k_brick_sort(Geometry g, const float4* __restrict__ tmp, const int* bstart,
                  float4* __restrict__ sorted, int* __restrict__ parent, int* __restrict__ minorig,
                  int* __restrict__ cnt, int* __restrict__ cell_start, int dense_min, CellLists lists,
-                 int heavy_from, int* __restrict__ err)
+                 int heavy_from, bool beside_heavy, int* __restrict__ err)
 {
+    // beside k_brick_sort_heavy where that runs just before (it needs nothing
+    // of it), else after the scatter
+    if (!beside_heavy)
+        pdl_wait();
+    pdl_trigger();
     extern __shared__ float4 sort_raw[];
     SortSmem& S = *reinterpret_cast<SortSmem*>(sort_raw);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -628,6 +638,8 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocks)
         }
     }
     cp_async_wait_all();
+    if (beside_heavy)
+        pdl_wait();
 }
 
 // Bricks above kHeavyBrick particles: a cluster of CTAs per brick, each CTA
@@ -644,11 +656,13 @@ constexpr int kHeavyFlight = 4;                 // loads in flight per thread
 static_assert(kMaxR3 / kCluster <= kHeavyThreads, "one cell per thread");
 
 __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kHeavyThreads, kHeavyBlocks)
-    k_brick_sort_heavy(Geometry g, const float4* __restrict__ tmp, const int* __restrict__ bstart,
-                       const int* __restrict__ heavy, const int* __restrict__ n_heavy, float4* __restrict__ sorted,
+    k_brick_sort_heavy(Geometry g, const float4* __restrict__ tmp, const int* bstart, const int* heavy,
+                       const int* n_heavy, float4* __restrict__ sorted,
                        int* __restrict__ parent, int* __restrict__ minorig, int* __restrict__ cnt,
                        int* __restrict__ cell_start, int dense_min, CellLists lists, int* __restrict__ err)
 {
+    pdl_wait();
+    pdl_trigger();
     namespace cg = cooperative_groups;
     __shared__ int hist[kMaxR3];
     __shared__ int part[kWarp];
@@ -768,6 +782,7 @@ __global__ void __launch_bounds__(256) k_relink_check(const float* __restrict__ 
                                                       float4* __restrict__ sorted, float4* __restrict__ tmp,
                                                       int* __restrict__ flags, int* __restrict__ err)
 {
+    pdl_trigger();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int f = 0, bad = 0;
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < g.total_n; s += stride) {
@@ -797,10 +812,12 @@ __global__ void __launch_bounds__(256) k_relink_check(const float* __restrict__ 
 
 // Forest and label initialisation of the binned slots (what k_brick_sort
 // does while it sorts): parent[s] = s, cnt[s] = 1, minorig[s] = local index.
-__global__ void __launch_bounds__(256) k_forest_init(int64_t total, const float4* __restrict__ sorted,
+__global__ void __launch_bounds__(256) k_forest_init(int64_t total, const float4* sorted,
                                                      int* __restrict__ parent, int* __restrict__ minorig,
                                                      int* __restrict__ cnt)
 {
+    pdl_wait();
+    pdl_trigger();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < total; s += stride) {
         parent[s] = (int)s;
@@ -864,12 +881,11 @@ int64_t scan_tiles(int64_t len)
     return (len + 1 + kScanTile - 1) / kScanTile;          // len + 1 outputs
 }
 
-cudaError_t launch_scan(const int* in, int pad, int* out, int64_t len, unsigned long long* state, int* ticket,
-                        int heavy_from, int* heavy, int* n_heavy, int* err, cudaStream_t s)
+cudaError_t launch_scan(int64_t n, const int* in, int pad, int* out, int64_t len, unsigned long long* state,
+                        int* ticket, int heavy_from, int* heavy, int* n_heavy, int* err, cudaStream_t s)
 {
-    k_scan<<<(unsigned)scan_tiles(len), kScanThreads, 0, s>>>(in, pad, out, len, state, ticket, heavy_from, heavy,
-                                                              n_heavy, err);
-    return cudaGetLastError();
+    return launch_next(n, k_scan, scan_tiles(len), kScanThreads, 0, s, in, pad, out, len, state, ticket, heavy_from,
+                       heavy, n_heavy, err);
 }
 
 cudaError_t launch_bin_scatter(const float* pos, const Geometry& g, const Work& w, cudaStream_t s)
@@ -878,9 +894,8 @@ cudaError_t launch_bin_scatter(const float* pos, const Geometry& g, const Work& 
         return cudaSuccess;
     // in the order in which the ranks were given out
     const int streams = g.total_bricks <= kTileBricks ? 1 : kBinStreams;
-    k_bin_scatter<<<(unsigned)(bin_tiles_per_stream(g.total_n, streams) * streams), kBinThreads, 0, s>>>(
-        pos, g, w.bstart, w.parent, streams, w.tmp, &w.status->err);
-    return cudaGetLastError();
+    return launch_next(g.total_n, k_bin_scatter, bin_tiles_per_stream(g.total_n, streams) * streams, kBinThreads, 0, s,
+                       pos, g, w.bstart, w.parent, streams, w.tmp, &w.status->err);
 }
 
 cudaError_t launch_brick_sort(const Geometry& g, const Work& w, int dense_min, cudaStream_t s)
@@ -894,10 +909,9 @@ cudaError_t launch_brick_sort(const Geometry& g, const Work& w, int dense_min, c
         int64_t clusters = g.total_n / kHeavyBrick;
         const int64_t most = (int64_t)sm_count() * kHeavyBlocks / kCluster;
         if (clusters > most) clusters = most;
-        k_brick_sort_heavy<<<(unsigned)(clusters * kCluster), kHeavyThreads, 0, s>>>(
-            g, w.tmp, w.bstart, w.heavy_list, w.n_heavy, w.sorted, w.parent, w.minorig, w.cnt, w.cell_start,
-            dense_min, lists, &w.status->err);
-        cudaError_t e = cudaGetLastError();
+        cudaError_t e = launch_next(g.total_n, k_brick_sort_heavy, clusters * kCluster, kHeavyThreads, 0, s, g, w.tmp,
+                                    w.bstart, w.heavy_list, w.n_heavy, w.sorted, w.parent, w.minorig, w.cnt,
+                                    w.cell_start, dense_min, lists, &w.status->err);
         if (e != cudaSuccess) return e;
     }
     // the shared-memory opt-in is per device; setting it again is harmless
@@ -913,10 +927,10 @@ cudaError_t launch_brick_sort(const Geometry& g, const Work& w, int dense_min, c
     int64_t blocks = g.total_bricks;
     int64_t cap = (int64_t)sm_count() * kSortBlocks;
     if (blocks > cap) blocks = cap;
-    k_brick_sort<<<(unsigned)blocks, kSortThreads, sizeof(SortSmem), s>>>(g, w.tmp, w.bstart, w.sorted, w.parent, w.minorig, w.cnt,
-                                                         w.cell_start, dense_min, lists, heavy_from(g.total_n),
-                                                         &w.status->err);
-    return cudaGetLastError();
+    const bool beside = heavy_bricks(g.total_n);
+    return launch_kernel(g.total_n <= (beside ? kBesideMax : kDependentMax), k_brick_sort, blocks, kSortThreads,
+                         sizeof(SortSmem), s, g, w.tmp, w.bstart, w.sorted, w.parent, w.minorig, w.cnt, w.cell_start,
+                         dense_min, lists, heavy_from(g.total_n), beside, &w.status->err);
 }
 
 // Bricks above this many particles go to k_brick_sort_heavy: the limit of the
@@ -947,9 +961,8 @@ cudaError_t launch_forest_init(const Geometry& g, const Work& w, cudaStream_t s)
 {
     if (g.total_n == 0)
         return cudaSuccess;
-    k_forest_init<<<grid_for(g.total_n, 256, 8), 256, 0, s>>>(g.total_n, w.sorted, w.parent, w.minorig,
-                                                             w.cnt);
-    return cudaGetLastError();
+    return launch_next(g.total_n, k_forest_init, grid_for(g.total_n, 256, 8), 256, 0, s, g.total_n, w.sorted, w.parent,
+                       w.minorig, w.cnt);
 }
 
 }  // namespace fofgpu

@@ -439,6 +439,10 @@ template <bool kVar, int kLo, int kM, int kThreads, int kBlocks>
 __global__ void __launch_bounds__(kThreads, kBlocks) k_dense_self(Geometry g, Work w, int dense_min,
                                                               UfArgs uf)
 {
+    // beside k_link, which never touches a dense cell's particles (it reads
+    // their records, but only to see which cell they are in), and beside the
+    // other size class: their unions are the same atomic ones
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const DenseSmem S = carve<kM>(smem_raw);
     int* err = uf.err;
@@ -562,12 +566,17 @@ __global__ void __launch_bounds__(kThreads, kBlocks) k_dense_self(Geometry g, Wo
         link_neighbours<kVar, kThreads>(S, w, b, ox, oy, oz, main, single, uf);
         __syncthreads();
     }
+    pdl_wait();
 }
 
 template <bool kVar, int kLo, int kM, int kThreads, int kBlocks>
 __global__ void __launch_bounds__(kThreads, kBlocks) k_dense_pairs(Geometry g, Work w, int dense_min,
                                                                UfArgs uf)
 {
+    // after dense_self; the second size class beside the first
+    if (kLo == 0)
+        pdl_wait();
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const DenseSmem S = carve<kM>(smem_raw);
     int* err = uf.err;
@@ -633,6 +642,8 @@ __global__ void __launch_bounds__(kThreads, kBlocks) k_dense_pairs(Geometry g, W
         link_neighbours<kVar, kThreads>(S, w, b, ox, oy, oz, main, single, uf);
         __syncthreads();
     }
+    if (kLo != 0)
+        pdl_wait();
 }
 
 }  // namespace
@@ -658,15 +669,15 @@ cudaError_t configure_dense()
 }
 
 template <bool kVar, int kLo, int kM, int kThreads, int kBlocks>
-void run_dense(const Geometry& g, const Work& w, int dense_min, const UfArgs& uf, bool pairs, cudaStream_t s)
+cudaError_t run_dense(const Geometry& g, const Work& w, int dense_min, const UfArgs& uf, bool pairs, cudaStream_t s)
 {
     const int blocks = sm_count() * kBlocks;
-    if (pairs)
-        k_dense_pairs<kVar, kLo, kM, kThreads, kBlocks><<<blocks, kThreads, dense_smem_bytes<kM>(), s>>>(
-            g, w, dense_min, uf);
-    else
-        k_dense_self<kVar, kLo, kM, kThreads, kBlocks><<<blocks, kThreads, dense_smem_bytes<kM>(), s>>>(
-            g, w, dense_min, uf);
+    if (pairs && kLo == 0)
+        return launch_next(g.total_n, k_dense_pairs<kVar, kLo, kM, kThreads, kBlocks>, blocks, kThreads,
+                           dense_smem_bytes<kM>(), s, g, w, dense_min, uf);
+    return launch_beside(g.total_n, pairs ? k_dense_pairs<kVar, kLo, kM, kThreads, kBlocks>
+                                          : k_dense_self<kVar, kLo, kM, kThreads, kBlocks>,
+                         blocks, kThreads, dense_smem_bytes<kM>(), s, g, w, dense_min, uf);
 }
 
 template <bool kVar>
@@ -679,19 +690,26 @@ cudaError_t configure_all()
 }
 
 template <bool kVar>
-void run_all(const Geometry& g, const Work& w, int dense_min, const UfArgs& uf, bool pairs, cudaStream_t s)
+cudaError_t run_all(const Geometry& g, const Work& w, int dense_min, const UfArgs& uf, bool pairs, cudaStream_t s)
 {
-    if (dense_one_launch(g.total_n)) {
-        run_dense<kVar, 0, kDenseMax, 1024, 1>(g, w, dense_min, uf, pairs, s);
-    } else {
-        run_dense<kVar, 0, kDenseSmall, 256, 6>(g, w, dense_min, uf, pairs, s);
-        run_dense<kVar, kDenseSmall, kDenseMax, 512, 2>(g, w, dense_min, uf, pairs, s);
-    }
+    if (dense_one_launch(g.total_n))
+        return run_dense<kVar, 0, kDenseMax, 1024, 1>(g, w, dense_min, uf, pairs, s);
+    cudaError_t e = run_dense<kVar, 0, kDenseSmall, 256, 6>(g, w, dense_min, uf, pairs, s);
+    return e != cudaSuccess ? e : run_dense<kVar, kDenseSmall, kDenseMax, 512, 2>(g, w, dense_min, uf, pairs, s);
+}
+
+int dense_launches(const Geometry& g, int dense_min)
+{
+    if (g.max_split_n < dense_min)
+        return 0;                               // no cell can be larger than its box
+    return dense_one_launch(g.total_n) ? 1 : 2;
 }
 
 cudaError_t launch_dense(const Geometry& g, const Work& w, int dense_min, const UfArgs& uf, bool pairs,
                          cudaStream_t s)
 {
+    if (dense_launches(g, dense_min) == 0)
+        return cudaSuccess;
     // the shared-memory opt-in is per device; setting it again is harmless
     static bool configured[64] = {};
     int dev = 0;
@@ -702,11 +720,7 @@ cudaError_t launch_dense(const Geometry& g, const Work& w, int dense_min, const 
         if ((e = configure_all<true>()) != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) configured[dev] = true;
     }
-    if (uf.var)
-        run_all<true>(g, w, dense_min, uf, pairs, s);
-    else
-        run_all<false>(g, w, dense_min, uf, pairs, s);
-    return cudaGetLastError();
+    return uf.var ? run_all<true>(g, w, dense_min, uf, pairs, s) : run_all<false>(g, w, dense_min, uf, pairs, s);
 }
 
 }  // namespace fofgpu

@@ -102,6 +102,84 @@ struct Status {
 };
 
 // ------------------------------------------------------------------------
+// dependent launches
+// ------------------------------------------------------------------------
+//
+// A kernel can be launched as a programmatic dependent of the one before it in
+// the stream: its CTAs may start once every CTA of that one has started and
+// called pdl_trigger (or exited), which takes the launch gap, 2 to 3 us a
+// kernel, off the small problems.  A kernel touches nothing that an earlier
+// kernel writes before pdl_wait, which returns when the kernel before it has
+// completed (and, since that one waited too, all earlier ones).
+//
+// A kernel that does not need the one just before it calls pdl_wait as its
+// last step instead, so that it runs beside it and still completes after it.
+// It starts when every CTA before it has triggered, and those trigger only
+// after their own wait at the top, so everything up to the kernel before the
+// one before it has completed by then.  (After a plain launch both calls return
+// at once, and the order in the stream does the rest.)
+//
+// Values that an earlier kernel writes are not read through `const
+// __restrict__` parameters or __ldg before a value that was read after the
+// wait decides their address: the compiler takes such loads for constant
+// during the kernel and may move them above the wait.
+//
+// Every kernel is launched so up to kDependentMax particles: above, launch gaps
+// count for nothing, and a CTA that starts early on an SM keeps the split of
+// its L1 that the kernel before wanted (768^3 box, step: 84.7 ms with all
+// launches dependent, 82.0 with none; 4 million particles, two steps: 1940 and
+// 2130 us).  Kernels that run beside the one before them are up to kBesideMax,
+// above which they find no idle SM (16.8 million: 3405 us with them, 3480
+// without; 512 boxes, 333 million: 62.8 ms and 62.6).
+
+constexpr int64_t kDependentMax = 1 << 22;
+constexpr int64_t kBesideMax = 1 << 26;
+
+__device__ __forceinline__ void pdl_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+__device__ __forceinline__ void pdl_trigger()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// dependent: as a programmatic dependent, else a plain launch
+template <class... P, class... A>
+cudaError_t launch_kernel(bool dependent, void (*kernel)(P...), int64_t grid, int block, size_t smem, cudaStream_t s,
+                          A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// The next kernel of a run over n particles.
+template <class... P, class... A>
+cudaError_t launch_next(int64_t n, void (*kernel)(P...), int64_t grid, int block, size_t smem, cudaStream_t s,
+                        A... args)
+{
+    return launch_kernel(n <= kDependentMax, kernel, grid, block, smem, s, args...);
+}
+
+// One that runs beside the kernel before it.
+template <class... P, class... A>
+cudaError_t launch_beside(int64_t n, void (*kernel)(P...), int64_t grid, int block, size_t smem, cudaStream_t s,
+                          A... args)
+{
+    return launch_kernel(n <= kBesideMax, kernel, grid, block, smem, s, args...);
+}
+
+// ------------------------------------------------------------------------
 // warp helpers
 // ------------------------------------------------------------------------
 
@@ -579,6 +657,7 @@ struct Geometry {
     const int64_t* box_p0;     // [nbox] first particle of each box
     const int64_t* box_brick0; // [nbox] first brick of each box
     int nbox;
+    int64_t max_split_n;       // particles of the largest box that splits cells (0: none)
     int64_t total_n;           // particles over all boxes
     int64_t total_bricks;
     int64_t total_cells;
@@ -632,10 +711,11 @@ constexpr int64_t kDirectMax = 1 << 24;
 int sm_count();
 
 cudaError_t launch_bin_count(const float* pos, const Geometry& g, const Work& w, cudaStream_t s);
-// exclusive prefix sum of in[i * pad], i < len, into out[0..len]; state
+// (of a run over n particles) exclusive prefix sum of in[i * pad], i < len,
+// into out[0..len]; state
 // (scan_tiles(len) words) and ticket start at zero; entries above heavy_from
 // are listed in `heavy` unless it is null
-cudaError_t launch_scan(const int* in, int pad, int* out, int64_t len, unsigned long long* state, int* ticket,
+cudaError_t launch_scan(int64_t n, const int* in, int pad, int* out, int64_t len, unsigned long long* state, int* ticket,
                         int heavy_from, int* heavy, int* n_heavy, int* err, cudaStream_t s);
 int heavy_from(int64_t total_n);
 bool heavy_bricks(int64_t total_n);   // whether a brick can be above heavy_from
@@ -649,7 +729,8 @@ cudaError_t launch_relink_check(const float* pos, const Geometry& g, const Work&
 cudaError_t launch_forest_init(const Geometry& g, const Work& w, cudaStream_t s);
 cudaError_t launch_dense(const Geometry& g, const Work& w, int dense_min, const UfArgs& uf, bool pairs,
                          cudaStream_t s);
-bool dense_one_launch(int64_t total_n);
+int dense_launches(const Geometry& g, int dense_min);   // kernels of one launch_dense
+int big_launches(const Geometry& g);                    // and of one launch_big
 cudaError_t launch_link(const Geometry& g, const Work& w, int dense_min, const UfArgs& uf,
                         cudaStream_t s);
 cudaError_t launch_team_self(const Geometry& g, const Work& w, cudaStream_t s);
@@ -658,7 +739,8 @@ cudaError_t launch_team_self(const Geometry& g, const Work& w, cudaStream_t s);
 cudaError_t launch_big(const Geometry& g, const Work& w, int dense_min, const UfArgs& uf, bool pairs,
                        cudaStream_t s);
 // size_count: 0 warp-aggregated atomics, 1 per-block shared-memory hash table
-cudaError_t launch_finalize(const Geometry& g, const Work& w, const UfArgs& uf, int size_count,
+// dependent: nothing but this library's kernels lies between in the stream
+cudaError_t launch_finalize(const Geometry& g, const Work& w, const UfArgs& uf, int size_count, bool dependent,
                             cudaStream_t s);
 cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t min_size, cudaStream_t s);
 cudaError_t launch_catalogue(const Geometry& g, const Work& w, int32_t* ids, int32_t* sizes,

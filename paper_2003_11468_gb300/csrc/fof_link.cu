@@ -273,6 +273,8 @@ __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4*
                                                        const int* __restrict__ cell_start, int* parent,
                                                        int dense_min, UfArgs uf)
 {
+    pdl_wait();
+    pdl_trigger();
     __shared__ TeamStage stage[kLinkWarps];
     __shared__ uint32_t spread_tab[16];
     if (threadIdx.x < 16)
@@ -866,9 +868,11 @@ __device__ __forceinline__ void team_cell_cta(TeamCtaSmem& S, int c0, int m, flo
 }
 
 __global__ void __launch_bounds__(kTeamWarps * 32, kTeamBlocks)
-    k_team_self(Geometry g, const int64_t* __restrict__ list, int64_t cap, const int* __restrict__ n_lo,
-                const int* __restrict__ n_hi, float4* sorted, int* __restrict__ parent, int* __restrict__ minorig)
+    k_team_self(Geometry g, const int64_t* list, int64_t cap, const int* n_lo, const int* n_hi, float4* sorted,
+                int* __restrict__ parent, int* __restrict__ minorig)
 {
+    pdl_wait();
+    pdl_trigger();
     extern __shared__ float4 team_raw[];
     TeamSmem& smem = *reinterpret_cast<TeamSmem*>(team_raw);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -988,9 +992,8 @@ cudaError_t launch_team_self(const Geometry& g, const Work& w, cudaStream_t s)
     int64_t blocks = w.team_cap / kTeamWarps + 1;
     const int64_t most = (int64_t)sm_count() * kTeamBlocks;
     if (blocks > most) blocks = most;
-    k_team_self<<<(unsigned)blocks, kTeamWarps * 32, sizeof(TeamSmem), s>>>(g, w.team_list, w.team_cap, w.n_team,
-                                                                           w.n_team_hi, w.sorted, w.parent, w.minorig);
-    return cudaGetLastError();
+    return launch_next(g.total_n, k_team_self, blocks, kTeamWarps * 32, sizeof(TeamSmem), s, g, w.team_list, w.team_cap,
+                       w.n_team, w.n_team_hi, w.sorted, w.parent, w.minorig);
 }
 
 cudaError_t launch_link(const Geometry& g, const Work& w, int dense_min, const UfArgs& uf, cudaStream_t s)
@@ -1001,11 +1004,8 @@ cudaError_t launch_link(const Geometry& g, const Work& w, int dense_min, const U
     int64_t blocks = (warps * kWarp + kLinkThreads - 1) / kLinkThreads;
     int64_t cap = (int64_t)sm_count() * 8;
     if (blocks > cap) blocks = cap;
-    if (uf.var)
-        k_link<true><<<(unsigned)blocks, kLinkThreads, 0, s>>>(g, w.sorted, w.cell_start, w.parent, dense_min, uf);
-    else
-        k_link<false><<<(unsigned)blocks, kLinkThreads, 0, s>>>(g, w.sorted, w.cell_start, w.parent, dense_min, uf);
-    return cudaGetLastError();
+    return launch_next(g.total_n, uf.var ? k_link<true> : k_link<false>, blocks, kLinkThreads, 0, s, g, w.sorted,
+                       w.cell_start, w.parent, dense_min, uf);
 }
 
 }  // namespace fofgpu

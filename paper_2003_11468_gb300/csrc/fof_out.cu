@@ -43,6 +43,8 @@ __global__ void __launch_bounds__(256) k_finalize(int64_t total, int* __restrict
                                                   int* __restrict__ minorig, int* __restrict__ cnt,
                                                   int* __restrict__ err, bool ordered)
 {
+    pdl_wait();
+    pdl_trigger();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < total; base += stride) {
         int64_t s = base + threadIdx.x;
@@ -79,6 +81,8 @@ __global__ void __launch_bounds__(256) k_finalize_hash(int64_t total, int* __res
                                                        int* __restrict__ minorig, int* __restrict__ cnt,
                                                        int* __restrict__ err, bool ordered)
 {
+    pdl_wait();
+    pdl_trigger();
     __shared__ int hkey[kHashSlots];
     __shared__ int hcnt[kHashSlots];
     __shared__ int hmin[kHashSlots];
@@ -169,15 +173,15 @@ __global__ void __launch_bounds__(256) k_finalize_hash(int64_t total, int* __res
 //            inputs: 2.6 ms), so the kernel leaves the tile's count, and a
 //            scan and k_catalogue follow (1.3 ms in all).
 template <bool kDirect>
-__global__ void __launch_bounds__(256) k_outputs_scatter(Geometry g, const float4* __restrict__ sorted,
-                                                         const int* __restrict__ parent,
-                                                         const int* __restrict__ minorig,
-                                                         const int* __restrict__ cnt, int32_t thr,
+__global__ void __launch_bounds__(256) k_outputs_scatter(Geometry g, const float4* sorted, const int* parent,
+                                                         const int* minorig, const int* cnt, int32_t thr,
                                                          unsigned long long* __restrict__ n_groups,
                                                          unsigned long long* __restrict__ n_cat,
                                                          int2* __restrict__ pairs,
                                                          int* __restrict__ out_cursor, int* __restrict__ err)
 {
+    pdl_wait();
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int acc_box = -1;                           // per-warp box counts not yet added
@@ -291,7 +295,7 @@ __device__ __forceinline__ int scan_rows(int* s_cnt, int lane)
 }
 
 template <bool kDirect>
-__global__ void __launch_bounds__(kOutThreads) k_outputs_write(Geometry g, const int2* __restrict__ pairs,
+__global__ void __launch_bounds__(kOutThreads) k_outputs_write(Geometry g, const int2* pairs,
                                                                int32_t* __restrict__ ids,
                                                                int32_t* __restrict__ sizes, int32_t thr,
                                                                int2* __restrict__ cat, int64_t cap,
@@ -299,6 +303,8 @@ __global__ void __launch_bounds__(kOutThreads) k_outputs_write(Geometry g, const
                                                                int* __restrict__ ticket,
                                                                int* __restrict__ out_cursor, Status* status)
 {
+    pdl_wait();
+    pdl_trigger();
     __shared__ int s_tile, s_off;
     __shared__ int s_cnt[kOutItems * kOutWarps];
     __shared__ int2 placed[kDirect ? 1 : kOutTile];
@@ -381,11 +387,12 @@ __global__ void __launch_bounds__(kOutThreads) k_outputs_write(Geometry g, const
 
 // Catalogue above kDirectMax inputs: one CTA per output tile that holds
 // entries writes them in ascending label order from tile_off[tile] on.
-__global__ void __launch_bounds__(kOutThreads) k_catalogue(Geometry g, const int32_t* __restrict__ sizes,
-                                                           const int* __restrict__ tile_off, int32_t thr,
-                                                           int2* __restrict__ cat, int64_t cap, int64_t n_tiles,
+__global__ void __launch_bounds__(kOutThreads) k_catalogue(Geometry g, const int32_t* sizes, const int* tile_off,
+                                                           int32_t thr, int2* __restrict__ cat, int64_t cap, int64_t n_tiles,
                                                            Status* status)
 {
+    pdl_wait();
+    pdl_trigger();
     __shared__ int s_cnt[kOutItems * kOutWarps];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (blockIdx.x == 0 && threadIdx.x == 0)
@@ -436,19 +443,18 @@ static int grid_for(int64_t items, int threads, int per_sm)
     return (int)(want < cap ? want : cap);
 }
 
-cudaError_t launch_finalize(const Geometry& g, const Work& w, const UfArgs& uf, int size_count,
+cudaError_t launch_finalize(const Geometry& g, const Work& w, const UfArgs& uf, int size_count, bool dependent,
                             cudaStream_t s)
 {
     if (g.total_n == 0)
         return cudaSuccess;
     const bool ordered = uf.link == 0;
+    dependent = dependent && g.total_n <= kDependentMax;
     if (size_count == 1)
-        k_finalize_hash<<<grid_for(g.total_n, 256 * kHashBatch, 4), 256, 0, s>>>(
-            g.total_n, w.parent, w.minorig, w.cnt, &w.status->err, ordered);
-    else
-        k_finalize<<<grid_for(g.total_n, 256, 8), 256, 0, s>>>(g.total_n, w.parent, w.minorig, w.cnt,
-                                                              &w.status->err, ordered);
-    return cudaGetLastError();
+        return launch_kernel(dependent, k_finalize_hash, grid_for(g.total_n, 256 * kHashBatch, 4), 256, 0, s, g.total_n,
+                             w.parent, w.minorig, w.cnt, &w.status->err, ordered);
+    return launch_kernel(dependent, k_finalize, grid_for(g.total_n, 256, 8), 256, 0, s, g.total_n, w.parent, w.minorig,
+                         w.cnt, &w.status->err, ordered);
 }
 
 cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t min_size, cudaStream_t s)
@@ -457,14 +463,9 @@ cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t min_size, c
         return cudaSuccess;
     int32_t thr = min_size < 1 ? 1 : min_size;
     int2* pairs = (int2*)w.tmp;            // the brick-order copy is dead by now
-    const int blocks = grid_for(g.total_n, 256, 8);
-    if (g.total_n <= kDirectMax)
-        k_outputs_scatter<true><<<blocks, 256, 0, s>>>(g, w.sorted, w.parent, w.minorig, w.cnt, thr, w.n_groups,
-                                                       w.n_cat, pairs, w.out_cursor, &w.status->err);
-    else
-        k_outputs_scatter<false><<<blocks, 256, 0, s>>>(g, w.sorted, w.parent, w.minorig, w.cnt, thr, w.n_groups,
-                                                        w.n_cat, pairs, w.out_cursor, &w.status->err);
-    return cudaGetLastError();
+    return launch_next(g.total_n, g.total_n <= kDirectMax ? k_outputs_scatter<true> : k_outputs_scatter<false>,
+                       grid_for(g.total_n, 256, 8), 256, 0, s, g, w.sorted, w.parent, w.minorig, w.cnt, thr,
+                       w.n_groups, w.n_cat, pairs, w.out_cursor, &w.status->err);
 }
 
 cudaError_t launch_catalogue(const Geometry& g, const Work& w, int32_t* ids, int32_t* sizes, int32_t min_size,
@@ -474,21 +475,18 @@ cudaError_t launch_catalogue(const Geometry& g, const Work& w, int32_t* ids, int
         return cudaSuccess;
     int32_t thr = min_size < 1 ? 1 : min_size;
     const int2* pairs = (const int2*)w.tmp;
-    const unsigned blocks = (unsigned)w.n_tiles;
-    if (g.total_n <= kDirectMax) {
-        k_outputs_write<true><<<blocks, kOutThreads, 0, s>>>(g, pairs, ids, sizes, thr, cat, cap, w.tile_state,
-                                                             w.tile_ticket, w.out_cursor, w.status);
-        return cudaGetLastError();
-    }
-    k_outputs_write<false><<<blocks, kOutThreads, 0, s>>>(g, pairs, ids, sizes, thr, cat, cap, w.tile_state,
-                                                          w.tile_ticket, w.out_cursor, w.status);
-    cudaError_t e = launch_scan(w.out_cursor, 1, w.tile_off, w.n_tiles, w.tile_state, w.tile_ticket,
-                                0, nullptr, nullptr, &w.status->err, s);
+    const bool direct = g.total_n <= kDirectMax;
+    cudaError_t e = launch_next(g.total_n, direct ? k_outputs_write<true> : k_outputs_write<false>, w.n_tiles, kOutThreads, 0, s,
+                                g, pairs, ids, sizes, thr, cat, cap, w.tile_state, w.tile_ticket, w.out_cursor,
+                                w.status);
+    if (e != cudaSuccess || direct)
+        return e;
+    e = launch_scan(g.total_n, w.out_cursor, 1, w.tile_off, w.n_tiles, w.tile_state, w.tile_ticket, 0, nullptr, nullptr,
+                    &w.status->err, s);
     if (e != cudaSuccess)
         return e;
-    k_catalogue<<<grid_for(w.n_tiles * kOutThreads, kOutThreads, 4), kOutThreads, 0, s>>>(
-        g, sizes, w.tile_off, thr, cat, cap, w.n_tiles, w.status);
-    return cudaGetLastError();
+    return launch_next(g.total_n, k_catalogue, grid_for(w.n_tiles * kOutThreads, kOutThreads, 4), kOutThreads, 0, s, g, sizes,
+                       w.tile_off, thr, cat, cap, w.n_tiles, w.status);
 }
 
 }  // namespace fofgpu

@@ -47,14 +47,16 @@ const char* kPhaseNames[kNumPhases] = {
     "dense_pairs", "big_pairs", "link", "finalize", "outputs", "catalogue",
 };
 
-// kernel launches of one phase over total_n particles
-int phase_launches(int ph, int64_t total_n)
+// kernel launches of one phase of a plan
+int phase_launches(int ph, const Geometry& g, int dense_min)
 {
     switch (ph) {
+    case kPhBigSort:
+    case kPhBigPairs: return big_launches(g);
     case kPhDenseSelf:
-    case kPhDensePairs: return dense_one_launch(total_n) ? 1 : 2;
-    case kPhBrickSort: return heavy_bricks(total_n) ? 2 : 1;
-    case kPhCatalogue: return total_n <= kDirectMax ? 1 : 3;
+    case kPhDensePairs: return dense_launches(g, dense_min);
+    case kPhBrickSort: return heavy_bricks(g.total_n) ? 2 : 1;
+    case kPhCatalogue: return g.total_n <= kDirectMax ? 1 : 3;
     default: return 1;
     }
 }
@@ -448,8 +450,13 @@ Layout layout(int nbox, int64_t total_n, int64_t total_bricks, int64_t total_cel
 }
 
 // Device pointers of a workspace laid out by L.
-void bind_workspace(char* ws, const Layout& L, int nbox, int64_t tn, int64_t tb, int64_t tc, Geometry& g, Work& w)
+void bind_workspace(char* ws, const Layout& L, const BoxDev* boxes, int nbox, int64_t tn, int64_t tb, int64_t tc,
+                    Geometry& g, Work& w)
 {
+    g.max_split_n = 0;
+    for (int i = 0; i < nbox; ++i)
+        if (boxes[i].q > 1)
+            g.max_split_n = std::max(g.max_split_n, boxes[i].n);
     g.boxes = (const BoxDev*)(ws + L.boxes);
     g.box_p0 = (const int64_t*)(ws + L.p0);
     g.box_brick0 = (const int64_t*)(ws + L.brick0);
@@ -547,8 +554,8 @@ int cuda_rc(cudaError_t e)
 
 void phase_begin(fof_plan* h, int ph, cudaStream_t s)
 {
-    h->launches += phase_launches(ph, h->g.total_n);
-    h->phase[ph].launches += phase_launches(ph, h->g.total_n);
+    h->launches += phase_launches(ph, h->g, h->dense_min);
+    h->phase[ph].launches += phase_launches(ph, h->g, h->dense_min);
     if (h->timing && !h->capturing) {
         cudaEventRecord(h->phase[ph].ev0, s);
     }
@@ -639,7 +646,7 @@ int create_plan(int32_t nbox, const double* box, const double* l_x, const int64_
         h->p0[i] = boxes[i].p0;
         h->brick0[i] = boxes[i].brick0;
     }
-    bind_workspace(ws, L, nbox, tn, tb, tc, h->g, h->w);
+    bind_workspace(ws, L, boxes.data(), nbox, tn, tb, tc, h->g, h->w);
     h->results_dev = ws + L.results;
     h->zero_dev = ws + L.bcount;
     h->zero_end = ws + L.zero_end;
@@ -668,8 +675,9 @@ UfArgs uf_args(const fof_plan* h)
     return u;
 }
 
-// Linking on the binned particles: self tasks of team cells, dense cells,
-// then the rest (shared by fof_link and fof_relink).
+// Linking on the binned particles: self tasks of team and big cells, then
+// k_link with the dense cells beside it (launch_next), then the pairs that need
+// every cell's slots in their final order (shared by fof_link and fof_relink).
 int enqueue_linking(fof_plan* h, cudaStream_t s)
 {
     const Geometry& g = h->g;
@@ -681,6 +689,9 @@ int enqueue_linking(fof_plan* h, cudaStream_t s)
     phase_begin(h, kPhBigSort, s);
     FOF_TRY(launch_big(g, w, h->dense_min, uf, false, s));
     phase_end(h, kPhBigSort, s);
+    phase_begin(h, kPhLink, s);
+    FOF_TRY(launch_link(g, w, h->dense_min, uf, s));
+    phase_end(h, kPhLink, s);
     phase_begin(h, kPhDenseSelf, s);
     FOF_TRY(launch_dense(g, w, h->dense_min, uf, false, s));
     phase_end(h, kPhDenseSelf, s);
@@ -690,9 +701,6 @@ int enqueue_linking(fof_plan* h, cudaStream_t s)
     phase_begin(h, kPhBigPairs, s);
     FOF_TRY(launch_big(g, w, h->dense_min, uf, true, s));
     phase_end(h, kPhBigPairs, s);
-    phase_begin(h, kPhLink, s);
-    FOF_TRY(launch_link(g, w, h->dense_min, uf, s));
-    phase_end(h, kPhLink, s);
     h->linked = true;
     return FOF_OK;
 }
@@ -712,7 +720,7 @@ int enqueue_link(fof_plan* h, const float* pos, cudaStream_t s)
     FOF_TRY(launch_bin_count(pos, g, w, s));
     phase_end(h, kPhBinCount, s);
     phase_begin(h, kPhScanBricks, s);
-    FOF_TRY(launch_scan(w.bcount, brick_pad(g.total_bricks), w.bstart, g.total_bricks, w.scan_state, w.scan_ticket,
+    FOF_TRY(launch_scan(g.total_n, w.bcount, brick_pad(g.total_bricks), w.bstart, g.total_bricks, w.scan_state, w.scan_ticket,
                         heavy_from(g.total_n), w.heavy_list, w.n_heavy, &w.status->err, s));
     phase_end(h, kPhScanBricks, s);
     phase_begin(h, kPhBinScatter, s);
@@ -735,13 +743,14 @@ int enqueue_groups(fof_plan* h, int32_t* ids, int32_t* sizes, fof_group* cat, in
     const Work& w = h->w;
     if (g.total_n > 0) {
         // status.err is kept from fof_link; counts start from zero
-        if (!h->groups_clean) {
+        const bool clean = h->groups_clean;
+        if (!clean) {
             char* from = h->results_dev + h->rl.groups_off;
             FOF_TRY(cudaMemsetAsync(from, 0, (size_t)(h->zero_end - from), s));
         }
         h->groups_clean = false;
         phase_begin(h, kPhFinalize, s);
-        FOF_TRY(launch_finalize(g, w, uf_args(h), h->size_count, s));
+        FOF_TRY(launch_finalize(g, w, uf_args(h), h->size_count, clean, s));
         phase_end(h, kPhFinalize, s);
         phase_begin(h, kPhOutputs, s);
         FOF_TRY(launch_outputs(g, w, min_size, s));
@@ -1133,8 +1142,8 @@ int fof_graph_launch(fof_handle h, void* stream)
     // a graph replays every phase once
     for (int k = 0; k < kNumPhases; ++k) {
         if (h->g.total_n > 0) {
-            h->launches += phase_launches(k, h->g.total_n);
-            h->phase[k].launches += phase_launches(k, h->g.total_n);
+            h->launches += phase_launches(k, h->g, h->dense_min);
+            h->phase[k].launches += phase_launches(k, h->g, h->dense_min);
         }
     }
     return FOF_OK;
@@ -1386,7 +1395,7 @@ extern "C" int fof_run_noalloc(double box, double l_x, int64_t n, const float* p
 
     Geometry g{};
     Work w{};
-    bind_workspace(ws, L, 1, n, tb, tc, g, w);
+    bind_workspace(ws, L, &b, 1, n, tb, tc, g, w);
     char* res = ws + L.results;
 
     // The array keeps the previous call's contents: the box table is
@@ -1398,7 +1407,7 @@ extern "C" int fof_run_noalloc(double box, double l_x, int64_t n, const float* p
     FOF_TRY(cudaMemsetAsync(ws + L.bcount, 0, L.zero_end - L.bcount, s));
     if (n > 0) {
         FOF_TRY(launch_bin_count(pos_dev, g, w, s));
-        FOF_TRY(launch_scan(w.bcount, brick_pad(g.total_bricks), w.bstart, g.total_bricks, w.scan_state, w.scan_ticket,
+        FOF_TRY(launch_scan(g.total_n, w.bcount, brick_pad(g.total_bricks), w.bstart, g.total_bricks, w.scan_state, w.scan_ticket,
                         heavy_from(g.total_n), w.heavy_list, w.n_heavy, &w.status->err, s));
         FOF_TRY(launch_bin_scatter(pos_dev, g, w, s));
         FOF_TRY(launch_brick_sort(g, w, kDefaultDenseMin, s));
@@ -1410,11 +1419,11 @@ extern "C" int fof_run_noalloc(double box, double l_x, int64_t n, const float* p
         uf.link = 0;
         uf.var = 0;
         FOF_TRY(launch_big(g, w, kDefaultDenseMin, uf, false, s));
+        FOF_TRY(launch_link(g, w, kDefaultDenseMin, uf, s));
         FOF_TRY(launch_dense(g, w, kDefaultDenseMin, uf, false, s));
         FOF_TRY(launch_dense(g, w, kDefaultDenseMin, uf, true, s));
         FOF_TRY(launch_big(g, w, kDefaultDenseMin, uf, true, s));
-        FOF_TRY(launch_link(g, w, kDefaultDenseMin, uf, s));
-        FOF_TRY(launch_finalize(g, w, uf, 0, s));
+        FOF_TRY(launch_finalize(g, w, uf, 0, true, s));
         FOF_TRY(launch_outputs(g, w, min_size, s));
         FOF_TRY(launch_catalogue(g, w, ids_dev, sizes_dev, min_size, (int2*)catalogue_dev, cat_capacity, s));
     }
