@@ -99,6 +99,7 @@ struct Status {
     int err;
     int pad;
     long long n_cat_total;
+    unsigned link_ticket;
 };
 
 // ------------------------------------------------------------------------
@@ -682,6 +683,7 @@ struct Work {
     int* tile_off;      // [n_tiles + 1] first catalogue entry of each tile (above kDirectMax inputs)
     int64_t n_tiles;
     Status* status;     // device status
+    unsigned* link_ticket; // batches of windows handed out by k_link
     unsigned long long* n_groups;  // [nbox]
     unsigned long long* n_cat;     // [nbox]
     int64_t* dense_list; // [dense_cap] cell keys of the subdivided cells

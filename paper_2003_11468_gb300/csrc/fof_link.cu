@@ -141,6 +141,7 @@ struct TeamStage {
 
 constexpr int kLinkThreads = 256;
 constexpr int kLinkWarps = kLinkThreads / 32;
+constexpr int kLinkBlocks = 4;   // resident CTAs per SM (64 registers)
 constexpr int kOwnCell = 13;     // stream index of a team's own cell (cells above kTeamSelfMax)
 
 // The buffered candidates S.cpos/cslot[0..c) of a team against its m
@@ -218,26 +219,29 @@ __device__ __forceinline__ void team_flush(TeamStage& S, int* __restrict__ paren
 // memory (most are dropped, so a team usually fills one buffer of 32) and
 // handed to team_flush when the buffer is full and at the end, so that the
 // roots, pair tests and unions of several chunks take one round.
-template <bool kVar>
+// kSplit: this warp takes chunks part, part + parts, ... of the stream.
+template <bool kVar, bool kSplit>
 __device__ __forceinline__ void team_cell(TeamStage& S, int* __restrict__ parent,
                                           const float4* __restrict__ sorted, const BoxDev& b, int lane,
                                           int lo, int m, int first, int j0k, int cntk,
-                                          const TeamBox& tb, bool filter, const UfArgs& uf)
+                                          const TeamBox& tb, bool filter, int part, int parts,
+                                          const UfArgs& uf)
 {
     const int start_k = warp_incl(cntk, lane) - cntk;
     const int total = __shfl_sync(kFull, start_k + cntk, 31);
     int nb = 0;                                 // candidates in the buffer
     // one pass past the end of the stream flushes the rest (team_flush is
     // inlined once)
-    for (int cb = 0; cb < total + kWarp; cb += kWarp) {
+    const int step = kSplit ? parts * kWarp : kWarp;
+    for (int cb = kSplit ? part * kWarp : 0; cb < total + step; cb += step) {
         const int t = cb + lane;
         bool jv = t < total;
         int k = 0;                              // last stream entry starting at or before t
 #pragma unroll
-        for (int step = 8; step; step >>= 1) {
-            const int probe = k + step <= 13 ? k + step : 13;
+        for (int half = 8; half; half >>= 1) {
+            const int probe = k + half <= 13 ? k + half : 13;
             const int sm = __shfl_sync(kFull, start_k, probe);
-            if (k + step <= 13 && sm <= t) k += step;
+            if (k + half <= 13 && sm <= t) k += half;
         }
         int j = __shfl_sync(kFull, j0k, k) + (t - __shfl_sync(kFull, start_k, k));
         float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -268,10 +272,15 @@ __device__ __forceinline__ void team_cell(TeamStage& S, int* __restrict__ parent
     }
 }
 
-template <bool kVar>
+// kSplit: each window is taken by `parts` warps, neighbours in the grid, that
+// all find its teams and their neighbour ranges and share the candidates
+// (small problems, which have fewer windows than the chip holds warps; 4,096
+// particles: 36 and 23 us).
+template <bool kVar, bool kSplit>
 __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4* __restrict__ sorted,
                                                        const int* __restrict__ cell_start, int* parent,
-                                                       int dense_min, UfArgs uf)
+                                                       int dense_min, int parts, int batch,
+                                                       unsigned* ticket, UfArgs uf)
 {
     pdl_wait();
     pdl_trigger();
@@ -286,19 +295,30 @@ __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4*
     const int lane = threadIdx.x & 31;
     TeamStage& S = stage[threadIdx.x >> 5];
     float4* pf = &ahead[threadIdx.x >> 5][0][0];
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    if (lane < 32)
-        S.lmask[lane] = 0u;
+    const unsigned total = (unsigned)g.total_n;         // slots fit in 31 bits
+    const unsigned nwarps = (gridDim.x * kLinkWarps) / (kSplit ? parts : 1);   // a multiple of parts
+    const unsigned warp = (blockIdx.x * kLinkWarps + (threadIdx.x >> 5)) / (kSplit ? parts : 1);
+    const int part = kSplit ? (int)((blockIdx.x * kLinkWarps + (threadIdx.x >> 5)) % parts) : 0;
+    S.lmask[lane] = 0u;
     __syncwarp();
-    if (warp * kWarp + lane < g.total_n)
-        cp_async16(pf + lane, sorted + warp * kWarp + lane);
+    // Batches of windows (a power of two each): a warp's first two by its number,
+    // the others by a ticket drawn two batches ahead.  Windows of blobs take ten
+    // times those of the background, and a warp sees too few of them to even out
+    // (a fixed share per warp against tickets, this kernel: 2 million particles
+    // 319 and 282 us, 453 million (768^3) 38.2 and 36.1 ms).
+    const unsigned span = (kSplit ? 1u : (unsigned)batch) * kWarp;
+    unsigned base = warp * span, next = (nwarps + warp) * span;
+    unsigned drawn = 0u;                                // lane 0: the batch after `next`
+    if (base + lane < total)
+        cp_async16(pf + lane, sorted + base + lane);
     cp_async_commit();
+    if (!kSplit && lane == 0)
+        drawn = atomicAdd(ticket, 1u);
 
-    int par = 0;
-    for (int64_t base = warp * kWarp; base < g.total_n; base += nwarps * kWarp, par ^= 1) {
-        const int64_t s = base + lane;
-        const bool valid = s < g.total_n;
+    for (int par = 0; base < total; par ^= 1) {
+        const unsigned s = base + lane;
+        const bool valid = s < total;
+        const unsigned ahead_base = ((base + kWarp) & (span - 1u)) != 0u ? base + kWarp : next;
         float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
         int bi = 0;
         Cell c{0, 0, 0};
@@ -308,8 +328,8 @@ __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4*
         if (valid)
             p = pf[par * kWarp + lane];
         // the other buffer was read one window ago: refill it
-        if (s + nwarps * kWarp < g.total_n)
-            cp_async16(pf + (par ^ 1) * kWarp + lane, sorted + s + nwarps * kWarp);
+        if (ahead_base + lane < total)
+            cp_async16(pf + (par ^ 1) * kWarp + lane, sorted + ahead_base + lane);
         cp_async_commit();
         if (valid) {
             bi = box_of(g.box_p0, g.nbox, s);
@@ -434,7 +454,8 @@ __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4*
             if (lane == 0)
                 S.box = tbx;
             __syncwarp();
-            team_cell<kVar>(S, parent, sorted, b, lane, lead, m, first, j0k, cntk, S.box, b.nc >= 3, uf);
+            team_cell<kVar, kSplit>(S, parent, sorted, b, lane, lead, m, first, j0k, cntk, S.box, b.nc >= 3, part,
+                                    parts, uf);
         }
 
         // ---- sparse particles: their (particle, cell) items, then their
@@ -485,7 +506,7 @@ __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4*
             }
             const int cstart = warp_incl(cnt, lane) - cnt;
             const int C = __shfl_sync(kFull, cstart + cnt, 31);
-            for (int cb = 0; cb < C; cb += kWarp) {
+            for (int cb = kSplit ? part * kWarp : 0; cb < C; cb += kSplit ? parts * kWarp : kWarp) {
                 const int u = cb + lane;
                 const bool uv = u < C;
                 const int it = owner_lane(cstart, uv ? u : C - 1);
@@ -500,6 +521,18 @@ __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4*
                         uunion<kVar>(parent, (int)(base + oo), jj, uf);
                 }
             }
+        }
+        if (((base + kWarp) & (span - 1u)) == 0u) {
+            base = next;
+            if constexpr (kSplit) {
+                next += nwarps * span;
+            } else {
+                next = (2u * nwarps + __shfl_sync(kFull, drawn, 0)) * span;
+                if (lane == 0)
+                    drawn = atomicAdd(ticket, 1u);
+            }
+        } else {
+            base += kWarp;
         }
     }
 }
@@ -1000,12 +1033,23 @@ cudaError_t launch_link(const Geometry& g, const Work& w, int dense_min, const U
 {
     if (g.total_n == 0)
         return cudaSuccess;
-    int64_t warps = (g.total_n + kWarp - 1) / kWarp;
-    int64_t blocks = (warps * kWarp + kLinkThreads - 1) / kLinkThreads;
-    int64_t cap = (int64_t)sm_count() * 8;
-    if (blocks > cap) blocks = cap;
-    return launch_next(g.total_n, uf.var ? k_link<true> : k_link<false>, blocks, kLinkThreads, 0, s, g, w.sorted,
-                       w.cell_start, w.parent, dense_min, uf);
+    const int64_t windows = (g.total_n + kWarp - 1) / kWarp;
+    const int64_t warps = (int64_t)sm_count() * kLinkBlocks * kLinkWarps;   // resident
+    // warps per window while half of the chip would have none, at most
+    // kLinkWarps (a CTA's warps are a whole number of windows)
+    int parts = 1;
+    while (parts < kLinkWarps && windows * parts * 2 <= warps / 2) parts *= 2;
+    // windows per ticket: 32 batches or more to a warp, and few enough tickets
+    // for their one counter (768^3 box: 40.4 ms with 1 window, 37.7 with 2, 36.1
+    // with 8, 36.7 with 32; 8 million particles: 703, 695 and, with 4, 741 us)
+    int batch = 1;
+    while (batch < 8 && windows >= warps * 64 * batch) batch *= 2;
+    int64_t blocks = (windows * parts + kLinkWarps - 1) / kLinkWarps;
+    if (blocks > warps / kLinkWarps) blocks = warps / kLinkWarps;
+    auto kernel = uf.var ? (parts > 1 ? k_link<true, true> : k_link<true, false>)
+                         : (parts > 1 ? k_link<false, true> : k_link<false, false>);
+    return launch_next(g.total_n, kernel, blocks, kLinkThreads, 0, s, g, w.sorted, w.cell_start, w.parent, dense_min,
+                       parts, batch, w.link_ticket, uf);
 }
 
 }  // namespace fofgpu

@@ -77,6 +77,8 @@ struct ResultsLayout {
     size_t status_off, groups_off, cat_off, bytes;
 };
 
+static_assert(sizeof(Status) <= 64, "the per-box counts follow at 64");
+
 ResultsLayout results_layout(int nbox)
 {
     ResultsLayout r;
@@ -467,6 +469,7 @@ void bind_workspace(char* ws, const Layout& L, const BoxDev* boxes, int nbox, in
     const ResultsLayout rl = results_layout(nbox);
     char* res = ws + L.results;
     w.status = (Status*)(res + rl.status_off);
+    w.link_ticket = &w.status->link_ticket;
     w.n_groups = (unsigned long long*)(res + rl.groups_off);
     w.n_cat = (unsigned long long*)(res + rl.cat_off);
     w.bcount = (int*)(ws + L.bcount);
