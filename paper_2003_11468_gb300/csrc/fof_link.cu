@@ -36,6 +36,12 @@ struct Cell {
     int cx, cy, cz;
 };
 
+// the cell of a window's particle (k_link: x | y << 16, z)
+__device__ __forceinline__ Cell cell_at(const int4& at)
+{
+    return Cell{at.x & 0xffff, at.x >> 16, at.y};
+}
+
 // cell_key with the Morton spreading of the in-brick coordinates (< 16)
 // read from a shared-memory table instead of computed
 __device__ __forceinline__ int64_t cell_key_tab(const BoxDev& b, int cx, int cy, int cz, const uint32_t* tab)
@@ -63,12 +69,12 @@ __device__ __forceinline__ int64_t nbr_key(const BoxDev& b, const Cell& c, int k
 
 // Neighbour k duplicates the own cell or an earlier neighbour (only when
 // fewer than 3 cells per axis).
-__device__ __forceinline__ bool nbr_duplicate(const BoxDev& b, const Cell& c, int k, int64_t self)
+__device__ __forceinline__ bool nbr_duplicate(const BoxDev& b, const Cell& c, int k)
 {
     if (b.nc >= 3)
         return false;
     int64_t key = nbr_key(b, c, k);
-    if (key == self)
+    if (key == cell_key(b, c.cx, c.cy, c.cz))
         return true;
     for (int q = 0; q < k; ++q)
         if (nbr_key(b, c, q) == key)
@@ -97,14 +103,6 @@ __device__ __forceinline__ unsigned reach_mask(const float4& p, const BoxDev& b,
     // k = 12: dz = dy = 0, dx = +1  (the order of fwd_offset)
     unsigned m9 = ((ym & 1u) ? xm : 0u) | ((ym & 2u) ? xm << 3 : 0u) | ((ym & 4u) ? xm << 6 : 0u);
     return (hz ? m9 : 0u) | (hy ? xm << 9 : 0u) | (hx << 12);
-}
-
-__device__ __forceinline__ float4 shfl4(float4 v, int src)
-{
-    v.x = __shfl_sync(kFull, v.x, src);
-    v.y = __shfl_sync(kFull, v.y, src);
-    v.z = __shfl_sync(kFull, v.z, src);
-    return v;
 }
 
 // Bounding box of the team's particles.
@@ -141,7 +139,7 @@ struct TeamStage {
 
 constexpr int kLinkThreads = 256;
 constexpr int kLinkWarps = kLinkThreads / 32;
-constexpr int kLinkBlocks = 4;   // resident CTAs per SM (64 registers)
+constexpr int kLinkBlocks = 5;   // resident CTAs per SM (48 registers)
 constexpr int kOwnCell = 13;     // stream index of a team's own cell (cells above kTeamSelfMax)
 
 // The buffered candidates S.cpos/cslot[0..c) of a team against its m
@@ -272,12 +270,13 @@ __device__ __forceinline__ void team_cell(TeamStage& S, int* __restrict__ parent
     }
 }
 
-// kSplit: each window is taken by `parts` warps, neighbours in the grid, that
-// all find its teams and their neighbour ranges and share the candidates
-// (small problems, which have fewer windows than the chip holds warps; 4,096
-// particles: 36 and 23 us).
+// kSplit (small problems, of no more than two windows to a resident warp): a
+// grid of one window per `parts` warps, neighbours in the grid, that all find
+// its teams and their neighbour ranges and share the candidates (4,096
+// particles, 8 warps and one: 23 and 36 us).  One window's chain counts there,
+// so these have 64 registers (300,007 particles: 76 us, with 48: 87).
 template <bool kVar, bool kSplit>
-__global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4* __restrict__ sorted,
+__global__ void __launch_bounds__(kLinkThreads, kSplit ? 4 : kLinkBlocks) k_link(Geometry g, const float4* __restrict__ sorted,
                                                        const int* __restrict__ cell_start, int* parent,
                                                        int dense_min, int parts, int batch,
                                                        unsigned* ticket, UfArgs uf)
@@ -292,23 +291,29 @@ __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4*
     // each lane's binned record of the warp's next window, copied ahead
     // (cp.async) while the current window is linked; two buffers
     __shared__ float4 ahead[kLinkWarps][2][kWarp];
+    // cell (x | y << 16, z) and box of each lane's particle, and the cell's end:
+    // read back where they are needed, like the record, because registers are
+    // what limits the warps per SM, and those the kernel (64 registers, 4 CTAs:
+    // 35.8 ms on the 768^3 box; 48, 5: 34.4; 40, 6, with 120 bytes spilled: 37.0)
+    __shared__ int4 where[kLinkWarps][kWarp];
     const int lane = threadIdx.x & 31;
     TeamStage& S = stage[threadIdx.x >> 5];
     float4* pf = &ahead[threadIdx.x >> 5][0][0];
+    int4* at = &where[threadIdx.x >> 5][0];
     const unsigned total = (unsigned)g.total_n;         // slots fit in 31 bits
     const unsigned nwarps = (gridDim.x * kLinkWarps) / (kSplit ? parts : 1);   // a multiple of parts
     const unsigned warp = (blockIdx.x * kLinkWarps + (threadIdx.x >> 5)) / (kSplit ? parts : 1);
     const int part = kSplit ? (int)((blockIdx.x * kLinkWarps + (threadIdx.x >> 5)) % parts) : 0;
     S.lmask[lane] = 0u;
     __syncwarp();
-    // Batches of windows (a power of two each): a warp's first two by its number,
-    // the others by a ticket drawn two batches ahead.  Windows of blobs take ten
-    // times those of the background, and a warp sees too few of them to even out
-    // (a fixed share per warp against tickets, this kernel: 2 million particles
-    // 319 and 282 us, 453 million (768^3) 38.2 and 36.1 ms).
+    // Batches of windows (a power of two each): a warp's first by its number, the
+    // others by a ticket drawn when the batch before is begun.  Windows of blobs
+    // take ten times those of the background, and a warp sees too few of them to
+    // even out (a fixed share per warp against tickets, this kernel: 2 million
+    // particles 319 and 282 us, 453 million (768^3) 38.2 and 36.1 ms).
     const unsigned span = (kSplit ? 1u : (unsigned)batch) * kWarp;
-    unsigned base = warp * span, next = (nwarps + warp) * span;
-    unsigned drawn = 0u;                                // lane 0: the batch after `next`
+    unsigned base = warp * span;
+    unsigned drawn = 0u;                                // lane 0: the next batch's ticket
     if (base + lane < total)
         cp_async16(pf + lane, sorted + base + lane);
     cp_async_commit();
@@ -318,47 +323,39 @@ __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4*
     for (int par = 0; base < total; par ^= 1) {
         const unsigned s = base + lane;
         const bool valid = s < total;
-        const unsigned ahead_base = ((base + kWarp) & (span - 1u)) != 0u ? base + kWarp : next;
-        float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
-        int bi = 0;
-        Cell c{0, 0, 0};
-        int64_t self = -1;
-        int c0 = 0, c1 = 0;
-        cp_async_wait_all();                    // this lane's copy of slot s
-        if (valid)
-            p = pf[par * kWarp + lane];
-        // the other buffer was read one window ago: refill it
-        if (ahead_base + lane < total)
-            cp_async16(pf + (par ^ 1) * kWarp + lane, sorted + ahead_base + lane);
-        cp_async_commit();
+        int c0 = 0;
+        bool sub = false, team = false;
+        cp_async_wait_all();
+        __syncwarp();                           // every lane's copy is in, and the last window's reads are done
+        const float4* rec = pf + par * kWarp;
         if (valid) {
-            bi = box_of(g.box_p0, g.nbox, s);
+            const int bi = box_of(g.box_p0, g.nbox, s);
             const BoxDev& b = g.boxes[bi];
-            c.cx = cell_coord(p.x, b);
-            c.cy = cell_coord(p.y, b);
-            c.cz = cell_coord(p.z, b);
-            self = cell_key_tab(b, c.cx, c.cy, c.cz, spread_tab);
+            const float4 p = rec[lane];
+            const int cx = cell_coord(p.x, b), cy = cell_coord(p.y, b), cz = cell_coord(p.z, b);
+            const int64_t self = cell_key_tab(b, cx, cy, cz, spread_tab);
             c0 = cell_start[self];
-            c1 = cell_start[self + 1];
+            const int c1 = cell_start[self + 1];
+            at[lane] = make_int4(cx | (cy << 16), cz, bi, c1);
+            sub = is_sub(c1 - c0, b, dense_min);
+            team = !sub && (c1 - c0) >= b.team_min;
         }
-        const bool sub = valid && is_sub(c1 - c0, g.boxes[bi], dense_min);
-        const bool team = valid && !sub && (c1 - c0) >= g.boxes[bi].team_min;
+        __syncwarp();
         unsigned tmask = __ballot_sync(kFull, team);
 
         // ---- team cells: the warp links each cell's members as a team ----
         while (tmask) {
             const int lead = __ffs(tmask) - 1;
-            const int64_t key = __shfl_sync(kFull, self, lead);
-            const bool mine = team && self == key;
+            // (a cell that holds particles is told by its first slot)
+            const int lead_c0 = __shfl_sync(kFull, c0, lead);
+            const bool mine = team && c0 == lead_c0;
             const unsigned peers = __ballot_sync(kFull, mine);
             tmask &= ~peers;
             const int m = __popc(peers);          // members: lanes lead .. lead + m - 1
-            const int tbi = __shfl_sync(kFull, bi, lead);
-            const BoxDev& b = g.boxes[tbi];
-            Cell tc;
-            tc.cx = __shfl_sync(kFull, c.cx, lead);
-            tc.cy = __shfl_sync(kFull, c.cy, lead);
-            tc.cz = __shfl_sync(kFull, c.cz, lead);
+            const int4 lead_at = at[lead];
+            const BoxDev& b = g.boxes[lead_at.z];
+            const Cell tc = cell_at(lead_at);
+            const float4 p = mine ? rec[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
             // coordinates are finite and >= 0 (x + 0 turns -0 into +0), so
             // their bit patterns order like the values: one integer
             // reduction per bound
@@ -381,13 +378,13 @@ __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4*
                 S.mroot[lane - lead] = ufind<kVar>(parent, (int)s, uf);
             }
             const int first = (int)__shfl_sync(kFull, s, lead);
-            const int cell_end = __shfl_sync(kFull, c1, lead);
-            const int cell_size = cell_end - __shfl_sync(kFull, c0, lead);
+            const int cell_end = lead_at.w;
+            const int cell_size = cell_end - lead_c0;
             // lane k < 13: neighbour k's range, if the team reaches it and
             // the dense kernels do not own it; lane 13: the own cell's
             // particles after the first member, for cells k_team_self skips
             int j0k = 0, cntk = 0;
-            if (lane < 13 && ((team_reach >> lane) & 1u) && !nbr_duplicate(b, tc, lane, key)) {
+            if (lane < 13 && ((team_reach >> lane) & 1u) && !nbr_duplicate(b, tc, lane)) {
                 const int64_t nk = nbr_key_tab(b, tc, lane, spread_tab);
                 const int j0 = cell_start[nk], j1 = cell_start[nk + 1];
                 if (j1 > j0 && !is_sub(j1 - j0, b, dense_min)) {
@@ -458,19 +455,30 @@ __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4*
                                     parts, uf);
         }
 
+        // the next window, into the buffer that was read one window ago
+        const bool last = ((base + kWarp) & (span - 1u)) == 0u;     // of its batch
+        unsigned next = base + kWarp;
+        if (last)
+            next = kSplit ? base + nwarps * span : (nwarps + __shfl_sync(kFull, drawn, 0)) * span;
+        if (next + lane < total)
+            cp_async16(pf + (par ^ 1) * kWarp + lane, sorted + next + lane);
+        cp_async_commit();
+
         // ---- sparse particles: their (particle, cell) items, then their
         // (particle, candidate) pairs, pooled across the warp ----
         const bool sparse = valid && !team && !sub;
         unsigned reach_s = 0u;
         int own_n = 0;
         if (sparse) {
-            const BoxDev& b = g.boxes[bi];
-            reach_s = reach_mask(p, b, c);
+            const int4 own_at = at[lane];
+            const BoxDev& b = g.boxes[own_at.z];
+            const Cell c = cell_at(own_at);
+            reach_s = reach_mask(rec[lane], b, c);
             if (b.nc < 3)
                 for (int k = 0; k < 13; ++k)
-                    if (((reach_s >> k) & 1u) && nbr_duplicate(b, c, k, self))
+                    if (((reach_s >> k) & 1u) && nbr_duplicate(b, c, k))
                         reach_s &= ~(1u << k);
-            own_n = c1 - (int)s - 1;
+            own_n = own_at.w - (int)s - 1;
         }
         const int nit = sparse ? (own_n > 0) + __popc(reach_s) : 0;
         const int istart = warp_incl(nit, lane) - nit;
@@ -483,20 +491,16 @@ __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4*
             const int r = t - __shfl_sync(kFull, istart, o);
             const int own_o = __shfl_sync(kFull, own_n, o);
             const unsigned reach_o = __shfl_sync(kFull, reach_s, o);
-            const int obi = __shfl_sync(kFull, bi, o);
-            Cell oc;
-            oc.cx = __shfl_sync(kFull, c.cx, o);
-            oc.cy = __shfl_sync(kFull, c.cy, o);
-            oc.cz = __shfl_sync(kFull, c.cz, o);
             int j0 = 0, cnt = 0;
             if (iv) {
                 if (own_o > 0 && r == 0) {
                     j0 = (int)(base + o) + 1;
                     cnt = own_o;
                 } else {
-                    const BoxDev& b = g.boxes[obi];
+                    const int4 o_at = at[o];
+                    const BoxDev& b = g.boxes[o_at.z];
                     const int k = nth_bit(reach_o, r - (own_o > 0));
-                    const int64_t nk = nbr_key_tab(b, oc, k, spread_tab);
+                    const int64_t nk = nbr_key_tab(b, cell_at(o_at), k, spread_tab);
                     const int a0 = cell_start[nk], a1 = cell_start[nk + 1];
                     if (!is_sub(a1 - a0, b, dense_min)) {
                         j0 = a0;
@@ -512,28 +516,18 @@ __global__ void __launch_bounds__(kLinkThreads) k_link(Geometry g, const float4*
                 const int it = owner_lane(cstart, uv ? u : C - 1);
                 int jj = __shfl_sync(kFull, j0, it) + (u - __shfl_sync(kFull, cstart, it));
                 const int oo = __shfl_sync(kFull, o, it);
-                const float4 po = shfl4(p, oo);
-                const int pbi = __shfl_sync(kFull, bi, oo);
                 if (uv) {
-                    const BoxDev& b = g.boxes[pbi];
+                    const float4 po = rec[oo];
+                    const BoxDev& b = g.boxes[at[oo].z];
                     FOF_DCHECK_SLOT(jj, b, uf.err);
                     if (linked(po, sorted[jj], b))
                         uunion<kVar>(parent, (int)(base + oo), jj, uf);
                 }
             }
         }
-        if (((base + kWarp) & (span - 1u)) == 0u) {
-            base = next;
-            if constexpr (kSplit) {
-                next += nwarps * span;
-            } else {
-                next = (2u * nwarps + __shfl_sync(kFull, drawn, 0)) * span;
-                if (lane == 0)
-                    drawn = atomicAdd(ticket, 1u);
-            }
-        } else {
-            base += kWarp;
-        }
+        base = next;
+        if (!kSplit && last && lane == 0)
+            drawn = atomicAdd(ticket, 1u);
     }
 }
 
@@ -1035,19 +1029,20 @@ cudaError_t launch_link(const Geometry& g, const Work& w, int dense_min, const U
         return cudaSuccess;
     const int64_t windows = (g.total_n + kWarp - 1) / kWarp;
     const int64_t warps = (int64_t)sm_count() * kLinkBlocks * kLinkWarps;   // resident
-    // warps per window while half of the chip would have none, at most
+    const bool split = windows <= 2 * warps;
+    // warps per window while a third of the chip would have none, at most
     // kLinkWarps (a CTA's warps are a whole number of windows)
     int parts = 1;
-    while (parts < kLinkWarps && windows * parts * 2 <= warps / 2) parts *= 2;
+    while (parts < kLinkWarps && windows * parts * 3 <= warps) parts *= 2;
     // windows per ticket: 32 batches or more to a warp, and few enough tickets
     // for their one counter (768^3 box: 40.4 ms with 1 window, 37.7 with 2, 36.1
     // with 8, 36.7 with 32; 8 million particles: 703, 695 and, with 4, 741 us)
     int batch = 1;
     while (batch < 8 && windows >= warps * 64 * batch) batch *= 2;
     int64_t blocks = (windows * parts + kLinkWarps - 1) / kLinkWarps;
-    if (blocks > warps / kLinkWarps) blocks = warps / kLinkWarps;
-    auto kernel = uf.var ? (parts > 1 ? k_link<true, true> : k_link<true, false>)
-                         : (parts > 1 ? k_link<false, true> : k_link<false, false>);
+    if (!split && blocks > warps / kLinkWarps) blocks = warps / kLinkWarps;
+    auto kernel = uf.var ? (split ? k_link<true, true> : k_link<true, false>)
+                         : (split ? k_link<false, true> : k_link<false, false>);
     return launch_next(g.total_n, kernel, blocks, kLinkThreads, 0, s, g, w.sorted, w.cell_start, w.parent, dense_min,
                        parts, batch, w.link_ticket, uf);
 }

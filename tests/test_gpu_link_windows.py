@@ -10,8 +10,8 @@ from paper_2003_11468_gb300 import synth
 pytestmark = pytest.mark.gpu
 
 
-# 8, 8, 8, 4, 2 and 1 warps per window
-@pytest.mark.parametrize("n", [33, 1_000, 9_727, 19_000, 38_911, 38_913])
+# 8, 8, 8, 4, 2, 2 and 1 warps per window, one window each up to 389,120 particles, then tickets
+@pytest.mark.parametrize("n", [33, 1_000, 9_727, 16_000, 32_000, 64_000, 100_000, 389_119, 389_153])
 @pytest.mark.parametrize("b", [0.2, 0.5])
 def test_small(cuda_lib, n, b):
     import torch
