@@ -367,8 +367,12 @@ __device__ __forceinline__ int code_of(const float4& p, const CodeGeo& c)
 // One CTA per brick of up to heavy_from particles.  A mean brick has 1,200
 // particles in 4,096 cells, most of them empty, and what bounds it is the
 // chain: load, histogram, scan, cursors, scatter.  So
-//   * the next brick's records are copied ahead into shared memory (cp.async;
-//     each thread reads back only its own copies) while this one is sorted;
+//   * the next brick's records are copied ahead into shared memory (cp.async)
+//     while this one is sorted;
+//   * the sort goes through the list of each slot's source, so that the four
+//     words of a slot are stored in slot order, as whole lines: stored from the
+//     particles' side they were 2.7 sectors a particle, which an SM writes at
+//     about two cycles each, two thirds of the kernel's time;
 //   * counts and cursors are 16-bit halves of shared-memory words, eight cells
 //     to a load, so two histograms fit and take turns (the one not in use is
 //     cleared meanwhile) and a brick takes three barriers;
@@ -377,21 +381,21 @@ __device__ __forceinline__ int code_of(const float4& p, const CodeGeo& c)
 // Warp w owns the cells of per_warp consecutive groups of eight, lane by lane,
 // so the histogram is read and written conflict-free; a lane's groups share one
 // warp scan as 16-bit fields.  Registers are what limits the copies and loads
-// in flight: a spill here costs 10 to 50%, because the scattered stores leave
-// little of L1.  Both sort kernels, before (1,024 threads, 32-bit counts, twelve
-// barriers) and after, us: 64 boxes of 36,000 particles 205 and 116, 16.8
-// million (256^3) 575 and 422, 512 boxes of 650,000 12850 and 8700, 453 million
-// (768^3) 12200 and 10900.
+// in flight: a spill here costs 10 to 50%.  Both sort kernels, before (1,024
+// threads, 32-bit counts, twelve barriers) and after, us: 4 million particles
+// (two steps) 537 and 254, 8 million 360 and 216, 512 boxes of 650,000 12850 and
+// 7500, 453 million (768^3) 12200 and 8990.
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortBlocks = 4;
-constexpr int kSortKeep = 3;                           // records of a brick copied ahead per thread
+constexpr int kSortKeep = 2;                           // records of a brick copied ahead per thread
 constexpr int kFlight = 2;                             // loads in flight per thread beyond them
 constexpr int kSortGroups = kMaxR3 / (8 * kSortThreads);   // groups of eight cells per lane
 static_assert(kSortGroups <= 4 && kBrickMax < 65536, "16-bit counts, four fields");
 
 struct SortSmem {
     float4 rec[2][kSortKeep * kSortThreads];
+    unsigned short source[kHeavyBrick];        // record that goes to each slot of the brick
     unsigned hist[2][kMaxR3 / 2];
     int part[kSortWarps];
     unsigned long long list_pack;
@@ -454,7 +458,6 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocks)
     int bi = 0, buf = 0, hb = 0;               // record buffer and histogram of this brick
     for (; gb < nb; gb += stride, buf ^= 1) {
         cp_async_wait_all();
-        fetch(n0, n1, buf ^ 1);                // each thread read its own copies there one brick ago
         const int a0 = s0, a1 = s1;
         s0 = n0;
         s1 = n1;
@@ -466,8 +469,11 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocks)
         }
         const float4* rec = S.rec[buf];
         unsigned* hist = S.hist[hb];
-        if (a1 - a0 > heavy_from)
-            continue;                          // k_brick_sort_heavy's (block-uniform)
+        if (a1 - a0 > heavy_from) {            // k_brick_sort_heavy's (block-uniform)
+            __syncthreads();                   // the last brick's records have been read
+            fetch(s0, s1, buf ^ 1);
+            continue;
+        }
         while (bi + 1 < g.nbox && g.box_brick0[bi + 1] <= gb) ++bi;
         const BoxDev& b = g.boxes[bi];
         const CodeGeo cg = code_geo(b);
@@ -493,8 +499,10 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocks)
                     bump(hist, code_of(v[i], cg));
         }
         __syncthreads();
-        // the other histogram was last used by the previous brick, which every
-        // thread has finished: cleared for the next one
+        // every thread has finished the previous brick: its record buffer takes
+        // the next one's
+        fetch(s0, s1, buf ^ 1);
+        // and its histogram is cleared for it
         for (int q = tid; q < kMaxR3 / 8; q += kSortThreads)
             reinterpret_cast<uint4*>(S.hist[hb ^ 1])[q] = make_uint4(0u, 0u, 0u, 0u);
         hb ^= 1;
@@ -582,37 +590,53 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocks)
             if (cells)
                 reserved = atomicAdd(list_counter(lists, tid), cells);
         }
+        if (n <= kHeavyBrick) {
+            // each slot's source, then all of the slot's words in slot order:
+            // the stores are whole lines
 #pragma unroll
-        for (int i = 0; i < kSortKeep; ++i) {
-            const int k = i * kSortThreads + tid;
-            if (k < n) {
-                const float4 v = rec[k];
-                const int slot = a0 + bump(hist, code[i]);
-                sorted[slot] = v;
-                minorig[slot] = __float_as_int(v.w);
+            for (int i = 0; i < kSortKeep; ++i) {
+                const int k = i * kSortThreads + tid;
+                if (k < n)
+                    S.source[bump(hist, code[i])] = (unsigned short)k;
             }
-        }
-        for (int kb = kSortKeep * kSortThreads + tid; kb < n; kb += kFlight * kSortThreads) {
-            float4 v[kFlight];
+            for (int kb = kSortKeep * kSortThreads + tid; kb < n; kb += kFlight * kSortThreads) {
+                float4 v[kFlight];
 #pragma unroll
-            for (int i = 0; i < kFlight; ++i)
-                if (kb + i * kSortThreads < n)
-                    v[i] = tmp[a0 + kb + i * kSortThreads];
+                for (int i = 0; i < kFlight; ++i)
+                    if (kb + i * kSortThreads < n)
+                        v[i] = tmp[a0 + kb + i * kSortThreads];
 #pragma unroll
-            for (int i = 0; i < kFlight; ++i)
-                if (kb + i * kSortThreads < n) {
-                    const int slot = a0 + bump(hist, code_of(v[i], cg));
-                    if (slot < a1) {
-                        sorted[slot] = v[i];
-                        minorig[slot] = __float_as_int(v[i].w);
-                    } else {
-                        atomicOr(err, kErrInternal);
+                for (int i = 0; i < kFlight; ++i)
+                    if (kb + i * kSortThreads < n) {
+                        const int at = bump(hist, code_of(v[i], cg));
+                        if (at < n)
+                            S.source[at] = (unsigned short)(kb + i * kSortThreads);
+                        else
+                            atomicOr(err, kErrInternal);
                     }
+            }
+            __syncthreads();
+            for (int t = tid; t < n; t += kSortThreads) {
+                const int k = min((int)S.source[t], n - 1);
+                const float4 v = k < kSortKeep * kSortThreads ? rec[k] : tmp[a0 + k];
+                sorted[a0 + t] = v;
+                minorig[a0 + t] = __float_as_int(v.w);
+                parent[a0 + t] = a0 + t;
+                cnt[a0 + t] = 1;
+            }
+        } else {
+            for (int k = tid; k < n; k += kSortThreads) {
+                const float4 v = k < kSortKeep * kSortThreads ? rec[k] : tmp[a0 + k];
+                const int slot = a0 + bump(hist, code_of(v, cg));
+                if (slot < a1) {
+                    sorted[slot] = v;
+                    minorig[slot] = __float_as_int(v.w);
+                } else {
+                    atomicOr(err, kErrInternal);
                 }
-        }
-        for (int k = a0 + tid; k < a1; k += kSortThreads) {
-            parent[k] = k;
-            cnt[k] = 1;
+                parent[a0 + k] = a0 + k;
+                cnt[a0 + k] = 1;
+            }
         }
         if (listed) {
             if (tid < 4)
@@ -647,8 +671,9 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocks)
 // equal share of the cells, whose counts it sums over the cluster through
 // distributed shared memory and turns into every CTA's cursors.  One CTA of
 // 1,024 threads took 570 us for the fullest brick of the 256^3 box (350,000
-// particles); the 150 bricks above kHeavyBrick together take 155 us here (260
-// with 1,024 threads per CTA, of which fewer clusters run at a time).
+// particles); the 150 bricks above kHeavyBrick together take 154 us here (260
+// with 1,024 threads per CTA, of which fewer clusters run at a time; 768^3 box,
+// fixed shares of the bricks against tickets: 4.48 and 2.88 ms).
 constexpr int kCluster = 8;
 constexpr int kHeavyThreads = 512;
 constexpr int kHeavyBlocks = 2;
@@ -657,7 +682,7 @@ static_assert(kMaxR3 / kCluster <= kHeavyThreads, "one cell per thread");
 
 __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kHeavyThreads, kHeavyBlocks)
     k_brick_sort_heavy(Geometry g, const float4* __restrict__ tmp, const int* bstart, const int* heavy,
-                       const int* n_heavy, float4* __restrict__ sorted,
+                       const int* n_heavy, int* __restrict__ ticket, float4* __restrict__ sorted,
                        int* __restrict__ parent, int* __restrict__ minorig, int* __restrict__ cnt,
                        int* __restrict__ cell_start, int dense_min, CellLists lists, int* __restrict__ err)
 {
@@ -669,10 +694,17 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kHeavyThreads
     __shared__ unsigned long long list_pack;
     __shared__ int list_base[4];
     __shared__ int cells_total;                    // particles in this CTA's cells
+    __shared__ int next_item;                      // rank 0's: the cluster's next brick
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const int n = *n_heavy;
-    for (int it = blockIdx.x / kCluster; it < n; it += gridDim.x / kCluster) {
+    // a cluster's first brick by its number, the others by ticket: the fullest
+    // brick of a box can hold a third of what all of them hold
+    int next = 0;
+    for (int it = blockIdx.x / kCluster; it < n; it = next) {
+        int drawn = 0;
+        if (rank == 0 && threadIdx.x == 0)
+            drawn = atomicAdd(ticket, 1);
         const int64_t gb = heavy[it];
         const int s0 = bstart[gb], s1 = bstart[gb + 1];
         const BoxDev& b = g.boxes[box_of(g.box_brick0, g.nbox, gb)];
@@ -715,9 +747,13 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kHeavyThreads
         unsigned long long at = 0ull;
         if (l >= 0)
             at = atomicAdd(&list_pack, list_one(l));
-        if (threadIdx.x == 0)
+        if (threadIdx.x == 0) {
             cells_total = total;
+            if (rank == 0)
+                next_item = (int)(gridDim.x / kCluster) + drawn;
+        }
         cluster.sync();
+        next = *cluster.map_shared_rank(&next_item, 0);
         int start = s0 + ex;
         for (int q = 0; q < rank; ++q)
             start += *cluster.map_shared_rank(&cells_total, q);
@@ -910,8 +946,8 @@ cudaError_t launch_brick_sort(const Geometry& g, const Work& w, int dense_min, c
         const int64_t most = (int64_t)sm_count() * kHeavyBlocks / kCluster;
         if (clusters > most) clusters = most;
         cudaError_t e = launch_next(g.total_n, k_brick_sort_heavy, clusters * kCluster, kHeavyThreads, 0, s, g, w.tmp,
-                                    w.bstart, w.heavy_list, w.n_heavy, w.sorted, w.parent, w.minorig, w.cnt,
-                                    w.cell_start, dense_min, lists, &w.status->err);
+                                    w.bstart, w.heavy_list, w.n_heavy, w.heavy_ticket, w.sorted, w.parent, w.minorig,
+                                    w.cnt, w.cell_start, dense_min, lists, &w.status->err);
         if (e != cudaSuccess) return e;
     }
     // the shared-memory opt-in is per device; setting it again is harmless

@@ -676,6 +676,7 @@ struct Work {
     unsigned long long* scan_state; // [scan_tiles] look-back words of the brick scan
     int* scan_ticket;   // scan tiles handed out
     int* n_heavy;       // bricks above heavy_from particles
+    int* heavy_ticket;  // heavy bricks handed out
     int* heavy_list;    // [total_n / kHeavyBrick + 1] their indices
     unsigned long long* tile_state; // look-back words of the output tiles, or of the scan of their counts
     int* tile_ticket;   // tiles handed out

@@ -67,7 +67,7 @@ constexpr int kDefaultDenseMin = 256;
 constexpr double kDefaultOccupancy = 0.30;
 constexpr int kDefaultTeamMin = 10;
 constexpr int kMinTeamMin = 2;                 // smallest team threshold in use
-constexpr int kNumCounters = 4;                 // dense, team (small, large), big cells
+constexpr int kNumCounters = 5;                 // dense, team (small, large), big cells; heavy bricks drawn
 constexpr int kCounterPad = 32;                // words between them: a 128-byte line each
 constexpr int kMaxCellsPerAxis = 4096;        // float32 cell-index precision (unsplit cells)
 constexpr int kMaxFinePerAxis = 16384;        // float32 index precision (sub-cells)
@@ -499,6 +499,7 @@ void bind_workspace(char* ws, const Layout& L, const BoxDev* boxes, int nbox, in
     w.n_team = counters + kCounterPad;
     w.n_team_hi = counters + 2 * kCounterPad;
     w.n_big = counters + 3 * kCounterPad;
+    w.heavy_ticket = counters + 4 * kCounterPad;
 }
 
 int dense_min_of(const fof_options* opt)
