@@ -548,16 +548,31 @@ __global__ void __launch_bounds__(kLinkThreads, kSplit ? 4 : kLinkBlocks) k_link
 // (one warp took 93,000 cycles for a cell of 256 when it sorted with a bitonic
 // network, mirrored blocks by a ballot per candidate and searched rows in
 // shared memory).  Before and after, us: 4,096 particles 78 and 14, 2 million
-// 153 and 57, 16.8 million (256^3) 642 and 348, 453 million (768^3) 13740 and
-// 9050.
+// 153 and 56, 16.8 million (256^3) 642 and 308, 453 million (768^3) 13740 and
+// 8150.
 constexpr int kTeamWarps = 4;
 constexpr int kTeamBlocks = 8;               // CTAs per SM (64 registers, 27 KB)
 constexpr int kZBins = 32;                   // z bins of the order of a team cell
 
+// The staged positions of a cell, axis by axis: one 16-byte load holds two
+// pairs of candidates for the packed arithmetic.
+template <int kMax>
+struct __align__(16) CellPos {
+    float x[kMax], y[kMax], z[kMax];
+
+    __device__ __forceinline__ void set(int k, float4 v)
+    {
+        x[k] = v.x;
+        y[k] = v.y;
+        z[k] = v.z;
+    }
+    __device__ __forceinline__ float4 get(int k) const { return make_float4(x[k], y[k], z[k], 0.f); }
+};
+
 struct TeamWarpSmem {                        // one warp's cell
     static constexpr int kWords = kTeamSplit / 32;
     static constexpr int kStride = kWords + 1;          // odd stride: conflict-free rows
-    float4 P[kTeamSplit];
+    CellPos<kTeamSplit> P;
     float4 Q[kTeamSplit];                    // the next cell, copied ahead
     unsigned adj[kTeamSplit * kStride];
     int bin[kZBins];
@@ -566,7 +581,7 @@ struct TeamWarpSmem {                        // one warp's cell
 struct TeamCtaSmem {                         // one CTA's cell
     static constexpr int kWords = kTeamSelfMax / 32;
     static constexpr int kStride = kWords + 1;
-    float4 P[kTeamSelfMax];
+    CellPos<kTeamSelfMax> P;
     unsigned adj[kTeamSelfMax * kStride];
     int bin[kZBins];
     unsigned todo[kWords];
@@ -589,46 +604,98 @@ __device__ __forceinline__ float4 far_point(float v)
     return make_float4(v, v, v, 0.f);
 }
 
-// Row word of particle pi against pj[0..jn8), jn8 a multiple of 8.  The float32
-// pre-test decides; pairs in the uncertainty band are noted and take the exact
-// test after the block, in a loop entered only when some lane has one.  Inside
-// one cell no pair needs the periodic wrap when the box has at least 3 cells
-// per axis (the cell side is then below L/2, so the wrapped float32 separation
-// equals the plain difference); kWrap takes the full predicate for boxes with
-// fewer cells.
-template <bool kWrap>
-__device__ __forceinline__ unsigned block_word(const float4& pi, const float4* pj, int jn8, const BoxDev& b)
+// Two float32 values in one register pair, and the packed operations on them
+// (each half rounded to nearest, as the single operation).
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi)
 {
-    const float t_lo = b.t_lo, t_hi = b.t_hi;
-    unsigned row = 0, band = 0;
-    for (int t0 = 0; t0 < jn8; t0 += 8) {
-        unsigned r8 = 0, b8 = 0;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const float4 q = pj[t0 + u];
-            float s2;
-            if (kWrap) {
-                s2 = d2_f32(pi, q, b.Lf);
-            } else {
-                const float dx = __fsub_rn(pi.x, q.x);
-                const float dy = __fsub_rn(pi.y, q.y);
-                const float dz = __fsub_rn(pi.z, q.z);
-                s2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
-            }
-            const bool hi = s2 <= t_hi;
-            if (hi)
-                r8 |= 1u << u;
-            if (hi && s2 >= t_lo)
-                b8 |= 1u << u;
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// Row word of particle pi against particles j0..j0+jn8 of the cell, jn8 a
+// multiple of 8 up to 32.  The float32 pre-test decides; pairs in the uncertainty
+// band are noted and take the exact test after the block, in a loop entered only
+// when some lane has one.  Inside one cell no pair needs the periodic wrap when
+// the box has at least 3 cells per axis (the cell side is then below L/2, so the
+// wrapped float32 separation equals the plain difference); kWrap takes the full
+// predicate for other boxes (plain_pairs).
+// Without the wrap, candidates go two to an operation, and the outcome of a
+// comparison is the sign of a difference, shifted into the word: s2 - t is
+// negative exactly when s2 < t (the rounded difference of two floats has the
+// sign of the exact one), and s2 <= t_hi when s2 is below the next float.  The
+// kernel is bound by issue, and this halves the instructions of a pair test:
+// k_team_self on the 768^3 box 9.05 ms with one candidate and one comparison at a
+// time, 8.15 so; 16.8 million particles (256^3) 348 and 308 us.
+__device__ __forceinline__ bool plain_pairs(const BoxDev& b)
+{
+    return b.nc >= 3 && b.t_hi <= FLT_MAX;     // a next float above t_hi exists
+}
+
+template <bool kWrap, int kMax>
+__device__ __forceinline__ unsigned block_word(const float4& pi, const CellPos<kMax>& P, int j0, int jn8,
+                                               const BoxDev& b)
+{
+    unsigned row = 0, certain = 0;
+    if constexpr (kWrap) {
+        for (int t = 0; t < jn8; ++t) {
+            const float s2 = d2_f32(pi, P.get(j0 + t), b.Lf);
+            row |= (unsigned)(s2 <= b.t_hi) << t;
+            certain |= (unsigned)(s2 < b.t_lo) << t;
         }
-        row |= r8 << t0;
-        band |= b8 << t0;
+    } else {
+        const unsigned long long nx = pack2(-pi.x, -pi.x), ny = pack2(-pi.y, -pi.y), nz = pack2(-pi.z, -pi.z);
+        const float above = __uint_as_float(__float_as_uint(b.t_hi) + 1u);     // t_hi > 0
+        const unsigned long long nhi = pack2(-above, -above), nlo = pack2(-b.t_lo, -b.t_lo);
+        for (int t0 = 0; t0 < jn8; t0 += 8) {
+#pragma unroll
+            for (int u = 0; u < 8; u += 4) {
+                const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(P.x + j0 + t0 + u);
+                const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(P.y + j0 + t0 + u);
+                const ulonglong2 z = *reinterpret_cast<const ulonglong2*>(P.z + j0 + t0 + u);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const unsigned long long dx = add2(h ? x.y : x.x, nx), dy = add2(h ? y.y : y.x, ny),
+                                             dz = add2(h ? z.y : z.x, nz);
+                    const unsigned long long s2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
+                    const unsigned long long hi = add2(s2, nhi), lo = add2(s2, nlo);
+                    row = __funnelshift_l((unsigned)hi, row, 1);
+                    row = __funnelshift_l((unsigned)(hi >> 32), row, 1);
+                    certain = __funnelshift_l((unsigned)lo, certain, 1);
+                    certain = __funnelshift_l((unsigned)(lo >> 32), certain, 1);
+                }
+            }
+        }
+        row = __brev(row) >> (32 - jn8);        // the first candidate was shifted in first
+        certain = __brev(certain) >> (32 - jn8);
     }
+    unsigned band = row & ~certain;
     if (__any_sync(kFull, band != 0u))
         while (band) {
             const int t = __ffs(band) - 1;
             band &= band - 1u;
-            if (!linked_exact_inl(pi, pj[t], b.L, b.l2))
+            if (!linked_exact_inl(pi, P.get(j0 + t), b.L, b.l2))
                 row &= ~(1u << t);
         }
     return row;
@@ -656,16 +723,16 @@ __device__ __forceinline__ int z_bin(float z, int cz, const BoxDev& b)
 
 // Adjacency block (ib, jb), jb >= ib, of the staged cell: its words and those
 // of the mirrored block.  `apart`: no pair of the block can be linked.
-template <int kStride>
-__device__ __forceinline__ void adjacency_block(const float4* P, unsigned* adj, int m, int ib, int jb, bool apart,
-                                                int lane, const BoxDev& b)
+template <int kStride, int kMax>
+__device__ __forceinline__ void adjacency_block(const CellPos<kMax>& P, unsigned* adj, int m, int ib, int jb,
+                                                bool apart, int lane, const BoxDev& b)
 {
     const int i = ib * 32 + lane;
     unsigned row = 0u;
     if (!apart) {
-        const float4 pi = i < m ? P[i] : far_point(-kFar);
+        const float4 pi = i < m ? P.get(i) : far_point(-kFar);
         const int jn8 = (min(32, m - jb * 32) + 7) & ~7;
-        row = b.nc >= 3 ? block_word<false>(pi, P + jb * 32, jn8, b) : block_word<true>(pi, P + jb * 32, jn8, b);
+        row = plain_pairs(b) ? block_word<false>(pi, P, jb * 32, jn8, b) : block_word<true>(pi, P, jb * 32, jn8, b);
     }
     if (jb == ib)
         row &= ~(1u << lane);                  // the particle itself
@@ -791,17 +858,17 @@ __device__ __forceinline__ void team_cell_cta(TeamCtaSmem& S, int c0, int m, flo
         const int k = r * kThreads + threadIdx.x;
         if (k < m) {
             const int at = S.bin[bin[r]] + rank[r];
-            S.P[at] = v[r];
+            S.P.set(at, v[r]);
             sorted[c0 + at] = v[r];
             minorig[c0 + at] = __float_as_int(v[r].w);
         } else if (k < nw * 32) {
-            S.P[k] = far_point(kFar);
+            S.P.set(k, far_point(kFar));
         }
     }
     __syncthreads();
     // the z range of each 32 particles: blocks too far apart hold no link
     for (int r = wid; r < nw; r += kTeamWarps) {
-        const unsigned z = __float_as_uint(S.P[r * 32 + lane].z + 0.f);    // finite and >= 0: ordered bits
+        const unsigned z = __float_as_uint(S.P.z[r * 32 + lane] + 0.f);    // finite and >= 0: ordered bits
         const bool in = r * 32 + lane < m;
         const unsigned lo = __reduce_min_sync(kFull, in ? z : 0x7f800000u), hi = __reduce_max_sync(kFull, in ? z : 0u);
         if (lane == 0) {
@@ -954,16 +1021,16 @@ __global__ void __launch_bounds__(kTeamWarps * 32, kTeamBlocks)
                 if (k < m) {
                     const int at = S.bin[place[r] >> 8] + (place[r] & 255);
                     const float4 v = S.Q[k];
-                    S.P[at] = v;
+                    S.P.set(at, v);
                     sorted[c0 + at] = v;
                     minorig[c0 + at] = __float_as_int(v.w);
                 }
             }
         } else if (lane < m) {                 // kSortMin <= 32: one particle per lane
-            S.P[lane] = S.Q[lane];
+            S.P.set(lane, S.Q[lane]);
         }
         if (nw * 32 - 32 + lane >= m)          // the ragged tail links nothing
-            S.P[nw * 32 - 32 + lane] = far_point(kFar);
+            S.P.set(nw * 32 - 32 + lane, far_point(kFar));
         __syncwarp();
         e = e_next;
         if (it + stride < n)
@@ -971,11 +1038,12 @@ __global__ void __launch_bounds__(kTeamWarps * 32, kTeamBlocks)
         e_next = it + 2 * stride < n ? list[it + 2 * stride] : 0;
 
         if (nw == 1) {
-            const float4 pi = lane < m ? S.P[lane] : far_point(-kFar);
+            const float4 pi = lane < m ? S.P.get(lane) : far_point(-kFar);
             const int jn8 = (m + 7) & ~7;
             unsigned rows[1][1];
-            rows[0][0] = (b.nc >= 3 ? block_word<false>(pi, S.P, jn8, b) : block_word<true>(pi, S.P, jn8, b)) &
-                         ~(1u << lane);
+            rows[0][0] =
+                (plain_pairs(b) ? block_word<false>(pi, S.P, 0, jn8, b) : block_word<true>(pi, S.P, 0, jn8, b)) &
+                ~(1u << lane);
             trace_components<1>(rows, parent, c0, lane);
             __syncwarp();                      // smem reused by the next cell
             continue;
@@ -984,7 +1052,7 @@ __global__ void __launch_bounds__(kTeamWarps * 32, kTeamBlocks)
         // pair's float32 separation squared exceeds t_hi; rounding is monotone)
         float zlo = 0.f, zhi = 0.f;            // lane r: the z range of block r
         for (int r = 0; r < nw; ++r) {
-            const unsigned z = __float_as_uint(S.P[r * 32 + lane].z + 0.f);    // finite and >= 0: ordered bits
+            const unsigned z = __float_as_uint(S.P.z[r * 32 + lane] + 0.f);    // finite and >= 0: ordered bits
             const bool in = r * 32 + lane < m;
             const unsigned lo = __reduce_min_sync(kFull, in ? z : 0x7f800000u),
                            hi = __reduce_max_sync(kFull, in ? z : 0u);

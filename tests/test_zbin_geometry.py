@@ -35,3 +35,17 @@ def test_bins_monotone_and_width(box, l_over_h, nc):
         for k in range(32):
             if np.any(bins == k):
                 assert F(highest[k] - width) <= lowest[k]
+
+
+@pytest.mark.parametrize("t_hi", [0.0, 1.4e-45, 1.2e-38, 3.7e-9, 0.04, 1.0, 16384.0, 3.4028235e38])
+def test_threshold_as_sign_of_a_difference(t_hi):
+    """s2 <= t_hi and s2 < t as the sign bit of s2 minus a float32, the form the
+    team kernel's packed pair tests take, on the neighbours of each threshold."""
+    t = F(t_hi)
+    with np.errstate(over="ignore"):
+        above = (t.view(np.uint32) + np.uint32(1)).view(F)
+        s2 = np.concatenate([t.view(np.uint32) + np.arange(-40, 40), [0, 1, 2, 0x00800000, 0x7f7fffff, 0x7f800000]])
+        s2 = np.clip(s2, 0, 0x7f800000).astype(np.uint32).view(F)
+        s2 = s2[~(np.isinf(s2) & np.isinf(above))]      # inf - inf: no sign on the device, and not <= t_hi
+        assert np.array_equal(np.signbit(s2 - above), s2 <= t)
+        assert np.array_equal(np.signbit(s2 - t), s2 < t)
