@@ -7,14 +7,15 @@
 //   scan         exclusive prefix sum of the brick counts
 //   bin_scatter  each particle to its brick's start + rank (float4: x, y, z,
 //                local index)
-//   brick_sort   one CTA per brick: cell histogram and scan in shared
+//   brick_sort   one CTA per brick (a cluster of eight for the few bricks
+//                that hold many particles): cell histogram and scan in shared
 //                memory, scatter into cell order, cell_start of the brick,
 //                and the forest initialisation parent[s] = s (Sec. 3.1)
 //
-// Bricks exist so that both atomics (brick cursors) and the scattered
-// writes stay in L2: the brick count is small enough that every brick's
-// write head is L2-resident, which turns the random-order scatter into
-// full-sector DRAM writes.
+// Bricks exist so that both the counters' atomics and the scattered writes
+// stay in L2: the brick count is small enough that every brick's write head
+// is L2-resident, which turns the random-order scatter into full-sector DRAM
+// writes.
 #include <cooperative_groups.h>
 
 #include "fof_internal.cuh"
@@ -52,10 +53,11 @@ __device__ __forceinline__ int64_t brick_of(const float* __restrict__ pos, int64
 // the same time and a brick's sectors fill up while they are in L2; CTAs that
 // stride over the input drift apart, and half-filled sectors leave L2 (768^3
 // box, scatter by the count's ranks: 11.8 ms striding, 6.5 ms by tiles; 7.9 ms
-// with a cursor atomic per particle instead).  The tiles of kBinStreams evenly spaced places of the input
-// take turns: inputs list a blob's particles one after the other, and tiles of
-// one place alone would all count into that blob's few bricks (a batch of 512
-// boxes: count 8.1 ms in input order, 2.5 ms with 64 places).
+// with a cursor atomic per particle instead).  The tiles of kBinStreams evenly
+// spaced places of the input take turns: inputs list a blob's particles one
+// after the other, and tiles of one place alone would all count into that
+// blob's few bricks (a batch of 512 boxes: count 8.1 ms in input order, 2.5 ms
+// with 64 places).
 //
 // The particle's rank in its brick (what the count's atomic returns) goes to
 // rank[i], so that the scatter needs no atomic.  The counters lie `pad` words

@@ -34,8 +34,8 @@
 // thread per particle or sub-cell and united it with each sub-cell of the
 // window whose recorded root looked different, which is every one of them
 // once the group's root has moved.  dense_self + dense_pairs before and after,
-// us: 60,000 particles 359 and 66, 2 million 422 and 107, 16.8 million (256^3)
-// 1107 and 395, 453 million (768^3) 8328 and 4435.
+// us: 60,000 particles 359 and 66, 2 million 422 and 95, 16.8 million (256^3)
+// 1107 and 370, 453 million (768^3) 8328 and 3940.
 #include "fof_internal.cuh"
 
 namespace fofgpu {

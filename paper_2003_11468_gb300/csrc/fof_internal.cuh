@@ -716,11 +716,10 @@ int sm_count();
 
 cudaError_t launch_bin_count(const float* pos, const Geometry& g, const Work& w, cudaStream_t s);
 // (of a run over n particles) exclusive prefix sum of in[i * pad], i < len,
-// into out[0..len]; state
-// (scan_tiles(len) words) and ticket start at zero; entries above heavy_from
-// are listed in `heavy` unless it is null
-cudaError_t launch_scan(int64_t n, const int* in, int pad, int* out, int64_t len, unsigned long long* state, int* ticket,
-                        int heavy_from, int* heavy, int* n_heavy, int* err, cudaStream_t s);
+// into out[0..len]; state (scan_tiles(len) words) and ticket start at zero;
+// entries above heavy_from are listed in `heavy` unless it is null
+cudaError_t launch_scan(int64_t n, const int* in, int pad, int* out, int64_t len, unsigned long long* state,
+                        int* ticket, int heavy_from, int* heavy, int* n_heavy, int* err, cudaStream_t s);
 int heavy_from(int64_t total_n);
 bool heavy_bricks(int64_t total_n);   // whether a brick can be above heavy_from
 int64_t scan_tiles(int64_t len);

@@ -276,10 +276,9 @@ __device__ __forceinline__ void team_cell(TeamStage& S, int* __restrict__ parent
 // particles, 8 warps and one: 23 and 36 us).  One window's chain counts there,
 // so these have 64 registers (300,007 particles: 76 us, with 48: 87).
 template <bool kVar, bool kSplit>
-__global__ void __launch_bounds__(kLinkThreads, kSplit ? 4 : kLinkBlocks) k_link(Geometry g, const float4* __restrict__ sorted,
-                                                       const int* __restrict__ cell_start, int* parent,
-                                                       int dense_min, int parts, int batch,
-                                                       unsigned* ticket, UfArgs uf)
+__global__ void __launch_bounds__(kLinkThreads, kSplit ? 4 : kLinkBlocks)
+    k_link(Geometry g, const float4* __restrict__ sorted, const int* __restrict__ cell_start, int* parent,
+           int dense_min, int parts, int batch, unsigned* ticket, UfArgs uf)
 {
     pdl_wait();
     pdl_trigger();
@@ -548,8 +547,8 @@ __global__ void __launch_bounds__(kLinkThreads, kSplit ? 4 : kLinkBlocks) k_link
 // (one warp took 93,000 cycles for a cell of 256 when it sorted with a bitonic
 // network, mirrored blocks by a ballot per candidate and searched rows in
 // shared memory).  Before and after, us: 4,096 particles 78 and 14, 2 million
-// 153 and 56, 16.8 million (256^3) 642 and 308, 453 million (768^3) 13740 and
-// 8150.
+// 153 and 51, 16.8 million (256^3) 642 and 266, 453 million (768^3) 13740 and
+// 6900.
 constexpr int kTeamWarps = 4;
 constexpr int kTeamBlocks = 8;               // CTAs per SM (64 registers, 27 KB)
 constexpr int kZBins = 32;                   // z bins of the order of a team cell
@@ -634,70 +633,90 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
     return r;
 }
 
-// Row word of particle pi against particles j0..j0+jn8 of the cell, jn8 a
-// multiple of 8 up to 32.  The float32 pre-test decides; pairs in the uncertainty
-// band are noted and take the exact test after the block, in a loop entered only
-// when some lane has one.  Inside one cell no pair needs the periodic wrap when
-// the box has at least 3 cells per axis (the cell side is then below L/2, so the
-// wrapped float32 separation equals the plain difference); kWrap takes the full
-// predicate for other boxes (plain_pairs).
-// Without the wrap, candidates go two to an operation, and the outcome of a
-// comparison is the sign of a difference, shifted into the word: s2 - t is
-// negative exactly when s2 < t (the rounded difference of two floats has the
-// sign of the exact one), and s2 <= t_hi when s2 is below the next float.  The
-// kernel is bound by issue, and this halves the instructions of a pair test:
-// k_team_self on the 768^3 box 9.05 ms with one candidate and one comparison at a
-// time, 8.15 so; 16.8 million particles (256^3) 348 and 308 us.
+// Inside one cell no pair needs the periodic wrap when the box has at least 3
+// cells per axis: the cell side is then below L/2, so the wrapped float32
+// separation equals the plain difference.
 __device__ __forceinline__ bool plain_pairs(const BoxDev& b)
 {
-    return b.nc >= 3 && b.t_hi <= FLT_MAX;     // a next float above t_hi exists
+    return b.nc >= 3 && b.t_hi <= FLT_MAX;     // block_word: a next float above t_hi exists
 }
 
-template <bool kWrap, int kMax>
+// The pairs of `band` (bits of a row word) by the exact test; x points to the
+// block's first candidate, the other axes follow `axis` words apart.
+static __device__ __noinline__ unsigned settle_band(unsigned row, unsigned band, float px, float py, float pz,
+                                                    const float* x, int axis, const BoxDev& b)
+{
+    while (band) {
+        const int t = __ffs(band) - 1;
+        band &= band - 1u;
+        const float* q = x + t;
+        if (!linked_exact_inl(make_float4(px, py, pz, 0.f), make_float4(q[0], q[axis], q[2 * axis], 0.f), b.L, b.l2))
+            row &= ~(1u << t);
+    }
+    return row;
+}
+
+// Row word with the periodic predicate.
+static __device__ __noinline__ unsigned wrapped_word(float px, float py, float pz, const float* x, int axis, int jn8,
+                                                     const BoxDev& b)
+{
+    unsigned row = 0, band = 0;
+    for (int t = 0; t < jn8; ++t) {
+        const float* q = x + t;
+        const float s2 = d2_f32(make_float4(px, py, pz, 0.f), make_float4(q[0], q[axis], q[2 * axis], 0.f), b.Lf);
+        row |= (unsigned)(s2 <= b.t_hi) << t;
+        band |= (unsigned)(s2 <= b.t_hi && s2 >= b.t_lo) << t;
+    }
+    return settle_band(row, band, px, py, pz, x, axis, b);
+}
+
+// Row word of particle pi against particles j0..j0+jn8 of the cell, jn8 a
+// multiple of 8 up to 32.  The float32 pre-test decides; pairs in the uncertainty
+// band are noted and take the exact test after the block, entered only when some
+// lane has one.  Candidates go two to an operation, and the outcome of a
+// comparison is the sign of a difference, shifted into the word: s2 - t is
+// negative exactly when s2 < t (the rounded difference of two floats has the
+// sign of the exact one), and s2 <= t_hi when s2 is below the next float.
+// The kernel is bound by issue, and this halves the instructions of a pair test
+// (k_team_self on the 768^3 box 9.05 ms with one candidate and one comparison at
+// a time, 8.25 so).  Its 32 warps per SM are at 32 different places of the code,
+// so what is rare (the band, the wrap) is out of line and the loop of a warp's
+// cell stands once for cells of every size: with copies in line the warps waited
+// for instructions most of all (8.25 ms, 6.9 without; 256^3 309 and 266 us).
+template <int kMax>
 __device__ __forceinline__ unsigned block_word(const float4& pi, const CellPos<kMax>& P, int j0, int jn8,
                                                const BoxDev& b)
 {
+    if (!plain_pairs(b))
+        return wrapped_word(pi.x, pi.y, pi.z, P.x + j0, kMax, jn8, b);
     unsigned row = 0, certain = 0;
-    if constexpr (kWrap) {
-        for (int t = 0; t < jn8; ++t) {
-            const float s2 = d2_f32(pi, P.get(j0 + t), b.Lf);
-            row |= (unsigned)(s2 <= b.t_hi) << t;
-            certain |= (unsigned)(s2 < b.t_lo) << t;
-        }
-    } else {
-        const unsigned long long nx = pack2(-pi.x, -pi.x), ny = pack2(-pi.y, -pi.y), nz = pack2(-pi.z, -pi.z);
-        const float above = __uint_as_float(__float_as_uint(b.t_hi) + 1u);     // t_hi > 0
-        const unsigned long long nhi = pack2(-above, -above), nlo = pack2(-b.t_lo, -b.t_lo);
-        for (int t0 = 0; t0 < jn8; t0 += 8) {
+    const unsigned long long nx = pack2(-pi.x, -pi.x), ny = pack2(-pi.y, -pi.y), nz = pack2(-pi.z, -pi.z);
+    const float above = __uint_as_float(__float_as_uint(b.t_hi) + 1u);     // t_hi > 0
+    const unsigned long long nhi = pack2(-above, -above), nlo = pack2(-b.t_lo, -b.t_lo);
+#pragma unroll 1
+    for (int t0 = 0; t0 < jn8; t0 += 8) {
 #pragma unroll
-            for (int u = 0; u < 8; u += 4) {
-                const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(P.x + j0 + t0 + u);
-                const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(P.y + j0 + t0 + u);
-                const ulonglong2 z = *reinterpret_cast<const ulonglong2*>(P.z + j0 + t0 + u);
+        for (int u = 0; u < 8; u += 4) {
+            const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(P.x + j0 + t0 + u);
+            const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(P.y + j0 + t0 + u);
+            const ulonglong2 z = *reinterpret_cast<const ulonglong2*>(P.z + j0 + t0 + u);
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const unsigned long long dx = add2(h ? x.y : x.x, nx), dy = add2(h ? y.y : y.x, ny),
-                                             dz = add2(h ? z.y : z.x, nz);
-                    const unsigned long long s2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
-                    const unsigned long long hi = add2(s2, nhi), lo = add2(s2, nlo);
-                    row = __funnelshift_l((unsigned)hi, row, 1);
-                    row = __funnelshift_l((unsigned)(hi >> 32), row, 1);
-                    certain = __funnelshift_l((unsigned)lo, certain, 1);
-                    certain = __funnelshift_l((unsigned)(lo >> 32), certain, 1);
-                }
+            for (int h = 0; h < 2; ++h) {
+                const unsigned long long dx = add2(h ? x.y : x.x, nx), dy = add2(h ? y.y : y.x, ny),
+                                         dz = add2(h ? z.y : z.x, nz);
+                const unsigned long long s2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
+                const unsigned long long hi = add2(s2, nhi), lo = add2(s2, nlo);
+                row = __funnelshift_l((unsigned)hi, row, 1);
+                row = __funnelshift_l((unsigned)(hi >> 32), row, 1);
+                certain = __funnelshift_l((unsigned)lo, certain, 1);
+                certain = __funnelshift_l((unsigned)(lo >> 32), certain, 1);
             }
         }
-        row = __brev(row) >> (32 - jn8);        // the first candidate was shifted in first
-        certain = __brev(certain) >> (32 - jn8);
     }
-    unsigned band = row & ~certain;
+    row = __brev(row) >> (32 - jn8);            // the first candidate was shifted in first
+    const unsigned band = row & ~(__brev(certain) >> (32 - jn8));
     if (__any_sync(kFull, band != 0u))
-        while (band) {
-            const int t = __ffs(band) - 1;
-            band &= band - 1u;
-            if (!linked_exact_inl(pi, P.get(j0 + t), b.L, b.l2))
-                row &= ~(1u << t);
-        }
+        row = settle_band(row, band, pi.x, pi.y, pi.z, P.x + j0, kMax, b);
     return row;
 }
 
@@ -721,22 +740,25 @@ __device__ __forceinline__ int z_bin(float z, int cz, const BoxDev& b)
     return min(max(k, 0), kZBins - 1);
 }
 
-// Adjacency block (ib, jb), jb >= ib, of the staged cell: its words and those
-// of the mirrored block.  `apart`: no pair of the block can be linked.
-template <int kStride, int kMax>
-__device__ __forceinline__ void adjacency_block(const CellPos<kMax>& P, unsigned* adj, int m, int ib, int jb,
-                                                bool apart, int lane, const BoxDev& b)
+// Row word of block (ib, jb), jb >= ib, of the staged cell.  `apart`: no pair of
+// the block can be linked.
+template <int kMax>
+__device__ __forceinline__ unsigned block_row(const CellPos<kMax>& P, int m, int ib, int jb, bool apart, int lane,
+                                              const BoxDev& b)
 {
+    if (apart)
+        return 0u;
     const int i = ib * 32 + lane;
-    unsigned row = 0u;
-    if (!apart) {
-        const float4 pi = i < m ? P.get(i) : far_point(-kFar);
-        const int jn8 = (min(32, m - jb * 32) + 7) & ~7;
-        row = plain_pairs(b) ? block_word<false>(pi, P, jb * 32, jn8, b) : block_word<true>(pi, P, jb * 32, jn8, b);
-    }
-    if (jb == ib)
-        row &= ~(1u << lane);                  // the particle itself
-    adj[i * kStride + jb] = row;
+    const float4 pi = i < m ? P.get(i) : far_point(-kFar);
+    const unsigned row = block_word(pi, P, jb * 32, (min(32, m - jb * 32) + 7) & ~7, b);
+    return jb == ib ? row & ~(1u << lane) : row;               // not the particle itself
+}
+
+// The block's words in the adjacency rows, and those of the mirrored block.
+template <int kStride>
+__device__ __forceinline__ void put_block(unsigned* adj, unsigned row, int ib, int jb, bool apart, int lane)
+{
+    adj[(ib * 32 + lane) * kStride + jb] = row;
     if (jb != ib)
         adj[(jb * 32 + lane) * kStride + ib] = apart ? 0u : transpose32(row, lane);
 }
@@ -885,8 +907,8 @@ __device__ __forceinline__ void team_cell_cta(TeamCtaSmem& S, int c0, int m, flo
         }
         jb += ib;
         const float gap = __fsub_rn(S.zlo[jb], S.zhi[ib]);
-        adjacency_block<kStride>(S.P, S.adj, m, ib, jb, b.nc >= 3 && gap > 0.f && __fmul_rn(gap, gap) > b.t_hi, lane,
-                                 b);
+        const bool apart = b.nc >= 3 && gap > 0.f && __fmul_rn(gap, gap) > b.t_hi;
+        put_block<kStride>(S.adj, block_row(S.P, m, ib, jb, apart, lane, b), ib, jb, apart, lane);
     }
     __syncthreads();
     // warp w searches row blocks w and w + kTeamWarps; the frontier's words are
@@ -1037,21 +1059,10 @@ __global__ void __launch_bounds__(kTeamWarps * 32, kTeamBlocks)
             team_fetch(S, e, sorted, lane);
         e_next = it + 2 * stride < n ? list[it + 2 * stride] : 0;
 
-        if (nw == 1) {
-            const float4 pi = lane < m ? S.P.get(lane) : far_point(-kFar);
-            const int jn8 = (m + 7) & ~7;
-            unsigned rows[1][1];
-            rows[0][0] =
-                (plain_pairs(b) ? block_word<false>(pi, S.P, 0, jn8, b) : block_word<true>(pi, S.P, 0, jn8, b)) &
-                ~(1u << lane);
-            trace_components<1>(rows, parent, c0, lane);
-            __syncwarp();                      // smem reused by the next cell
-            continue;
-        }
         // 32 to a block, in z order: blocks too far apart hold no link (every
         // pair's float32 separation squared exceeds t_hi; rounding is monotone)
         float zlo = 0.f, zhi = 0.f;            // lane r: the z range of block r
-        for (int r = 0; r < nw; ++r) {
+        for (int r = 0; nw > 1 && r < nw; ++r) {
             const unsigned z = __float_as_uint(S.P.z[r * 32 + lane] + 0.f);    // finite and >= 0: ordered bits
             const bool in = r * 32 + lane < m;
             const unsigned lo = __reduce_min_sync(kFull, in ? z : 0x7f800000u),
@@ -1059,14 +1070,21 @@ __global__ void __launch_bounds__(kTeamWarps * 32, kTeamBlocks)
             zlo = lane == r ? __uint_as_float(lo) : zlo;
             zhi = lane == r ? __uint_as_float(hi) : zhi;
         }
+        unsigned rows[1][1];                   // the last block's words
+#pragma unroll 1
         for (int ib = 0; ib < nw; ++ib)
+#pragma unroll 1
             for (int jb = ib; jb < nw; ++jb) {
                 const float gap = __fsub_rn(__shfl_sync(kFull, zlo, jb), __shfl_sync(kFull, zhi, ib));
-                adjacency_block<TeamWarpSmem::kStride>(
-                    S.P, S.adj, m, ib, jb, b.nc >= 3 && gap > 0.f && __fmul_rn(gap, gap) > b.t_hi, lane, b);
+                const bool apart = b.nc >= 3 && ib != jb && gap > 0.f && __fmul_rn(gap, gap) > b.t_hi;
+                rows[0][0] = block_row(S.P, m, ib, jb, apart, lane, b);
+                if (nw > 1)
+                    put_block<TeamWarpSmem::kStride>(S.adj, rows[0][0], ib, jb, apart, lane);
             }
         __syncwarp();
-        if (nw == 2)
+        if (nw == 1)
+            trace_components<1>(rows, parent, c0, lane);
+        else if (nw == 2)
             trace_staged<2>(S, parent, c0, lane);
         else if (nw == 3)
             trace_staged<3>(S, parent, c0, lane);

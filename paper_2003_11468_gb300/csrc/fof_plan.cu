@@ -401,8 +401,8 @@ struct fof_plan {
 namespace {
 
 struct Layout {
-    size_t boxes, p0, brick0, results, bcount, bstart, scan_state, scan_ticket, heavy_list, tile_state, tile_ticket, out_cursor, tile_off,
-        cell_start, tmp, sorted, parent, minorig, cnt, dense_list, counters, dense_root, team_list, big_list, total;
+    size_t boxes, p0, brick0, results, bcount, bstart, scan_state, scan_ticket, heavy_list, tile_state, tile_ticket,
+        out_cursor, tile_off, cell_start, tmp, sorted, parent, minorig, cnt, dense_list, counters, dense_root, team_list, big_list, total;
     size_t zero_end;     // [bcount, zero_end) starts each run at zero
     int64_t n_tiles, dense_cap, team_cap;
 };
