@@ -11,6 +11,8 @@
 //              per-box group and catalogue counts.
 //   catalogue  ids[i] = smallest index of i's group; sizes[label] = size, 0
 //              elsewhere; (label, size) entries in ascending label order.
+#include <algorithm>
+
 #include "fof_internal.cuh"
 
 namespace fofgpu {
@@ -19,9 +21,8 @@ namespace {
 
 // Root of slot s by a plain walk, then parent[s] = root.  `ordered`: every
 // parent is at most its child (hooks onto the smaller root), checked.
-__device__ __forceinline__ int final_root(int* __restrict__ parent, int s, bool ordered, int* err)
+__device__ __forceinline__ int final_root(int* __restrict__ parent, int s, int p, bool ordered, int* err)
 {
-    const int p = parent[s];
     if (p == s)
         return s;
     int x = p;
@@ -39,6 +40,9 @@ __device__ __forceinline__ int final_root(int* __restrict__ parent, int s, bool 
     return x;
 }
 
+// Bound by the latency of the walk to the root, so a slot's own words are read
+// one slot ahead (453 million slots: 1.97 and 1.54 ms; with 16 CTAs per SM in
+// the grid instead of 8, 1.48).
 __global__ void __launch_bounds__(256) k_finalize(int64_t total, int* __restrict__ parent,
                                                   int* __restrict__ minorig, int* __restrict__ cnt,
                                                   int* __restrict__ err, bool ordered)
@@ -46,20 +50,32 @@ __global__ void __launch_bounds__(256) k_finalize(int64_t total, int* __restrict
     pdl_wait();
     pdl_trigger();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < total; base += stride) {
-        int64_t s = base + threadIdx.x;
-        bool valid = s < total;
+    int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int p_next = 0, mo_next = 0;
+    if (s < total) {
+        p_next = parent[s];
+        mo_next = minorig[s];
+    }
+    for (; s - threadIdx.x < total; s += stride) {
+        const bool valid = s < total;
+        const int p = p_next, mo = mo_next;
+        // the next slot's words: only this thread writes them, unless the slot
+        // is a root, whose words are not used
+        if (s + stride < total) {
+            p_next = parent[s + stride];
+            mo_next = minorig[s + stride];
+        }
         unsigned active = __ballot_sync(kFull, valid);
         if (!valid)
             continue;
-        const int root = final_root(parent, (int)s, ordered, err);
+        const int root = final_root(parent, (int)s, p, ordered, err);
         bool nonroot = root != (int)s;
         unsigned nr = __ballot_sync(active, nonroot);
         if (!nonroot)
             continue;
         unsigned peers = __match_any_sync(nr, root);
         int leader = __ffs(peers) - 1;
-        unsigned mn = __reduce_min_sync(peers, (unsigned)minorig[s]);
+        unsigned mn = __reduce_min_sync(peers, (unsigned)mo);
         if ((threadIdx.x & 31) == leader) {
             atomicAdd(cnt + root, __popc(peers));
             atomicMin(minorig + root, (int)mn);
@@ -95,7 +111,7 @@ __global__ void __launch_bounds__(256) k_finalize_hash(int64_t total, int* __res
             const int64_t s = b0 + (int64_t)t * blockDim.x + threadIdx.x;
             if (s >= total)
                 break;
-            const int root = final_root(parent, (int)s, ordered, err);
+            const int root = final_root(parent, (int)s, parent[s], ordered, err);
             if (root == (int)s)
                 continue;
             const int mo = minorig[s];
@@ -160,9 +176,9 @@ __global__ void __launch_bounds__(256) k_finalize_hash(int64_t total, int* __res
 //            are appended to the bucket of the input's tile instead, whose
 //            write heads stay in L2.  A tile holds exactly kOutTile inputs (the
 //            last one fewer), so bucket t starts at t * kOutTile.  (Direct and
-//            bucketed, this kernel: 2 million inputs 25 and 270 us, the
-//            buckets' cursors sharing lines; 16.7 million 0.27 and 0.38 ms;
-//            453 million 17.2 and 7.4 ms.)
+//            bucketed, this kernel when its CTAs strode over the slots: 2
+//            million inputs 25 and 270 us, the buckets' cursors sharing lines;
+//            16.7 million 0.27 and 0.38 ms; 453 million 17.2 and 7.4 ms.)
 //   write    one CTA per tile: ids and sizes written out coalesced (a bucket's
 //            pairs placed in shared memory first), and the tile's catalogue
 //            entries (sizes at least thr, ascending label).  Up to kDirectMax
@@ -172,43 +188,77 @@ __global__ void __launch_bounds__(256) k_finalize_hash(int64_t total, int* __res
 //            the tiles takes longer than the tiles themselves (453 million
 //            inputs: 2.6 ms), so the kernel leaves the tile's count, and a
 //            scan and k_catalogue follow (1.3 ms in all).
+constexpr int kScatterThreads = 256, kScatterWarps = kScatterThreads / 32;
+constexpr int kScatterTiles = 4;             // tiles of kScatterThreads slots per CTA
+constexpr int kScatterStreams = 64;          // places of the slots that take turns (buckets)
+
+// Bound by the scattered stores and the cursors' atomics.  A slot's words are
+// read one slot ahead, and nothing waits for another load but the group's words
+// for the root.  A CTA takes kScatterTiles consecutive tiles, and CTAs start in
+// order, so that the slots at work lie close together; CTAs that stride over the
+// slots drift apart, and a sector of the pairs is written in several pieces.
+// Buckets: neighbouring slots also use the same few cursors (a batch's boxes have
+// a hundred each), so chunks of kScatterStreams evenly spaced places take turns
+// (a batch of 512 boxes: 21.1 ms with 1 place, 4.1 with 16, 3.3 with 64 and 256).
+// The box counters get one addition per CTA: one per warp would be more atomics
+// on one address than the rest takes.  Striding before and so, us: 2 million slots
+// 25 and 20, 16.8 million 261 and 233 (1 tile: 222, but 7.8 instead of 5.6 ms in
+// the 768^3 box, and 70 instead of 49 for 4 million), 453 million 7370 and 5620,
+// the batch 4430 and 3270.
+
 template <bool kDirect>
-__global__ void __launch_bounds__(256) k_outputs_scatter(Geometry g, const float4* sorted, const int* parent,
+__global__ void __launch_bounds__(kScatterThreads) k_outputs_scatter(Geometry g, const float4* sorted,
+                                                         const int* parent,
                                                          const int* minorig, const int* cnt, int32_t thr,
                                                          unsigned long long* __restrict__ n_groups,
                                                          unsigned long long* __restrict__ n_cat,
                                                          int2* __restrict__ pairs,
-                                                         int* __restrict__ out_cursor, int* __restrict__ err)
+                                                         int* __restrict__ out_cursor, int per, int streams,
+                                                         int* __restrict__ err)
 {
     pdl_wait();
     pdl_trigger();
+    __shared__ int s_box[kScatterWarps];
+    __shared__ int2 s_acc[kScatterWarps];
     const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int acc_box = -1;                           // per-warp box counts not yet added
-    unsigned long long acc_ng = 0, acc_nk = 0;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < g.total_n; base += stride) {
-        int64_t s = base + threadIdx.x;
-        bool valid = s < g.total_n;
+    int acc_ng = 0, acc_nk = 0;
+    // this CTA's slots
+    constexpr int stride = kScatterThreads;
+    const int64_t chunk = (int64_t)(blockIdx.x % streams) * (gridDim.x / streams) + blockIdx.x / streams;
+    int64_t s = chunk * per * stride + threadIdx.x;
+    const int64_t end = min(g.total_n, (chunk + 1) * per * stride);
+    int root_next = 0, mo_next = 0, cnt_next = 0;
+    if (s < end) {
+        root_next = parent[s];
+        mo_next = minorig[s];
+        cnt_next = cnt[s];
+    }
+    for (; s - threadIdx.x < end; s += stride) {
+        const bool valid = s < end;
+        const int root = root_next, own = mo_next, own_cnt = cnt_next;
+        if (s + stride < end) {                 // the next slot's words
+            root_next = parent[s + stride];
+            mo_next = minorig[s + stride];
+            cnt_next = cnt[s + stride];
+        }
         unsigned active = __ballot_sync(kFull, valid);
         if (!valid)
             continue;
-        int bi = box_of(g.box_p0, g.nbox, s);
-        int64_t p0 = g.boxes[bi].p0;
+        const bool is_root = root == (int)s;
         // the input index o of slot s: minorig keeps it for every non-root
         // (the label pass only lowers roots' entries) and for singleton
-        // roots; only a root of a larger group reads it from the binned record
-        const int root = parent[s];
-        const bool is_root = root == (int)s;
-        int o, label, size;
+        // roots; only a root of a larger group reads it from the binned record.
+        // The loads do not wait for one another.
+        int label = own, size = own_cnt, o = own;
         if (!is_root) {
-            o = minorig[s];
             label = minorig[root];
-            size = o == label ? cnt[root] : 0;
-        } else {
-            size = cnt[s];
-            label = minorig[s];
-            o = size == 1 ? label : __float_as_int(sorted[s].w);
+            size = cnt[root];
+        } else if (own_cnt != 1) {
+            o = __float_as_int(sorted[s].w);
         }
+        int bi = box_of(g.box_p0, g.nbox, s);
+        int64_t p0 = g.boxes[bi].p0;
         // a record that binning never wrote is reported, and stays inside the box
         const bool ok = (unsigned long long)o < (unsigned long long)g.boxes[bi].n;
         const int64_t gidx = p0 + (ok ? o : 0);
@@ -242,8 +292,8 @@ __global__ void __launch_bounds__(256) k_outputs_scatter(Geometry g, const float
         if (__all_sync(active, bi == bi0)) {
             if (bi0 != acc_box) {
                 if (lane == 0 && acc_box >= 0) {
-                    if (acc_ng) atomicAdd(n_groups + acc_box, acc_ng);
-                    if (acc_nk) atomicAdd(n_cat + acc_box, acc_nk);
+                    if (acc_ng) atomicAdd(n_groups + acc_box, (unsigned long long)acc_ng);
+                    if (acc_nk) atomicAdd(n_cat + acc_box, (unsigned long long)acc_nk);
                 }
                 acc_box = bi0;
                 acc_ng = acc_nk = 0;
@@ -262,9 +312,27 @@ __global__ void __launch_bounds__(256) k_outputs_scatter(Geometry g, const float
         }
     }
     // lane 0 took part in every iteration (its slot is the warp's smallest)
-    if (lane == 0 && acc_box >= 0) {
-        if (acc_ng) atomicAdd(n_groups + acc_box, acc_ng);
-        if (acc_nk) atomicAdd(n_cat + acc_box, acc_nk);
+    if (lane == 0) {
+        s_box[threadIdx.x >> 5] = acc_box;
+        s_acc[threadIdx.x >> 5] = make_int2(acc_ng, acc_nk);
+    }
+    __syncthreads();
+    // the CTA's warps mostly end in one box: one addition for each run of them
+    if (threadIdx.x == 0) {
+        int box = -1, ng = 0, nk = 0;
+        for (int w = 0; w <= kScatterWarps; ++w) {
+            const int wb = w < kScatterWarps ? s_box[w] : -1;
+            if (wb != box) {
+                if (ng) atomicAdd(n_groups + box, (unsigned long long)ng);
+                if (nk) atomicAdd(n_cat + box, (unsigned long long)nk);
+                box = wb;
+                ng = nk = 0;
+            }
+            if (w < kScatterWarps) {
+                ng += s_acc[w].x;
+                nk += s_acc[w].y;
+            }
+        }
     }
 }
 
@@ -388,8 +456,8 @@ __global__ void __launch_bounds__(kOutThreads) k_outputs_write(Geometry g, const
 // Catalogue above kDirectMax inputs: one CTA per output tile that holds
 // entries writes them in ascending label order from tile_off[tile] on.
 __global__ void __launch_bounds__(kOutThreads) k_catalogue(Geometry g, const int32_t* sizes, const int* tile_off,
-                                                           int32_t thr, int2* __restrict__ cat, int64_t cap, int64_t n_tiles,
-                                                           Status* status)
+                                                           int32_t thr, int2* __restrict__ cat, int64_t cap,
+                                                           int64_t n_tiles, Status* status)
 {
     pdl_wait();
     pdl_trigger();
@@ -453,8 +521,8 @@ cudaError_t launch_finalize(const Geometry& g, const Work& w, const UfArgs& uf, 
     if (size_count == 1)
         return launch_kernel(dependent, k_finalize_hash, grid_for(g.total_n, 256 * kHashBatch, 4), 256, 0, s, g.total_n,
                              w.parent, w.minorig, w.cnt, &w.status->err, ordered);
-    return launch_kernel(dependent, k_finalize, grid_for(g.total_n, 256, 8), 256, 0, s, g.total_n, w.parent, w.minorig,
-                         w.cnt, &w.status->err, ordered);
+    return launch_kernel(dependent, k_finalize, grid_for(g.total_n, 256, 16), 256, 0, s, g.total_n, w.parent,
+                         w.minorig, w.cnt, &w.status->err, ordered);
 }
 
 cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t min_size, cudaStream_t s)
@@ -463,9 +531,15 @@ cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t min_size, c
         return cudaSuccess;
     int32_t thr = min_size < 1 ? 1 : min_size;
     int2* pairs = (int2*)w.tmp;            // the brick-order copy is dead by now
+    const int64_t tiles = (g.total_n + kScatterThreads - 1) / kScatterThreads;
+    // as many slots per CTA as leave eight CTAs to an SM
+    const int per = (int)std::min<int64_t>(kScatterTiles, std::max<int64_t>(1, tiles / ((int64_t)sm_count() * 8)));
+    const int streams = g.total_n <= kDirectMax ? 1 : kScatterStreams;
+    const int64_t chunks = (tiles + per - 1) / per;
     return launch_next(g.total_n, g.total_n <= kDirectMax ? k_outputs_scatter<true> : k_outputs_scatter<false>,
-                       grid_for(g.total_n, 256, 8), 256, 0, s, g, w.sorted, w.parent, w.minorig, w.cnt, thr,
-                       w.n_groups, w.n_cat, pairs, w.out_cursor, &w.status->err);
+                       (chunks + streams - 1) / streams * streams, kScatterThreads, 0, s, g, w.sorted, w.parent,
+                       w.minorig, w.cnt, thr, w.n_groups, w.n_cat, pairs, w.out_cursor, per, streams,
+                       &w.status->err);
 }
 
 cudaError_t launch_catalogue(const Geometry& g, const Work& w, int32_t* ids, int32_t* sizes, int32_t min_size,
@@ -476,9 +550,9 @@ cudaError_t launch_catalogue(const Geometry& g, const Work& w, int32_t* ids, int
     int32_t thr = min_size < 1 ? 1 : min_size;
     const int2* pairs = (const int2*)w.tmp;
     const bool direct = g.total_n <= kDirectMax;
-    cudaError_t e = launch_next(g.total_n, direct ? k_outputs_write<true> : k_outputs_write<false>, w.n_tiles, kOutThreads, 0, s,
-                                g, pairs, ids, sizes, thr, cat, cap, w.tile_state, w.tile_ticket, w.out_cursor,
-                                w.status);
+    cudaError_t e =
+        launch_next(g.total_n, direct ? k_outputs_write<true> : k_outputs_write<false>, w.n_tiles, kOutThreads, 0, s,
+                    g, pairs, ids, sizes, thr, cat, cap, w.tile_state, w.tile_ticket, w.out_cursor, w.status);
     if (e != cudaSuccess || direct)
         return e;
     e = launch_scan(g.total_n, w.out_cursor, 1, w.tile_off, w.n_tiles, w.tile_state, w.tile_ticket, 0, nullptr, nullptr,

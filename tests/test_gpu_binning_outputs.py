@@ -49,6 +49,20 @@ def test_tile_edges(cuda_lib, n):
             _check(_run(fof, plan.h, dpos, n, min_size), want, min_size)
 
 
+# chunks of one to four tiles of 256 slots per CTA of the output scatter, with
+# ragged last chunks: 152 SMs x 8 CTAs x 256 slots are 311,296
+@pytest.mark.parametrize("n", [311_295, 622_593, 934_145, 1_245_183, 1_556_737])
+def test_output_chunk_edges(cuda_lib, n):
+    import torch
+    fof = cuda_lib
+    box = 40.0
+    pos = synth.uniform_box(n, box, seed=900 + n)
+    l_x = synth.linking_length(n, box)
+    want = oracle.groups(pos, box, l_x)
+    with fof.FoF(box, l_x, n) as plan:
+        _check(_run(fof, plan.h, torch.from_numpy(pos).cuda(), n, 2), want, 2)
+
+
 # bricks of one cell: counters a line apart and counted per tile in shared
 # memory (up to 12,288), a sector apart (up to 131,072), side by side
 @pytest.mark.parametrize("nc", [23, 24, 50, 51])
