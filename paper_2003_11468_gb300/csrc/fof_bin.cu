@@ -89,12 +89,13 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(const float* __restri
     int bad = 0;
     int brick[kBinItems], off[kBinItems];
     unsigned peers[kBinItems];
+    BoxCursor box;
 #pragma unroll
     for (int k = 0; k < kBinItems; ++k) {
         const int64_t i = base + k * kBinThreads;
+        const BoxDev& b = g.boxes[box.at(g.box_p0, g.nbox, i - lane, i, lane)];
         brick[k] = -1;
         if (i < g.total_n) {
-            const BoxDev& b = g.boxes[box_of(g.box_p0, g.nbox, i)];
             float4 rec;
             bool ok;
             brick[k] = (int)brick_of(pos, i, b, rec, ok);   // fits in 31 bits (checked when the plan is made)
@@ -138,12 +139,13 @@ __global__ void __launch_bounds__(kCountThreads) k_bin_count_tile(const float* _
     const int64_t base = (int64_t)blockIdx.x * (kItems * kCountThreads) + threadIdx.x;
     int brick[kItems], local[kItems];
     int bad = 0;
+    BoxCursor box;
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
         const int64_t i = base + k * kCountThreads;
+        const BoxDev& b = g.boxes[box.at(g.box_p0, g.nbox, i - lane, i, lane)];
         brick[k] = -1;
         if (i < g.total_n) {
-            const BoxDev& b = g.boxes[box_of(g.box_p0, g.nbox, i)];
             float4 rec;
             bool ok;
             brick[k] = (int)brick_of(pos, i, b, rec, ok);
@@ -186,12 +188,14 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_scatter(const float* __rest
     float4 rec[kBinItems];
     int64_t brick[kBinItems];
     int r[kBinItems];
+    const int lane = threadIdx.x & 31;
+    BoxCursor box;
 #pragma unroll
     for (int k = 0; k < kBinItems; ++k) {
         const int64_t i = base + k * kBinThreads;
+        const BoxDev& b = g.boxes[box.at(g.box_p0, g.nbox, i - lane, i, lane)];
         brick[k] = -1;
         if (i < g.total_n) {
-            const BoxDev& b = g.boxes[box_of(g.box_p0, g.nbox, i)];
             bool ok;
             r[k] = rank[i];
             brick[k] = brick_of(pos, i, b, rec[k], ok);
@@ -709,7 +713,7 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kHeavyThreads
             drawn = atomicAdd(ticket, 1);
         const int64_t gb = heavy[it];
         const int s0 = bstart[gb], s1 = bstart[gb + 1];
-        const BoxDev& b = g.boxes[box_of(g.box_brick0, g.nbox, gb)];
+        const BoxDev& b = g.boxes[box_of_warp(g.box_brick0, g.nbox, gb, threadIdx.x & 31)];
         const CodeGeo geo = code_geo(b);
         const int r3 = b.r * b.r * b.r;
         for (int c = threadIdx.x; c < r3; c += kHeavyThreads) hist[c] = 0;

@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(kThreads, kBlocks) k_dense_self(Geometry g, Wo
         const int m = c1 - c0;
         if (m <= kLo || m > kM)
             continue;                             // the other size class's cell (block-uniform)
-        const BoxDev& b = g.boxes[box_of(g.box_p0, g.nbox, c0)];
+        const BoxDev& b = g.boxes[box_of_warp(g.box_p0, g.nbox, c0, threadIdx.x & 31)];
         const int q = b.q, q3 = q * q * q;
         const float4 p0 = w.sorted[c0];
         const int cx = cell_coord(p0.x, b), cy = cell_coord(p0.y, b), cz = cell_coord(p0.z, b);
@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(kThreads, kBlocks) k_dense_pairs(Geometry g, W
         const int m = c1 - c0;
         if (m <= kLo || m > kM)
             continue;                             // the other size class's cell (block-uniform)
-        const BoxDev& b = g.boxes[box_of(g.box_p0, g.nbox, c0)];
+        const BoxDev& b = g.boxes[box_of_warp(g.box_p0, g.nbox, c0, threadIdx.x & 31)];
         const int q = b.q, q3 = q * q * q;
         const float4 p0 = w.sorted[c0];
         const int cx = cell_coord(p0.x, b), cy = cell_coord(p0.y, b), cz = cell_coord(p0.z, b);

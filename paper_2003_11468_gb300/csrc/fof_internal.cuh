@@ -241,6 +241,42 @@ __device__ __forceinline__ int box_of(const int64_t* __restrict__ starts, int nb
     return lo;
 }
 
+// The same by a whole warp (i is the same in all lanes): 32 starts are compared
+// at a time, where the search above is a chain of loads (9 for 512 boxes, 2
+// here; batch of 512 boxes, binning, self links and outputs together 24.4 and
+// 22.6 ms).
+__device__ __forceinline__ int box_of_warp(const int64_t* __restrict__ starts, int nbox, int64_t i, int lane)
+{
+    int lo = 0;
+    for (int n = nbox; n > 1;) {
+        const int step = (n + 31) >> 5;
+        const bool below = lane * step < n && __ldg(starts + lo + lane * step) <= i;
+        const int k = max(__popc(__ballot_sync(kFull, below)) - 1, 0);
+        lo += k * step;
+        n = min(step, n - k * step);
+    }
+    return lo;
+}
+
+// The box of a warp's particles in ascending order: looked up once and kept
+// until the particles pass its end.
+struct BoxCursor {
+    int bi = 0;
+    int64_t end = 0;
+
+    // the box of particle i; `first` is the warp's lowest, all lanes take part
+    __device__ __forceinline__ int at(const int64_t* starts, int nbox, int64_t first, int64_t i, int lane)
+    {
+        if (nbox == 1)
+            return 0;
+        if (first >= end) {
+            bi = box_of_warp(starts, nbox, first, lane);
+            end = bi + 1 < nbox ? __ldg(starts + bi + 1) : INT64_MAX;
+        }
+        return i < end ? bi : box_of(starts, nbox, i);
+    }
+};
+
 // ------------------------------------------------------------------------
 // cells
 // ------------------------------------------------------------------------

@@ -328,6 +328,8 @@ __global__ void __launch_bounds__(kLinkThreads, kSplit ? 4 : kLinkBlocks)
         __syncwarp();                           // every lane's copy is in, and the last window's reads are done
         const float4* rec = pf + par * kWarp;
         if (valid) {
+            // (the warp's search of box_of_warp spills here: batch of 512 boxes
+            // 24.5 and 24.4 ms, but the 768^3 box 33.9 and 34.2)
             const int bi = box_of(g.box_p0, g.nbox, s);
             const BoxDev& b = g.boxes[bi];
             const float4 p = rec[lane];
@@ -996,7 +998,8 @@ __global__ void __launch_bounds__(kTeamWarps * 32, kTeamBlocks)
     for (int it = blockIdx.x, n = *n_hi; it < n; it += gridDim.x) {
         const int64_t e = list[cap - 1 - it];
         const int c0 = (int)(uint32_t)e;
-        team_cell_cta(smem.cta, c0, (int)(e >> 32), sorted, parent, minorig, g.boxes[box_of(g.box_p0, g.nbox, c0)]);
+        team_cell_cta(smem.cta, c0, (int)(e >> 32), sorted, parent, minorig,
+                      g.boxes[box_of_warp(g.box_p0, g.nbox, c0, lane)]);
     }
     // the others, one per warp, the last CTAs first (they have the fewest
     // large cells).  Software pipeline: the next cell's positions are copied
@@ -1011,7 +1014,7 @@ __global__ void __launch_bounds__(kTeamWarps * 32, kTeamBlocks)
     for (; it < n; it += stride) {
         const int c0 = (int)(uint32_t)e, m = (int)(e >> 32);
         const int nw = (m + 31) >> 5;
-        const BoxDev& b = g.boxes[box_of(g.box_p0, g.nbox, c0)];
+        const BoxDev& b = g.boxes[box_of_warp(g.box_p0, g.nbox, c0, lane)];
         cp_async_wait_all();                   // each lane reads back only its own copies
         // the cell in z order (bins of 1/32 of the cell), also in global
         // memory: the streams of the neighbours below then read only a

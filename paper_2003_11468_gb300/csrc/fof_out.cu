@@ -228,6 +228,7 @@ __global__ void __launch_bounds__(kScatterThreads) k_outputs_scatter(Geometry g,
     const int64_t chunk = (int64_t)(blockIdx.x % streams) * (gridDim.x / streams) + blockIdx.x / streams;
     int64_t s = chunk * per * stride + threadIdx.x;
     const int64_t end = min(g.total_n, (chunk + 1) * per * stride);
+    BoxCursor box;
     int root_next = 0, mo_next = 0, cnt_next = 0;
     if (s < end) {
         root_next = parent[s];
@@ -243,6 +244,7 @@ __global__ void __launch_bounds__(kScatterThreads) k_outputs_scatter(Geometry g,
             cnt_next = cnt[s + stride];
         }
         unsigned active = __ballot_sync(kFull, valid);
+        const int bi = box.at(g.box_p0, g.nbox, s - lane, s, lane);
         if (!valid)
             continue;
         const bool is_root = root == (int)s;
@@ -257,8 +259,7 @@ __global__ void __launch_bounds__(kScatterThreads) k_outputs_scatter(Geometry g,
         } else if (own_cnt != 1) {
             o = __float_as_int(sorted[s].w);
         }
-        int bi = box_of(g.box_p0, g.nbox, s);
-        int64_t p0 = g.boxes[bi].p0;
+        const int64_t p0 = g.boxes[bi].p0;
         // a record that binning never wrote is reported, and stays inside the box
         const bool ok = (unsigned long long)o < (unsigned long long)g.boxes[bi].n;
         const int64_t gidx = p0 + (ok ? o : 0);
@@ -394,6 +395,9 @@ __global__ void __launch_bounds__(kOutThreads) k_outputs_write(Geometry g, const
         e[k] = i < g.total_n ? pairs[i] : make_int2(0, 0);
     }
     if constexpr (!kDirect) {
+        // the box of the tile's first input, and where it ends
+        const int bi = box_of_warp(g.box_p0, g.nbox, base, lane);
+        const int64_t p0 = g.boxes[bi].p0, p1 = p0 + g.boxes[bi].n;
 #pragma unroll
         for (int k = 0; k < kOutItems; ++k) {
             const int64_t i = base + k * kOutThreads + threadIdx.x;
@@ -401,7 +405,7 @@ __global__ void __launch_bounds__(kOutThreads) k_outputs_write(Geometry g, const
                 const int off = e[k].x & (kOutTile - 1);
                 if (e[k].x < 0) {                        // the input is its group's label
                     const int64_t gidx = base + off;
-                    e[k].x = (int)(gidx - g.boxes[box_of(g.box_p0, g.nbox, gidx)].p0);
+                    e[k].x = (int)(gidx - (gidx < p1 ? p0 : g.boxes[box_of(g.box_p0, g.nbox, gidx)].p0));
                 } else {
                     e[k] = make_int2(e[k].y, 0);
                 }
