@@ -960,7 +960,11 @@ cudaError_t launch_brick_sort(const Geometry& g, const Work& w, int dense_min, c
                              w.team_cap};
     if (heavy_bricks(g.total_n)) {
         int64_t clusters = g.total_n / kHeavyBrick;
-        const int64_t most = (int64_t)sm_count() * kHeavyBlocks / kCluster;
+        // twice the resident clusters: the others take over while the last bricks
+        // of the first end, and k_brick_sort has the rest (both kernels, with 1
+        // and 2 times, 8 million particles: 219 and 209 us, 16.8 million 421 and
+        // 404; with half as many 234 and 474)
+        const int64_t most = (int64_t)sm_count() * 2 * kHeavyBlocks / kCluster;
         if (clusters > most) clusters = most;
         cudaError_t e = launch_next(g.total_n, k_brick_sort_heavy, clusters * kCluster, kHeavyThreads, 0, s, g, w.tmp,
                                     w.bstart, w.heavy_list, w.n_heavy, w.heavy_ticket, w.sorted, w.parent, w.minorig,
