@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocks)
 #pragma unroll
             for (int i = 0; i < kSortKeep; ++i) {
                 const int k = i * kSortThreads + tid;
-                if (s0 + k < s1)
+                if (slot_before(s0, k, s1))
                     cp_async16(&S.rec[buf][k], tmp + s0 + k);
             }
         }
@@ -719,17 +719,17 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kHeavyThreads
         for (int c = threadIdx.x; c < r3; c += kHeavyThreads) hist[c] = 0;
         __syncthreads();
         // this CTA's particles
-        const int share = (s1 - s0 + kCluster - 1) / kCluster;
-        const int k0 = s0 + rank * share, k1 = min(k0 + share, s1);
-        for (int kb = k0 + threadIdx.x; kb < k1; kb += kHeavyFlight * kHeavyThreads) {
+        const SlotRange own_slots = slot_share(s0, s1 - s0, rank, kCluster);
+        const int k0 = own_slots.first, kn = own_slots.count;
+        for (int kb = threadIdx.x; kb < kn; kb += kHeavyFlight * kHeavyThreads) {
             float4 v[kHeavyFlight];
 #pragma unroll
             for (int i = 0; i < kHeavyFlight; ++i)
-                if (kb + i * kHeavyThreads < k1)
-                    v[i] = tmp[kb + i * kHeavyThreads];
+                if (kb + i * kHeavyThreads < kn)
+                    v[i] = tmp[k0 + kb + i * kHeavyThreads];
 #pragma unroll
             for (int i = 0; i < kHeavyFlight; ++i)
-                if (kb + i * kHeavyThreads < k1)
+                if (kb + i * kHeavyThreads < kn)
                     atomicAdd(hist + code_of(v[i], geo), 1);
         }
         cluster.sync();
@@ -779,16 +779,16 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kHeavyThreads
                 reserved = atomicAdd(list_counter(lists, threadIdx.x), cells);
         }
         cluster.sync();
-        for (int kb = k0 + threadIdx.x; kb < k1; kb += kHeavyFlight * kHeavyThreads) {
+        for (int kb = threadIdx.x; kb < kn; kb += kHeavyFlight * kHeavyThreads) {
             float4 v[kHeavyFlight];
 #pragma unroll
             for (int i = 0; i < kHeavyFlight; ++i)
-                if (kb + i * kHeavyThreads < k1)
-                    v[i] = tmp[kb + i * kHeavyThreads];
+                if (kb + i * kHeavyThreads < kn)
+                    v[i] = tmp[k0 + kb + i * kHeavyThreads];
 #pragma unroll
             for (int i = 0; i < kHeavyFlight; ++i) {
-                const int k = kb + i * kHeavyThreads;
-                if (k < k1) {
+                if (kb + i * kHeavyThreads < kn) {
+                    const int k = k0 + kb + i * kHeavyThreads;
                     const int slot = atomicAdd(hist + code_of(v[i], geo), 1);
                     if (slot < s1) {
                         sorted[slot] = v[i];

@@ -104,6 +104,33 @@ struct Status {
 };
 
 // ------------------------------------------------------------------------
+// ranges of slots
+// ------------------------------------------------------------------------
+//
+// Slots are int32 and a plan may hold 2^31 - 2 of them, so a loop that steps
+// past the end of a range counts from the range's start: the slot itself has no
+// room to step past.
+
+struct SlotRange {
+    int first, count;
+};
+
+// Share `rank` of `of` of the slots [first, first + count).
+__host__ __device__ __forceinline__ SlotRange slot_share(int first, int count, int rank, int of)
+{
+    const int share = count / of + (count % of != 0);
+    const int64_t at = (int64_t)rank * share;
+    const int off = at < count ? (int)at : count;
+    return SlotRange{first + off, count - off < share ? count - off : share};
+}
+
+// Slot `first + k` lies before `end`.
+__host__ __device__ __forceinline__ bool slot_before(int first, int k, int end)
+{
+    return k < end - first;
+}
+
+// ------------------------------------------------------------------------
 // dependent launches
 // ------------------------------------------------------------------------
 //
