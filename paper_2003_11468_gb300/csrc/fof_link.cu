@@ -596,9 +596,11 @@ union TeamSmem {
 };
 
 // Positions that link to nothing: rows and columns beyond the cell's
-// particles.  Any difference with a real position or the other sentinel
-// squares to +inf in float32, so the pre-test rejects it.
-constexpr float kFar = 1e30f;
+// particles.  Any difference with a real position (at most 1e30, the largest
+// box) or the other sentinel squares to +inf in float32, which the pre-test
+// rejects; where its bound is +inf too (linking lengths above 1.8e19), the exact
+// test does: one period of the box brings no sentinel back into it.
+constexpr float kFar = 3e38f;
 
 __device__ __forceinline__ float4 far_point(float v)
 {
