@@ -421,14 +421,16 @@ __device__ __forceinline__ int half_of(const unsigned* hist, int c)
 }
 
 __global__ void __launch_bounds__(kSortThreads, kSortBlocks)
-    k_brick_sort(Geometry g, const float4* __restrict__ tmp, const int* bstart,
+    k_brick_sort(Geometry g, const float4* tmp, const int* bstart,
                  float4* __restrict__ sorted, int* __restrict__ parent, int* __restrict__ minorig,
                  int* __restrict__ cnt, int* __restrict__ cell_start, int dense_min, CellLists lists,
-                 int heavy_from, bool beside_heavy, int* __restrict__ err)
+                 int heavy_from, const unsigned* beside, int* __restrict__ err)
 {
     // beside k_brick_sort_heavy where that runs just before (it needs nothing
     // of it), else after the scatter
-    if (!beside_heavy)
+    if (beside)
+        pdl_join(beside);
+    else
         pdl_wait();
     pdl_trigger();
     extern __shared__ float4 sort_raw[];
@@ -668,7 +670,7 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocks)
         }
     }
     cp_async_wait_all();
-    if (beside_heavy)
+    if (beside)
         pdl_wait();
 }
 
@@ -690,10 +692,11 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kHeavyThreads
     k_brick_sort_heavy(Geometry g, const float4* __restrict__ tmp, const int* bstart, const int* heavy,
                        const int* n_heavy, int* __restrict__ ticket, float4* __restrict__ sorted,
                        int* __restrict__ parent, int* __restrict__ minorig, int* __restrict__ cnt,
-                       int* __restrict__ cell_start, int dense_min, CellLists lists, int* __restrict__ err)
+                       int* __restrict__ cell_start, int dense_min, CellLists lists, unsigned* pass_on,
+                       int* __restrict__ err)
 {
     pdl_wait();
-    pdl_trigger();
+    pdl_pass_on(pass_on);
     namespace cg = cooperative_groups;
     __shared__ int hist[kMaxR3];
     __shared__ int part[kWarp];
@@ -968,7 +971,8 @@ cudaError_t launch_brick_sort(const Geometry& g, const Work& w, int dense_min, c
         if (clusters > most) clusters = most;
         cudaError_t e = launch_next(g.total_n, k_brick_sort_heavy, clusters * kCluster, kHeavyThreads, 0, s, g, w.tmp,
                                     w.bstart, w.heavy_list, w.n_heavy, w.heavy_ticket, w.sorted, w.parent, w.minorig,
-                                    w.cnt, w.cell_start, dense_min, lists, &w.status->err);
+                                    w.cnt, w.cell_start, dense_min, lists, w.status->passed_on + kPassBrickOrder,
+                                    &w.status->err);
         if (e != cudaSuccess) return e;
     }
     // the shared-memory opt-in is per device; setting it again is harmless
@@ -987,7 +991,8 @@ cudaError_t launch_brick_sort(const Geometry& g, const Work& w, int dense_min, c
     const bool beside = heavy_bricks(g.total_n);
     return launch_kernel(g.total_n <= (beside ? kBesideMax : kDependentMax), k_brick_sort, blocks, kSortThreads,
                          sizeof(SortSmem), s, g, w.tmp, w.bstart, w.sorted, w.parent, w.minorig, w.cnt, w.cell_start,
-                         dense_min, lists, heavy_from(g.total_n), beside, &w.status->err);
+                         dense_min, lists, heavy_from(g.total_n),
+                         beside ? w.status->passed_on + kPassBrickOrder : (unsigned*)nullptr, &w.status->err);
 }
 
 // Bricks above this many particles go to k_brick_sort_heavy: the limit of the

@@ -439,9 +439,12 @@ template <bool kVar, int kLo, int kM, int kThreads, int kBlocks>
 __global__ void __launch_bounds__(kThreads, kBlocks) k_dense_self(Geometry g, Work w, int dense_min,
                                                               UfArgs uf)
 {
-    // beside k_link, which never touches a dense cell's particles (it reads
-    // their records, but only to see which cell they are in), and beside the
-    // other size class: their unions are the same atomic ones
+    // beside k_link, which links no particle of a dense cell, and beside the
+    // other size class: their unions are the same atomic ones.  k_link reads the
+    // records that are put in sub-cell order here, but only to see which cell they
+    // are in: every record written there is of the same cell, and so is any mix
+    // of two, since a cell is a product of intervals.
+    pdl_join(w.status->passed_on + kPassCellOrder);
     pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const DenseSmem S = carve<kM>(smem_raw);
@@ -574,9 +577,13 @@ __global__ void __launch_bounds__(kThreads, kBlocks) k_dense_pairs(Geometry g, W
                                                                UfArgs uf)
 {
     // after dense_self; the second size class beside the first
-    if (kLo == 0)
+    if (kLo == 0) {
         pdl_wait();
-    pdl_trigger();
+        pdl_pass_on(w.status->passed_on + kPassDenseOrder);
+    } else {
+        pdl_join(w.status->passed_on + kPassDenseOrder);
+        pdl_trigger();
+    }
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const DenseSmem S = carve<kM>(smem_raw);
     int* err = uf.err;

@@ -101,6 +101,7 @@ struct Status {
     int pad;
     long long n_cat_total;
     unsigned link_ticket;
+    unsigned passed_on[3];    // pdl_pass_on
 };
 
 // ------------------------------------------------------------------------
@@ -141,12 +142,18 @@ __host__ __device__ __forceinline__ bool slot_before(int first, int k, int end)
 // kernel writes before pdl_wait, which returns when the kernel before it has
 // completed (and, since that one waited too, all earlier ones).
 //
-// A kernel that does not need the one just before it calls pdl_wait as its
-// last step instead, so that it runs beside it and still completes after it.
-// It starts when every CTA before it has triggered, and those trigger only
-// after their own wait at the top, so everything up to the kernel before the
-// one before it has completed by then.  (After a plain launch both calls return
-// at once, and the order in the stream does the rest.)
+// A kernel that does not need the one just before it starts beside it: it calls
+// pdl_wait as its last step, so that it still completes after it.  What the
+// kernels before both wrote has completed by then, but only pdl_wait makes it
+// visible to a grid, and this grid has not waited.  So the kernel before it
+// passes on what its own wait showed it: after that wait it stores a word with
+// release order and then triggers (pdl_pass_on), and the kernel beside it loads
+// the word with acquire order before it reads anything (pdl_join).  Release and
+// acquire are cumulative at gpu scope: every write that the storing thread could
+// see comes before every read after the load.  A CTA that does not find the word
+// waits at the top instead; the word starts each run at zero.  (After a plain
+// launch the word is there, both waits return at once, and the order in the
+// stream does the rest.)
 //
 // Values that an earlier kernel writes are not read through `const
 // __restrict__` parameters or __ldg before a value that was read after the
@@ -172,6 +179,29 @@ __device__ __forceinline__ void pdl_wait()
 __device__ __forceinline__ void pdl_trigger()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// The words of Status::passed_on.
+enum { kPassBrickOrder, kPassCellOrder, kPassDenseOrder, kPassWords };
+
+// By every thread of a kernel that another one may run beside, after pdl_wait.
+__device__ __forceinline__ void pdl_pass_on(unsigned* word)
+{
+    if (threadIdx.x == 0) {                    // the trigger after the store
+        if (blockIdx.x == 0)
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(word), "r"(1u) : "memory");
+        pdl_trigger();
+    }
+}
+
+// By every thread of the kernel beside it, before it reads what earlier kernels wrote.
+__device__ __forceinline__ void pdl_join(const unsigned* word)
+{
+    unsigned there = 0u;
+    if (threadIdx.x == 0)
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(there) : "l"(word) : "memory");
+    if (!__syncthreads_or((int)there))
+        pdl_wait();
 }
 
 // dependent: as a programmatic dependent, else a plain launch
@@ -748,7 +778,6 @@ struct Work {
     int* tile_off;      // [n_tiles + 1] first catalogue entry of each tile (above kDirectMax inputs)
     int64_t n_tiles;
     Status* status;     // device status
-    unsigned* link_ticket; // batches of windows handed out by k_link
     unsigned long long* n_groups;  // [nbox]
     unsigned long long* n_cat;     // [nbox]
     int64_t* dense_list; // [dense_cap] cell keys of the subdivided cells

@@ -278,10 +278,10 @@ __device__ __forceinline__ void team_cell(TeamStage& S, int* __restrict__ parent
 template <bool kVar, bool kSplit>
 __global__ void __launch_bounds__(kLinkThreads, kSplit ? 4 : kLinkBlocks)
     k_link(Geometry g, const float4* __restrict__ sorted, const int* __restrict__ cell_start, int* parent,
-           int dense_min, int parts, int batch, unsigned* ticket, UfArgs uf)
+           int dense_min, int parts, int batch, Status* status, UfArgs uf)
 {
     pdl_wait();
-    pdl_trigger();
+    pdl_pass_on(status->passed_on + kPassCellOrder);
     __shared__ TeamStage stage[kLinkWarps];
     __shared__ uint32_t spread_tab[16];
     if (threadIdx.x < 16)
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(kLinkThreads, kSplit ? 4 : kLinkBlocks)
         cp_async16(pf + lane, sorted + base + lane);
     cp_async_commit();
     if (!kSplit && lane == 0)
-        drawn = atomicAdd(ticket, 1u);
+        drawn = atomicAdd(&status->link_ticket, 1u);
 
     for (int par = 0; base < total; par ^= 1) {
         const unsigned s = base + lane;
@@ -528,7 +528,7 @@ __global__ void __launch_bounds__(kLinkThreads, kSplit ? 4 : kLinkBlocks)
         }
         base = next;
         if (!kSplit && last && lane == 0)
-            drawn = atomicAdd(ticket, 1u);
+            drawn = atomicAdd(&status->link_ticket, 1u);
     }
 }
 
@@ -1135,7 +1135,7 @@ cudaError_t launch_link(const Geometry& g, const Work& w, int dense_min, const U
     auto kernel = uf.var ? (split ? k_link<true, true> : k_link<true, false>)
                          : (split ? k_link<false, true> : k_link<false, false>);
     return launch_next(g.total_n, kernel, blocks, kLinkThreads, 0, s, g, w.sorted, w.cell_start, w.parent, dense_min,
-                       parts, batch, w.link_ticket, uf);
+                       parts, batch, w.status, uf);
 }
 
 }  // namespace fofgpu

@@ -78,6 +78,7 @@ struct ResultsLayout {
 };
 
 static_assert(sizeof(Status) <= 64, "the per-box counts follow at 64");
+static_assert(kPassWords == sizeof(Status::passed_on) / sizeof(unsigned), "one word per pair of kernels");
 
 ResultsLayout results_layout(int nbox)
 {
@@ -469,7 +470,6 @@ void bind_workspace(char* ws, const Layout& L, const BoxDev* boxes, int nbox, in
     const ResultsLayout rl = results_layout(nbox);
     char* res = ws + L.results;
     w.status = (Status*)(res + rl.status_off);
-    w.link_ticket = &w.status->link_ticket;
     w.n_groups = (unsigned long long*)(res + rl.groups_off);
     w.n_cat = (unsigned long long*)(res + rl.cat_off);
     w.bcount = (int*)(ws + L.bcount);
