@@ -100,6 +100,7 @@ struct Status {
     int err;
     int pad;
     long long n_cat_total;
+    int flat;                 // the forest is flattened: parent, minorig and cnt are final
     unsigned link_ticket;
     unsigned passed_on[3];    // pdl_pass_on
 };
@@ -778,6 +779,8 @@ struct Work {
     int* tile_off;      // [n_tiles + 1] first catalogue entry of each tile (above kDirectMax inputs)
     int64_t n_tiles;
     Status* status;     // device status
+    int* group_words;   // what fof_groups counts in, cleared when it starts: n_groups, n_cat,
+    int64_t n_group_words; // tile_state, out_cursor and tile_ticket
     unsigned long long* n_groups;  // [nbox]
     unsigned long long* n_cat;     // [nbox]
     int64_t* dense_list; // [dense_cap] cell keys of the subdivided cells
@@ -834,9 +837,7 @@ cudaError_t launch_team_self(const Geometry& g, const Work& w, cudaStream_t s);
 cudaError_t launch_big(const Geometry& g, const Work& w, int dense_min, const UfArgs& uf, bool pairs,
                        cudaStream_t s);
 // size_count: 0 warp-aggregated atomics, 1 per-block shared-memory hash table
-// dependent: nothing but this library's kernels lies between in the stream
-cudaError_t launch_finalize(const Geometry& g, const Work& w, const UfArgs& uf, int size_count, bool dependent,
-                            cudaStream_t s);
+cudaError_t launch_finalize(const Geometry& g, const Work& w, const UfArgs& uf, int size_count, cudaStream_t s);
 cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t min_size, cudaStream_t s);
 cudaError_t launch_catalogue(const Geometry& g, const Work& w, int32_t* ids, int32_t* sizes,
                              int32_t min_size, int2* cat, int64_t cap, cudaStream_t s);

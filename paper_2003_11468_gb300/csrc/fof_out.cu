@@ -6,7 +6,9 @@
 //              size 1 and their own index, so they take part in no atomic:
 //              the paper's early elimination of singletons (Sec. 3.4.2),
 //              with the atomic additions of its parallel size count
-//              (Sec. 3.4.1) aggregated per warp.
+//              (Sec. 3.4.1) aggregated per warp.  Once per run: the sizes
+//              are sums, so a second fof_groups finds them final (Status::flat)
+//              and only clears the words that the outputs count in.
 //   outputs    (label, size) of every slot's group stored at the input index;
 //              per-box group and catalogue counts.
 //   catalogue  ids[i] = smallest index of i's group; sizes[label] = size, 0
@@ -40,12 +42,21 @@ __device__ __forceinline__ int final_root(int* __restrict__ parent, int s, int p
     return x;
 }
 
+// The words that fof_groups counts in start at zero, whatever ran before: also
+// where a graph replays fof_groups alone, which no state of the host could tell.
+__device__ __forceinline__ void clear_group_words(int* words, int64_t n)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        words[i] = 0;
+}
+
 // Bound by the latency of the walk to the root, so a slot's own words are read
 // one slot ahead (453 million slots: 1.97 and 1.54 ms; with 16 CTAs per SM in
 // the grid instead of 8, 1.48).
 __global__ void __launch_bounds__(256) k_finalize(int64_t total, int* __restrict__ parent,
                                                   int* __restrict__ minorig, int* __restrict__ cnt,
-                                                  int* __restrict__ err, bool ordered)
+                                                  int* group_words, int64_t n_group_words, Status* status,
+                                                  bool ordered)
 {
     pdl_wait();
     pdl_trigger();
@@ -56,6 +67,8 @@ __global__ void __launch_bounds__(256) k_finalize(int64_t total, int* __restrict
         p_next = parent[s];
         mo_next = minorig[s];
     }
+    const bool flat = status->flat != 0;       // used last: its load overlaps the walk
+    clear_group_words(group_words, n_group_words);
     for (; s - threadIdx.x < total; s += stride) {
         const bool valid = s < total;
         const int p = p_next, mo = mo_next;
@@ -68,7 +81,7 @@ __global__ void __launch_bounds__(256) k_finalize(int64_t total, int* __restrict
         unsigned active = __ballot_sync(kFull, valid);
         if (!valid)
             continue;
-        const int root = final_root(parent, (int)s, p, ordered, err);
+        const int root = final_root(parent, (int)s, p, ordered, &status->err);
         bool nonroot = root != (int)s;
         unsigned nr = __ballot_sync(active, nonroot);
         if (!nonroot)
@@ -76,7 +89,7 @@ __global__ void __launch_bounds__(256) k_finalize(int64_t total, int* __restrict
         unsigned peers = __match_any_sync(nr, root);
         int leader = __ffs(peers) - 1;
         unsigned mn = __reduce_min_sync(peers, (unsigned)mo);
-        if ((threadIdx.x & 31) == leader) {
+        if ((threadIdx.x & 31) == leader && !flat) {
             atomicAdd(cnt + root, __popc(peers));
             atomicMin(minorig + root, (int)mn);
         }
@@ -95,10 +108,14 @@ constexpr int kHashProbes = 16;
 
 __global__ void __launch_bounds__(256) k_finalize_hash(int64_t total, int* __restrict__ parent,
                                                        int* __restrict__ minorig, int* __restrict__ cnt,
-                                                       int* __restrict__ err, bool ordered)
+                                                       int* group_words, int64_t n_group_words, Status* status,
+                                                       bool ordered)
 {
     pdl_wait();
     pdl_trigger();
+    clear_group_words(group_words, n_group_words);
+    if (status->flat)
+        return;
     __shared__ int hkey[kHashSlots];
     __shared__ int hcnt[kHashSlots];
     __shared__ int hmin[kHashSlots];
@@ -111,7 +128,7 @@ __global__ void __launch_bounds__(256) k_finalize_hash(int64_t total, int* __res
             const int64_t s = b0 + (int64_t)t * blockDim.x + threadIdx.x;
             if (s >= total)
                 break;
-            const int root = final_root(parent, (int)s, parent[s], ordered, err);
+            const int root = final_root(parent, (int)s, parent[s], ordered, &status->err);
             if (root == (int)s)
                 continue;
             const int mo = minorig[s];
@@ -214,10 +231,12 @@ __global__ void __launch_bounds__(kScatterThreads) k_outputs_scatter(Geometry g,
                                                          unsigned long long* __restrict__ n_cat,
                                                          int2* __restrict__ pairs,
                                                          int* __restrict__ out_cursor, int per, int streams,
-                                                         int* __restrict__ err)
+                                                         Status* status)
 {
     pdl_wait();
     pdl_trigger();
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        status->flat = 1;                       // every CTA of the finalisation has read it
     __shared__ int s_box[kScatterWarps];
     __shared__ int2 s_acc[kScatterWarps];
     const int lane = threadIdx.x & 31;
@@ -283,7 +302,7 @@ __global__ void __launch_bounds__(kScatterThreads) k_outputs_scatter(Geometry g,
         if (room)
             pairs[at] = e;
         else
-            atomicOr(err, kErrInternal);
+            atomicOr(&status->err, kErrInternal);
         const bool in_cat = is_root && size >= thr;
         // per-box counts: summed in registers while the warp stays inside one
         // box and added once per box (one counter per box would otherwise
@@ -515,18 +534,16 @@ static int grid_for(int64_t items, int threads, int per_sm)
     return (int)(want < cap ? want : cap);
 }
 
-cudaError_t launch_finalize(const Geometry& g, const Work& w, const UfArgs& uf, int size_count, bool dependent,
-                            cudaStream_t s)
+cudaError_t launch_finalize(const Geometry& g, const Work& w, const UfArgs& uf, int size_count, cudaStream_t s)
 {
     if (g.total_n == 0)
         return cudaSuccess;
     const bool ordered = uf.link == 0;
-    dependent = dependent && g.total_n <= kDependentMax;
     if (size_count == 1)
-        return launch_kernel(dependent, k_finalize_hash, grid_for(g.total_n, 256 * kHashBatch, 4), 256, 0, s, g.total_n,
-                             w.parent, w.minorig, w.cnt, &w.status->err, ordered);
-    return launch_kernel(dependent, k_finalize, grid_for(g.total_n, 256, 16), 256, 0, s, g.total_n, w.parent,
-                         w.minorig, w.cnt, &w.status->err, ordered);
+        return launch_next(g.total_n, k_finalize_hash, grid_for(g.total_n, 256 * kHashBatch, 4), 256, 0, s, g.total_n,
+                           w.parent, w.minorig, w.cnt, w.group_words, w.n_group_words, w.status, ordered);
+    return launch_next(g.total_n, k_finalize, grid_for(g.total_n, 256, 16), 256, 0, s, g.total_n, w.parent, w.minorig,
+                       w.cnt, w.group_words, w.n_group_words, w.status, ordered);
 }
 
 cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t min_size, cudaStream_t s)
@@ -543,7 +560,7 @@ cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t min_size, c
     return launch_next(g.total_n, g.total_n <= kDirectMax ? k_outputs_scatter<true> : k_outputs_scatter<false>,
                        (chunks + streams - 1) / streams * streams, kScatterThreads, 0, s, g, w.sorted, w.parent,
                        w.minorig, w.cnt, thr, w.n_groups, w.n_cat, pairs, w.out_cursor, per, streams,
-                       &w.status->err);
+                       w.status);
 }
 
 cudaError_t launch_catalogue(const Geometry& g, const Work& w, int32_t* ids, int32_t* sizes, int32_t min_size,

@@ -360,7 +360,6 @@ struct fof_plan {
     char* results_dev = nullptr;
     char* zero_dev = nullptr;       // [zero_dev, zero_end) starts each run at zero
     char* zero_end = nullptr;
-    bool groups_clean = false;      // fof_groups' counters are zero (no fof_groups since fof_link)
     char* results_host = nullptr;   // pinned
     bool results_from_slab = false;
     ResultsLayout rl{};
@@ -422,8 +421,8 @@ Layout layout(int nbox, int64_t total_n, int64_t total_bricks, int64_t total_cel
     L.p0 = take(8 * (size_t)nbox);
     L.brick0 = take(8 * (size_t)nbox);
     // what starts each run at zero lies together: one memset before fof_link's
-    // kernels ([bcount, zero_end)), and, for a repeated fof_groups, one of its
-    // tail from the counts in the results block on
+    // kernels ([bcount, zero_end)); its tail, from the counts in the results block
+    // on, is cleared again by each finalisation (a repeated fof_groups)
     L.bcount = take(4 * (size_t)(total_bricks * brick_pad(total_bricks)));
     L.scan_state = take(8 * (size_t)scan_tiles(total_bricks) + 8);      // and the ticket and n_heavy
     L.scan_ticket = L.scan_state + 8 * (size_t)scan_tiles(total_bricks);
@@ -470,6 +469,8 @@ void bind_workspace(char* ws, const Layout& L, const BoxDev* boxes, int nbox, in
     const ResultsLayout rl = results_layout(nbox);
     char* res = ws + L.results;
     w.status = (Status*)(res + rl.status_off);
+    w.group_words = (int*)(res + rl.groups_off);
+    w.n_group_words = (int64_t)(L.zero_end - L.results - rl.groups_off) / 4;
     w.n_groups = (unsigned long long*)(res + rl.groups_off);
     w.n_cat = (unsigned long long*)(res + rl.cat_off);
     w.bcount = (int*)(ws + L.bcount);
@@ -715,7 +716,6 @@ int enqueue_link(fof_plan* h, const float* pos, cudaStream_t s)
     const Work& w = h->w;
     const UfArgs uf = uf_args(h);
     FOF_TRY(cudaMemsetAsync(h->zero_dev, 0, (size_t)(h->zero_end - h->zero_dev), s));
-    h->groups_clean = true;
     if (g.total_n == 0) {
         h->linked = true;
         return FOF_OK;
@@ -746,15 +746,9 @@ int enqueue_groups(fof_plan* h, int32_t* ids, int32_t* sizes, fof_group* cat, in
     const Geometry& g = h->g;
     const Work& w = h->w;
     if (g.total_n > 0) {
-        // status.err is kept from fof_link; counts start from zero
-        const bool clean = h->groups_clean;
-        if (!clean) {
-            char* from = h->results_dev + h->rl.groups_off;
-            FOF_TRY(cudaMemsetAsync(from, 0, (size_t)(h->zero_end - from), s));
-        }
-        h->groups_clean = false;
+        // status.err is kept from fof_link; the counts start from zero there
         phase_begin(h, kPhFinalize, s);
-        FOF_TRY(launch_finalize(g, w, uf_args(h), h->size_count, clean, s));
+        FOF_TRY(launch_finalize(g, w, uf_args(h), h->size_count, s));
         phase_end(h, kPhFinalize, s);
         phase_begin(h, kPhOutputs, s);
         FOF_TRY(launch_outputs(g, w, min_size, s));
@@ -864,7 +858,6 @@ int fof_relink(fof_handle h, const float* pos_dev, int32_t* path_out, void* stre
     if (h->binned && !h->capturing && g.total_n > 0) {
         // which particles left their cell or brick: one flag word, read back
         FOF_TRY(cudaMemsetAsync(h->results_dev, 0, (size_t)(h->zero_end - h->results_dev), s));
-        h->groups_clean = true;
         phase_begin(h, kPhBinCount, s);
         FOF_TRY(launch_relink_check(pos_dev, g, w, &w.status->pad, s));
         phase_end(h, kPhBinCount, s);
@@ -1140,7 +1133,6 @@ int fof_graph_launch(fof_handle h, void* stream)
         return h ? FOF_ERR_STATE : FOF_ERR_ARG;
     FOF_TRY(cudaGraphLaunch(h->gexec, (cudaStream_t)stream));
     h->linked = true;
-    h->groups_clean = false;
     h->pending = true;
     h->last_cap = h->graph_cap;
     // a graph replays every phase once
@@ -1427,7 +1419,7 @@ extern "C" int fof_run_noalloc(double box, double l_x, int64_t n, const float* p
         FOF_TRY(launch_dense(g, w, kDefaultDenseMin, uf, false, s));
         FOF_TRY(launch_dense(g, w, kDefaultDenseMin, uf, true, s));
         FOF_TRY(launch_big(g, w, kDefaultDenseMin, uf, true, s));
-        FOF_TRY(launch_finalize(g, w, uf, 0, true, s));
+        FOF_TRY(launch_finalize(g, w, uf, 0, s));
         FOF_TRY(launch_outputs(g, w, min_size, s));
         FOF_TRY(launch_catalogue(g, w, ids_dev, sizes_dev, min_size, (int2*)catalogue_dev, cat_capacity, s));
     }
