@@ -834,7 +834,9 @@ __global__ void __launch_bounds__(256) k_relink_check(const float* __restrict__ 
         const BoxDev& b = g.boxes[box_of(g.box_p0, g.nbox, s)];
         const float4 old = sorted[s];
         const int o = __float_as_int(old.w);
-        const int64_t i = b.p0 + o;
+        // a record that binning never wrote names no particle: bin again
+        const bool named = (unsigned long long)o < (unsigned long long)b.n;
+        const int64_t i = b.p0 + (named ? o : 0);
         float4 rec;
         bool ok;
         const int64_t nb = brick_of(pos, i, b, rec, ok);
@@ -843,7 +845,7 @@ __global__ void __launch_bounds__(256) k_relink_check(const float* __restrict__ 
         const int nx = cell_coord(rec.x, b), ny = cell_coord(rec.y, b), nz = cell_coord(rec.z, b);
         if (nx != ox || ny != oy || nz != oz)
             f |= 1;
-        if (nb != b.brick0 + brick_local(b, ox, oy, oz))
+        if (!named || nb != b.brick0 + brick_local(b, ox, oy, oz))
             f |= 2;
         sorted[s] = rec;
         tmp[s] = rec;

@@ -1103,12 +1103,18 @@ int fof_graph_build(fof_handle h, const float* pos_dev, int32_t* ids_dev, int32_
         h->gexec = nullptr;
     }
     FOF_TRY(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+    // nothing runs yet: what the plan holds stays as it is until the launch
+    const bool linked = h->linked, binned = h->binned, pending = h->pending;
+    const int64_t last_cap = h->last_cap;
     h->capturing = true;
     rc = enqueue_link(h, pos_dev, s);
     if (rc == FOF_OK)
         rc = enqueue_groups(h, ids_dev, sizes_dev, catalogue_dev, cat_capacity, min_size, s);
     h->capturing = false;
-    h->pending = false;
+    h->linked = linked;
+    h->binned = binned;
+    h->pending = pending;
+    h->last_cap = last_cap;
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamEndCapture(s, &graph);
     if (rc != FOF_OK) {
@@ -1133,6 +1139,7 @@ int fof_graph_launch(fof_handle h, void* stream)
         return h ? FOF_ERR_STATE : FOF_ERR_ARG;
     FOF_TRY(cudaGraphLaunch(h->gexec, (cudaStream_t)stream));
     h->linked = true;
+    h->binned = h->g.total_n > 0;
     h->pending = true;
     h->last_cap = h->graph_cap;
     // a graph replays every phase once
