@@ -140,6 +140,11 @@ struct TeamStage {
 constexpr int kLinkThreads = 256;
 constexpr int kLinkWarps = kLinkThreads / 32;
 constexpr int kLinkBlocks = 5;   // resident CTAs per SM (48 registers)
+// The form that reads the union-find options at run time holds more, and spills
+// at 48 (link phase, 134 million particles, with 5 and 4 CTAs: the defaults through
+// it 14.9 and 14.4 ms, halving at every depth 16.2 and 15.6, no compression 17.7 and
+// 17.2, random linking 15.0 and 14.5; full compression 17.6 and 18.2).
+constexpr int kLinkVarBlocks = 4;
 constexpr int kOwnCell = 13;     // stream index of a team's own cell (cells above kTeamSelfMax)
 
 // The buffered candidates S.cpos/cslot[0..c) of a team against its m
@@ -276,7 +281,7 @@ __device__ __forceinline__ void team_cell(TeamStage& S, int* __restrict__ parent
 // particles, 8 warps and one: 23 and 36 us).  One window's chain counts there,
 // so these have 64 registers (300,007 particles: 76 us, with 48: 87).
 template <bool kVar, bool kSplit>
-__global__ void __launch_bounds__(kLinkThreads, kSplit ? 4 : kLinkBlocks)
+__global__ void __launch_bounds__(kLinkThreads, kSplit ? 4 : (kVar ? kLinkVarBlocks : kLinkBlocks))
     k_link(Geometry g, const float4* __restrict__ sorted, const int* __restrict__ cell_start, int* parent,
            int dense_min, int parts, int batch, Status* status, UfArgs uf)
 {
@@ -1119,7 +1124,7 @@ cudaError_t launch_link(const Geometry& g, const Work& w, int dense_min, const U
     if (g.total_n == 0)
         return cudaSuccess;
     const int64_t windows = (g.total_n + kWarp - 1) / kWarp;
-    const int64_t warps = (int64_t)sm_count() * kLinkBlocks * kLinkWarps;   // resident
+    const int64_t warps = (int64_t)sm_count() * (uf.var ? kLinkVarBlocks : kLinkBlocks) * kLinkWarps;   // resident
     const bool split = windows <= 2 * warps;
     // warps per window while a third of the chip would have none, at most
     // kLinkWarps (a CTA's warps are a whole number of windows)
