@@ -838,8 +838,12 @@ cudaError_t launch_big(const Geometry& g, const Work& w, int dense_min, const Uf
                        cudaStream_t s);
 // size_count: 0 warp-aggregated atomics, 1 per-block shared-memory hash table
 cudaError_t launch_finalize(const Geometry& g, const Work& w, const UfArgs& uf, int size_count, cudaStream_t s);
-cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t min_size, cudaStream_t s);
-cudaError_t launch_catalogue(const Geometry& g, const Work& w, int32_t* ids, int32_t* sizes,
-                             int32_t min_size, int2* cat, int64_t cap, cudaStream_t s);
+// both output kernels, and up to kDirectMax inputs the catalogue with them
+cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t* ids, int32_t* sizes, int32_t min_size,
+                           int2* cat, int64_t cap, cudaStream_t s);
+// the catalogue's own kernels, above
+cudaError_t launch_catalogue(const Geometry& g, const Work& w, const int32_t* sizes, int32_t min_size, int2* cat,
+                             int64_t cap, cudaStream_t s);
+int catalogue_launches(const Geometry& g);
 
 }  // namespace fofgpu

@@ -546,38 +546,43 @@ cudaError_t launch_finalize(const Geometry& g, const Work& w, const UfArgs& uf, 
                        w.cnt, w.group_words, w.n_group_words, w.status, ordered);
 }
 
-cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t min_size, cudaStream_t s)
+cudaError_t launch_outputs(const Geometry& g, const Work& w, int32_t* ids, int32_t* sizes, int32_t min_size,
+                           int2* cat, int64_t cap, cudaStream_t s)
 {
     if (g.total_n == 0)
         return cudaSuccess;
-    int32_t thr = min_size < 1 ? 1 : min_size;
+    const int32_t thr = min_size < 1 ? 1 : min_size;
     int2* pairs = (int2*)w.tmp;            // the brick-order copy is dead by now
     const int64_t tiles = (g.total_n + kScatterThreads - 1) / kScatterThreads;
     // as many slots per CTA as leave eight CTAs to an SM
     const int per = (int)std::min<int64_t>(kScatterTiles, std::max<int64_t>(1, tiles / ((int64_t)sm_count() * 8)));
-    const int streams = g.total_n <= kDirectMax ? 1 : kScatterStreams;
+    const bool direct = g.total_n <= kDirectMax;
+    const int streams = direct ? 1 : kScatterStreams;
     const int64_t chunks = (tiles + per - 1) / per;
-    return launch_next(g.total_n, g.total_n <= kDirectMax ? k_outputs_scatter<true> : k_outputs_scatter<false>,
-                       (chunks + streams - 1) / streams * streams, kScatterThreads, 0, s, g, w.sorted, w.parent,
-                       w.minorig, w.cnt, thr, w.n_groups, w.n_cat, pairs, w.out_cursor, per, streams,
+    cudaError_t e = launch_next(g.total_n, direct ? k_outputs_scatter<true> : k_outputs_scatter<false>,
+                                (chunks + streams - 1) / streams * streams, kScatterThreads, 0, s, g, w.sorted,
+                                w.parent, w.minorig, w.cnt, thr, w.n_groups, w.n_cat, pairs, w.out_cursor, per,
+                                streams, w.status);
+    if (e != cudaSuccess)
+        return e;
+    return launch_next(g.total_n, direct ? k_outputs_write<true> : k_outputs_write<false>, w.n_tiles, kOutThreads, 0, s,
+                       g, (const int2*)pairs, ids, sizes, thr, cat, cap, w.tile_state, w.tile_ticket, w.out_cursor,
                        w.status);
 }
 
-cudaError_t launch_catalogue(const Geometry& g, const Work& w, int32_t* ids, int32_t* sizes, int32_t min_size,
-                             int2* cat, int64_t cap, cudaStream_t s)
+int catalogue_launches(const Geometry& g)
 {
-    if (g.total_n == 0)
+    return g.total_n <= kDirectMax ? 0 : 2;     // k_outputs_write leaves it behind too
+}
+
+cudaError_t launch_catalogue(const Geometry& g, const Work& w, const int32_t* sizes, int32_t min_size, int2* cat,
+                             int64_t cap, cudaStream_t s)
+{
+    if (catalogue_launches(g) == 0)
         return cudaSuccess;
-    int32_t thr = min_size < 1 ? 1 : min_size;
-    const int2* pairs = (const int2*)w.tmp;
-    const bool direct = g.total_n <= kDirectMax;
-    cudaError_t e =
-        launch_next(g.total_n, direct ? k_outputs_write<true> : k_outputs_write<false>, w.n_tiles, kOutThreads, 0, s,
-                    g, pairs, ids, sizes, thr, cat, cap, w.tile_state, w.tile_ticket, w.out_cursor, w.status);
-    if (e != cudaSuccess || direct)
-        return e;
-    e = launch_scan(g.total_n, w.out_cursor, 1, w.tile_off, w.n_tiles, w.tile_state, w.tile_ticket, 0, nullptr, nullptr,
-                    &w.status->err, s);
+    const int32_t thr = min_size < 1 ? 1 : min_size;
+    cudaError_t e = launch_scan(g.total_n, w.out_cursor, 1, w.tile_off, w.n_tiles, w.tile_state, w.tile_ticket, 0,
+                                nullptr, nullptr, &w.status->err, s);
     if (e != cudaSuccess)
         return e;
     return launch_next(g.total_n, k_catalogue, grid_for(w.n_tiles * kOutThreads, kOutThreads, 4), kOutThreads, 0, s, g, sizes,

@@ -56,7 +56,8 @@ int phase_launches(int ph, const Geometry& g, int dense_min)
     case kPhDenseSelf:
     case kPhDensePairs: return dense_launches(g, dense_min);
     case kPhBrickSort: return heavy_bricks(g.total_n) ? 2 : 1;
-    case kPhCatalogue: return g.total_n <= kDirectMax ? 1 : 3;
+    case kPhOutputs: return 2;
+    case kPhCatalogue: return catalogue_launches(g);
     default: return 1;
     }
 }
@@ -751,10 +752,10 @@ int enqueue_groups(fof_plan* h, int32_t* ids, int32_t* sizes, fof_group* cat, in
         FOF_TRY(launch_finalize(g, w, uf_args(h), h->size_count, s));
         phase_end(h, kPhFinalize, s);
         phase_begin(h, kPhOutputs, s);
-        FOF_TRY(launch_outputs(g, w, min_size, s));
+        FOF_TRY(launch_outputs(g, w, ids, sizes, min_size, (int2*)cat, cap, s));
         phase_end(h, kPhOutputs, s);
         phase_begin(h, kPhCatalogue, s);
-        FOF_TRY(launch_catalogue(g, w, ids, sizes, min_size, (int2*)cat, cap, s));
+        FOF_TRY(launch_catalogue(g, w, sizes, min_size, (int2*)cat, cap, s));
         phase_end(h, kPhCatalogue, s);
     }
     FOF_TRY(cudaMemcpyAsync(h->results_host, h->results_dev, h->rl.bytes, cudaMemcpyDeviceToHost, s));
@@ -1427,8 +1428,8 @@ extern "C" int fof_run_noalloc(double box, double l_x, int64_t n, const float* p
         FOF_TRY(launch_dense(g, w, kDefaultDenseMin, uf, true, s));
         FOF_TRY(launch_big(g, w, kDefaultDenseMin, uf, true, s));
         FOF_TRY(launch_finalize(g, w, uf, 0, s));
-        FOF_TRY(launch_outputs(g, w, min_size, s));
-        FOF_TRY(launch_catalogue(g, w, ids_dev, sizes_dev, min_size, (int2*)catalogue_dev, cat_capacity, s));
+        FOF_TRY(launch_outputs(g, w, ids_dev, sizes_dev, min_size, (int2*)catalogue_dev, cat_capacity, s));
+        FOF_TRY(launch_catalogue(g, w, sizes_dev, min_size, (int2*)catalogue_dev, cat_capacity, s));
     }
     alignas(16) unsigned char host_res[128];
     FOF_TRY(cudaMemcpyAsync(host_res, res, rl.bytes, cudaMemcpyDeviceToHost, s));
