@@ -558,13 +558,18 @@ int cuda_rc(cudaError_t e)
         if (e_ != cudaSuccess) return cuda_rc(e_);     \
     } while (0)
 
-void phase_begin(fof_plan* h, int ph, cudaStream_t s)
+void phase_begin(fof_plan* h, int ph, int launches, cudaStream_t s)
 {
-    h->launches += phase_launches(ph, h->g, h->dense_min);
-    h->phase[ph].launches += phase_launches(ph, h->g, h->dense_min);
+    h->launches += launches;
+    h->phase[ph].launches += launches;
     if (h->timing && !h->capturing) {
         cudaEventRecord(h->phase[ph].ev0, s);
     }
+}
+
+void phase_begin(fof_plan* h, int ph, cudaStream_t s)
+{
+    phase_begin(h, ph, phase_launches(ph, h->g, h->dense_min), s);
 }
 
 void phase_end(fof_plan* h, int ph, cudaStream_t s)
@@ -883,7 +888,7 @@ int fof_relink(fof_handle h, const float* pos_dev, int32_t* path_out, void* stre
             phase_end(h, kPhBrickSort, s);
         } else {
             // every particle kept its cell: cells, starts and lists stand
-            phase_begin(h, kPhBrickSort, s);
+            phase_begin(h, kPhBrickSort, 1, s);
             FOF_TRY(launch_forest_init(g, w, s));
             phase_end(h, kPhBrickSort, s);
         }

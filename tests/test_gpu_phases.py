@@ -28,3 +28,11 @@ def test_outputs_hold_both_output_kernels(cuda_lib, n, catalogue):
     phases, = _run(cuda_lib, n)
     assert phases["outputs"][1] == 2
     assert phases["catalogue"][1] == catalogue
+
+
+# with and without the second sort kernel (plans above 65,535 particles)
+@pytest.mark.parametrize("n,sorts", [(65_535, 1), (65_536, 2)])
+def test_relink_in_place_counts_one_launch(cuda_lib, n, sorts):
+    first, again = _run(cuda_lib, n, relinks=1)
+    assert first["brick_sort"][1] == sorts
+    assert again["brick_sort"][1] == 1        # the forest alone is started anew
