@@ -354,9 +354,10 @@ int fof_merge_links(int64_t npairs, const int64_t *a, const int64_t *b, int64_t 
  * no cudaMalloc/cudaFree, no pinned memory, no events, no plan.  The
  * workspace is a fixed 32 MiB array in the library's own device memory,
  * which every GPU that loads the library holds until the process exits.
- *   - Problems whose workspace (fof_workspace_bytes with NULL options)
- *     exceeds 32 MiB are rejected with FOF_ERR_TOO_LARGE, checked before any
- *     pointer; that is about 580,000 particles at the default occupancy.
+ *   - Problems too large for it are rejected with FOF_ERR_TOO_LARGE, checked
+ *     before any pointer.  A problem counts about 48 bytes per particle, 4 per
+ *     cell and 12 per brick, whatever the workspace's layout needs of them:
+ *     about 550,000 to 580,000 particles at the default options.
  *   - The first call on a device looks up the array's device address
  *     (cudaGetSymbolAddress) with that device current, and later calls in
  *     the same context reuse it; a call after the context was re-created

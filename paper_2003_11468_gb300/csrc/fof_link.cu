@@ -298,7 +298,8 @@ __global__ void __launch_bounds__(kLinkThreads, kSplit ? 4 : (kVar ? kLinkVarBlo
     // cell (x | y << 16, z) and box of each lane's particle, and the cell's end:
     // read back where they are needed, like the record, because registers are
     // what limits the warps per SM, and those the kernel (64 registers, 4 CTAs:
-    // 35.8 ms on the 768^3 box; 48, 5: 34.4; 40, 6, with 120 bytes spilled: 37.0)
+    // 35.8 ms on the 768^3 box; 48, 5, with 28 bytes spilled: 34.4; 40, 6, with 120
+    // bytes: 37.0)
     __shared__ int4 where[kLinkWarps][kWarp];
     const int lane = threadIdx.x & 31;
     TeamStage& S = stage[threadIdx.x >> 5];
@@ -333,8 +334,8 @@ __global__ void __launch_bounds__(kLinkThreads, kSplit ? 4 : (kVar ? kLinkVarBlo
         __syncwarp();                           // every lane's copy is in, and the last window's reads are done
         const float4* rec = pf + par * kWarp;
         if (valid) {
-            // (the warp's search of box_of_warp spills here: batch of 512 boxes
-            // 24.5 and 24.4 ms, but the 768^3 box 33.9 and 34.2)
+            // (with the warp's search of box_of_warp, this kernel: batch of 512
+            // boxes 24.4 ms instead of 24.5, but the 768^3 box 34.2 instead of 33.9)
             const int bi = box_of(g.box_p0, g.nbox, s);
             const BoxDev& b = g.boxes[bi];
             const float4 p = rec[lane];
@@ -557,7 +558,7 @@ __global__ void __launch_bounds__(kLinkThreads, kSplit ? 4 : (kVar ? kLinkVarBlo
 // 153 and 51, 16.8 million (256^3) 642 and 266, 453 million (768^3) 13740 and
 // 6900.
 constexpr int kTeamWarps = 4;
-constexpr int kTeamBlocks = 8;               // CTAs per SM (64 registers, 27 KB)
+constexpr int kTeamBlocks = 8;               // CTAs per SM (64 registers, 28 bytes spilled; 27 KB)
 constexpr int kZBins = 32;                   // z bins of the order of a team cell
 
 // The staged positions of a cell, axis by axis: one 16-byte load holds two
@@ -851,7 +852,7 @@ __device__ __forceinline__ void team_fetch(TeamWarpSmem& S, int64_t e, const flo
     cp_async_commit();
 }
 
-// One cell of 33..kTeamSelfMax particles by the whole CTA.
+// One cell of kTeamSplit + 1..kTeamSelfMax particles by the whole CTA.
 __device__ __forceinline__ void team_cell_cta(TeamCtaSmem& S, int c0, int m, float4* sorted, int* parent,
                                               int* minorig, const BoxDev& b)
 {

@@ -687,7 +687,7 @@ UfArgs uf_args(const fof_plan* h)
 }
 
 // Linking on the binned particles: self tasks of team and big cells, then
-// k_link with the dense cells beside it (launch_next), then the pairs that need
+// k_link with the dense cells beside it (launch_beside), then the pairs that need
 // every cell's slots in their final order (shared by fof_link and fof_relink).
 int enqueue_linking(fof_plan* h, cudaStream_t s)
 {
@@ -1299,7 +1299,7 @@ std::mutex g_noalloc_mu;
 char* g_noalloc_ptr[kNoallocMaxDevices];                 // device address of the array, per device
 unsigned long long g_noalloc_ctx[kNoallocMaxDevices];    // id of the context it belongs to
 
-// What a problem counts against the array: a fixed accounting of 62 bytes per
+// What a problem counts against the array: a fixed accounting of 48 bytes per
 // particle (records in two orders 32, forest and labels 12, lists and output
 // cursors), 4 per cell and 12 per brick, so that the sizes that fit do not
 // change with the workspace layout, which needs no more than this.
