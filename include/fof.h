@@ -214,8 +214,9 @@ int fof_relink(fof_handle h, const float *pos_dev, int32_t *path_out, void *stre
  * order, min_size applies to every box, and n_groups_out / n_cat_out
  * (host, may be NULL) receive one count per box.  If the catalogue has more
  * than cat_capacity entries in total, the first cat_capacity are written,
- * the counts are still reported and FOF_ERR_CAPACITY is returned.  Errors:
- * FOF_ERR_STATE (no fof_link yet), FOF_ERR_RANGE, FOF_ERR_TIMEOUT,
+ * the counts are still reported and FOF_ERR_CAPACITY is returned.  It may be
+ * called again for the same fof_link, with other buffers or another
+ * min_size.  Errors: FOF_ERR_STATE (no fof_link yet), FOF_ERR_RANGE, FOF_ERR_TIMEOUT,
  * FOF_ERR_CAPACITY, FOF_ERR_ARG, FOF_ERR_CUDA. */
 int fof_groups(fof_handle h, int32_t *ids_dev, int32_t *sizes_dev,
                fof_group *catalogue_dev, int64_t cat_capacity, int32_t min_size,
